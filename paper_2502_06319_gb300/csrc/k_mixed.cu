@@ -57,15 +57,14 @@ __device__ __forceinline__ bool step(const LaunchArgs &a, Lane &L, Acc<ACC> &x, 
 {
     m32::Drift c;
     const P32<kSetsPerPage> q{L.q};
-    float lnP;
+    float fr, fth, fph, lnP, sin_th;
+    x.view(fr, fth, fph, lnP, sin_th);
     if constexpr (EN) {
         // rigidity from the integrated kinetic energy: P = (A/|Z|) sqrt(T (T + 2 m0))
         const float T = en.fT();
         lnP = __logf(en.aoz * sqrtf(T * (T + 2.0f * en.m0)));
-    } else {
-        lnP = x.flnP();
     }
-    m32::eval<EXT, FULL, kSetsPerPage>(q, L.M2, L.sq, x.fr(), x.fth(), x.sin_th(), x.fph(), lnP, c);
+    m32::eval<EXT, FULL, kSetsPerPage>(q, L.M2, L.sq, fr, fth, sin_th, fph, lnP, c);
     const float sdt = sqrtf(c.dt);
     const float dr = fmaf(c.Ar_tot, c.dt, c.l00 * z0 * sdt);
     const float dth = fmaf(c.dth_drift, c.dt, c.l11 * z1 * sdt * c.inv_r);
@@ -75,9 +74,9 @@ __device__ __forceinline__ bool step(const LaunchArgs &a, Lane &L, Acc<ACC> &x, 
         const float T = en.fT();
         const float alpha = __fdividef(T + 2.0f * en.m0, T + en.m0);
         en.add(c.dlnP * alpha * T * c.dt, c.dlnP * fmaf(c.beta, c.beta, 1.0f) * c.dt);
-        x.add(dr, dth, dph, 0.0f, c.dt);
+        x.template add<false>(dr, dth, dph, 0.0f, c.dt);
     } else {
-        x.add(dr, dth, dph, c.dlnP * c.dt, c.dt);
+        x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
     }
     x.boundaries(P32F(q, r_in));
     L.k += 1u;

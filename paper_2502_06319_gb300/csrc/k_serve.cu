@@ -150,12 +150,14 @@ __global__ void __launch_bounds__(256) k_serve(ServeArgs a)
 
         m32::Drift c;
         const P32<1> q{S.L.q};
-        m32::eval<EXT, FULL, 1>(q, S.L.M2, S.L.sq, x.fr(), x.fth(), x.sin_th(), x.fph(), x.flnP(), c);
+        float fr, fth, fph, lnP, sin_th;
+        x.view(fr, fth, fph, lnP, sin_th);
+        m32::eval<EXT, FULL, 1>(q, S.L.M2, S.L.sq, fr, fth, sin_th, fph, lnP, c);
         const float sdt = sqrtf(c.dt);
         const float dr = fmaf(c.Ar_tot, c.dt, c.l00 * z0 * sdt);
         const float dth = fmaf(c.dth_drift, c.dt, c.l11 * z1 * sdt * c.inv_r);
         const float dph = fmaf(c.dph_drift, c.dt, fmaf(c.l20, z0, c.l22 * z2) * sdt * c.inv_rs);
-        x.add(dr, dth, dph, c.dlnP * c.dt, c.dt);
+        x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
         x.boundaries(P32F(q, r_in));
         S.L.k += 1u;
         used += 1u;

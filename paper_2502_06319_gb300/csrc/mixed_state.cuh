@@ -4,6 +4,7 @@
 // pairs or in FP64, with the boundary handling of the step.
 #pragma once
 #include "common.cuh"
+#include "f64bits.h"
 #include "model32.cuh"
 
 namespace cosmica {
@@ -37,7 +38,6 @@ struct Acc<COSMICA_PREC_MIXED> {
     __device__ float fr() const { return r.hi; }
     __device__ float fth() const { return th.hi; }
     __device__ float fph() const { return ph.hi; }
-    __device__ float flnP() const { return lnP.hi; }
     // distance of theta (hi + lo, in [0, pi]) to the nearer pole, to FP32 accuracy:
     // near pi it is formed from the float-float splits of pi and theta (the high
     // parts subtract exactly), so it keeps its sign and relative accuracy even
@@ -47,13 +47,20 @@ struct Acc<COSMICA_PREC_MIXED> {
         if (th.hi < m32::kHalfPiF) return th.hi;
         return __fadd_rn(__fsub_rn(m32::kPiF, th.hi), __fsub_rn(m32::kPiLoF, th.lo));
     }
-    __device__ float sin_th() const { return m32::sin_from_pole_distance(pole_distance()); }
+    // r, theta, phi, lnP and sin(theta) as the step reads them
+    __device__ void view(float &fr, float &fth, float &fph, float &flnP, float &sin_th) const
+    {
+        fr = r.hi; fth = th.hi; fph = ph.hi; flnP = lnP.hi;
+        sin_th = m32::sin_from_pole_distance(pole_distance());
+    }
+    // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone)
+    template <bool P>
     __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
     {
         m32::ff_add(r, dr);
         m32::ff_add(th, dth);
         m32::ff_add(ph, dph);
-        m32::ff_add(lnP, dlnP);
+        if (P) m32::ff_add(lnP, dlnP);
         m32::ff_add(s, dt);
     }
     // reflect at r_in, fold theta at the poles, wrap phi; all rare branches
@@ -99,7 +106,25 @@ struct Acc<COSMICA_PREC_MIXED> {
     }
 };
 
-// FP64 accumulation of FP32 increments
+// FP64 <-> FP32 for the FP64-accumulated state: integer forms (f64bits.h) with the
+// conversion instruction left for the rare values those do not take.
+__device__ __forceinline__ uint64_t bits64(double x) { return (uint64_t)__double_as_longlong(x); }
+__device__ __forceinline__ double widen64(float d)
+{
+    return __longlong_as_double((long long)f64bits::widen(__float_as_uint(d)));
+}
+__device__ __forceinline__ bool widen64_ok(float d) { return f64bits::widen_ok(__float_as_uint(d)); }
+__device__ __forceinline__ float narrow64(double x)
+{
+    return f64bits::narrow_ok((uint32_t)__double2hiint(x)) ? __uint_as_float(f64bits::narrow(bits64(x))) : (float)x;
+}
+
+// FP64 accumulation of FP32 increments.
+// Bound by the FP64 pipe (64 clocks per warp instruction and scheduler): only the sums stay on
+// it; conversions, comparisons and the finiteness test run on the bits (f64bits.h), with one
+// rarely taken branch each for the values that need the instruction.  The results are the
+// same bits.  Measured: 4 heliospheres x 3 species x 30 energies, 1.4e5 paths 738 -> 328 ms;
+// one squashed heliosphere 316 -> 175 ms.
 template <>
 struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     double r, th, ph, lnP, s, Rout, r_in;
@@ -107,27 +132,61 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     {
         r = r0; th = th0; ph = ph0; lnP = lnP0; s = 0.0; Rout = R_out; r_in = (double)r_in_f;
     }
-    __device__ float fr() const { return (float)r; }
-    __device__ float fth() const { return (float)th; }
-    __device__ float fph() const { return (float)ph; }
-    __device__ float flnP() const { return (float)lnP; }
-    __device__ float sin_th() const { return m32::sin_theta_f64(th); }
+    __device__ float fr() const { return narrow64(r); }
+    __device__ float fth() const { return narrow64(th); }
+    __device__ float fph() const { return narrow64(ph); }
+    // r, theta, phi, lnP and sin(theta) as the step reads them
+    __device__ void view(float &fr, float &fth, float &fph, float &flnP, float &sin_th) const
+    {
+        const uint64_t bt = bits64(th);
+        const bool north = f64bits::less(bt, f64bits::kHalfPiBits);
+        const uint64_t units = f64bits::pi_minus_units(bt);
+        fr = __uint_as_float(f64bits::narrow(bits64(r)));
+        fth = __uint_as_float(f64bits::narrow(bt));
+        fph = __uint_as_float(f64bits::narrow(bits64(ph)));
+        flnP = __uint_as_float(f64bits::narrow(bits64(lnP)));
+        float d = north ? fth : f64bits::pi_minus(units);    // distance to the nearer pole
+        if (!(f64bits::narrow_ok((uint32_t)__double2hiint(r)) & f64bits::narrow_ok((uint32_t)__double2hiint(th)) &
+              f64bits::narrow_ok((uint32_t)__double2hiint(ph)) & f64bits::narrow_ok((uint32_t)__double2hiint(lnP)) &
+              (north | f64bits::pi_minus_ok(units)))) {
+            fr = (float)r; fth = (float)th; fph = (float)ph; flnP = (float)lnP;
+            d = (float)(th < 0.5 * kPi ? th : kPi - th);
+        }
+        sin_th = m32::sin_from_pole_distance(d);
+    }
+    // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone)
+    template <bool P>
     __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
     {
-        r += (double)dr; th += (double)dth; ph += (double)dph; lnP += (double)dlnP; s += (double)dt;
+        double ar = widen64(dr), ath = widen64(dth), aph = widen64(dph), aP = widen64(dlnP), at = widen64(dt);
+        if (!(widen64_ok(dr) & widen64_ok(dth) & widen64_ok(dph) & (!P | widen64_ok(dlnP)) & widen64_ok(dt))) {
+            ar = (double)dr; ath = (double)dth; aph = (double)dph; aP = (double)dlnP; at = (double)dt;
+        }
+        r += ar; th += ath; ph += aph;
+        if (P) lnP += aP;
+        s += at;
     }
     __device__ void boundaries(float)
     {
-        if (r < r_in) r = 2.0 * r_in - r;
-        if (th < 0.0 || th > kPi) {
-            double t = th - kTwoPi * floor(th / kTwoPi);
-            if (t > kPi) { t = kTwoPi - t; ph += kPi; }
-            th = t;
+        // one rarely taken branch for the three boundaries; inside it the FP64 comparisons decide
+        if (f64bits::less(bits64(r), bits64(r_in)) | f64bits::outside_closed(bits64(th), f64bits::kPiBits) |
+            f64bits::outside_half_open(bits64(ph), f64bits::kTwoPiBits)) {
+            if (r < r_in) r = 2.0 * r_in - r;
+            if (th < 0.0 || th > kPi) {
+                double t = th - kTwoPi * floor(th / kTwoPi);
+                if (t > kPi) { t = kTwoPi - t; ph += kPi; }
+                th = t;
+            }
+            if (ph < 0.0 || ph >= kTwoPi) ph = ph - kTwoPi * floor(ph / kTwoPi);
         }
-        if (ph < 0.0 || ph >= kTwoPi) ph = ph - kTwoPi * floor(ph / kTwoPi);
     }
-    __device__ bool exited() const { return r >= Rout; }
-    __device__ bool finite() const { return isfinite(r + th + ph + lnP + s); }
+    // (a non-NaN comparison; finite() is asked first)
+    __device__ bool exited() const { return !f64bits::less(bits64(r), bits64(Rout)); }
+    __device__ bool finite() const
+    {
+        return f64bits::is_finite(bits64(r)) & f64bits::is_finite(bits64(th)) & f64bits::is_finite(bits64(ph)) &
+               f64bits::is_finite(bits64(lnP)) & f64bits::is_finite(bits64(s));
+    }
     __device__ void write(const ExitPtrs &out, uint64_t g) const
     {
         out.r[g] = r; out.th[g] = th; out.ph[g] = ph; out.lnP[g] = lnP; out.s[g] = s;
@@ -164,8 +223,13 @@ struct EnergyAcc<COSMICA_PREC_MIXED_F64ACC, true> {
     double T, Lam;
     float m0, aoz;
     __device__ void init(double T0, float m0_, float aoz_) { T = T0; Lam = 0.0; m0 = m0_; aoz = aoz_; }
-    __device__ float fT() const { return (float)T; }
-    __device__ void add(float dT, float dLam) { T += (double)dT; Lam += (double)dLam; }
+    __device__ float fT() const { return narrow64(T); }
+    __device__ void add(float dT, float dLam)
+    {
+        double aT = widen64(dT), aL = widen64(dLam);
+        if (!(widen64_ok(dT) & widen64_ok(dLam))) { aT = (double)dT; aL = (double)dLam; }
+        T += aT; Lam += aL;
+    }
     __device__ double T64() const { return T; }
     __device__ double lw() const { return -Lam; }
 };
