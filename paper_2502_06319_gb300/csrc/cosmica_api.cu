@@ -677,11 +677,61 @@ static cosmica_status upload_lis(const cosmica_lis *lis, DevBuf &buf, Staging &s
     return COSMICA_OK;
 }
 
-static cosmica_status spectrum_of_hist(const std::vector<SpecItem> &its, const cosmica_lis *lis, uint32_t nbins,
-                                       double x_lo, double dx, const uint64_t *hist, double *J, double *sigma,
-                                       DevBuf &ibuf, Staging &istage, DevBuf &lbuf, Staging &lstage, cudaStream_t s);
+// Spectrum items of a call: species numbered in order of first use.
+struct SpecItems {
+    std::vector<SpecItem> its;
+    std::vector<uint32_t> sp_item;     // an item of each species
+    void add(double T, const cosmica_species &sp, uint32_t &number)   // number: UINT32_MAX before the species' first use
+    {
+        if (number == UINT32_MAX) {
+            number = (uint32_t)sp_item.size();
+            sp_item.push_back((uint32_t)its.size());
+        }
+        its.push_back(SpecItem{T, (double)sp.A, (double)sp.Z, sp.m0_GeV, number, 0u});
+    }
+};
 
-static cosmica_status run_spectrum(const cosmica_exit_states *ex, const std::vector<SpecItem> &its,
+// Bin weights are tabulated per species for up to this many bins; above, an item evaluates those
+// of its nonzero bins (the table would rival the histogram in size, most of it unused).
+constexpr uint32_t kMaxWeightBins = 65536;
+
+// Eq. 4 per item: upload of the items, histogram of the exit states (or the given histogram when
+// ex is NULL), spectra.
+static cosmica_status spectrum_of(const cosmica_exit_states *ex, const SpecItems &si, const cosmica_lis *lis,
+                                  uint32_t nbins, double x_lo, double dx, uint64_t *hist, double *J, double *sigma,
+                                  DevBuf &ibuf, Staging &istage, DevBuf &lbuf, Staging &lstage, cudaStream_t s)
+{
+    const uint32_t n_items = (uint32_t)si.its.size(), n_sp = (uint32_t)si.sp_item.size();
+    const bool table = nbins <= kMaxWeightBins;
+    const size_t b_items = align_up(n_items * sizeof(SpecItem), 256);
+    const size_t up = b_items + align_up(n_sp * sizeof(uint32_t), 256);
+    const size_t b_sums = align_up(n_items * spectrum_sums_bytes(), 256);
+    cosmica_status st = ibuf.reserve(up + b_sums + (table ? (size_t)n_sp * nbins * sizeof(double) : 0));
+    if (st != COSMICA_OK) return st;
+    st = istage.reserve(up);
+    if (st != COSMICA_OK) return st;
+    std::memcpy(istage.h, si.its.data(), n_items * sizeof(SpecItem));
+    std::memcpy((char *)istage.h + b_items, si.sp_item.data(), n_sp * sizeof(uint32_t));
+    st = istage.upload(ibuf.d, up, s);
+    if (st != COSMICA_OK) return st;
+    int kind; const double *lnT, *lnJ; uint32_t ln;
+    st = upload_lis(lis, lbuf, lstage, s, &kind, &lnT, &lnJ, &ln);
+    if (st != COSMICA_OK) return st;
+    const SpecItem *d_items = (const SpecItem *)ibuf.d;
+    void *d_sums = (char *)ibuf.d + up;
+    double *d_w = table ? (double *)((char *)ibuf.d + up + b_sums) : nullptr;
+    unsigned long long *h = (unsigned long long *)hist;
+    cudaError_t e = launch_spec_prep(h, ex ? (uint64_t)n_items * COSMICA_HIST_STRIDE(nbins) : 0, d_items,
+                                     (const uint32_t *)((const char *)ibuf.d + b_items), n_sp, nbins, x_lo, dx, kind,
+                                     lnT, lnJ, ln, d_w, s);
+    if (e != cudaSuccess) return cuda_fail(e, "spectrum set-up launch");
+    if (ex) e = launch_histogram(exit_ptrs(ex), ex->n, n_items, nbins, x_lo, dx, h, num_sms(), s);
+    if (e != cudaSuccess) return cuda_fail(e, "histogram kernel launch");
+    e = launch_spectrum(h, n_items, nbins, x_lo, dx, d_items, d_w, kind, lnT, lnJ, ln, d_sums, J, sigma, s);
+    return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "spectrum kernel launch");
+}
+
+static cosmica_status run_spectrum(const cosmica_exit_states *ex, const SpecItems &si,
                                    const cosmica_lis *lis, const cosmica_bins *bins, double *J, double *sigma,
                                    uint64_t *hist, DevBuf &ibuf, Staging &istage, DevBuf &lbuf, Staging &lstage,
                                    cudaStream_t s)
@@ -689,42 +739,14 @@ static cosmica_status run_spectrum(const cosmica_exit_states *ex, const std::vec
     double x_lo, dx;
     cosmica_status st = check_bins(bins, &x_lo, &dx);
     if (st != COSMICA_OK) return st;
-    const uint32_t n_items = (uint32_t)its.size();
-    if (n_items == 0) return COSMICA_OK;
+    if (si.its.empty()) return COSMICA_OK;
     if (!J || !sigma || !hist) return fail(COSMICA_ERR_INVALID, "J / sigma / hist must be non-NULL");
     if (!ex) return fail(COSMICA_ERR_INVALID, "exit states NULL");
     if (ex->n > 0 && !valid_exit(ex)) return fail(COSMICA_ERR_INVALID, "exit-state arrays must be non-NULL");
     if (ex->n > 0 && !is_device_ptr(ex->lnP)) return fail(COSMICA_ERR_INVALID, "exit states must be device memory");
     if (!is_device_ptr(J) || !is_device_ptr(sigma) || !is_device_ptr(hist))
         return fail(COSMICA_ERR_INVALID, "J / sigma / hist must be device memory");
-    const size_t hbytes = (size_t)n_items * COSMICA_HIST_STRIDE(bins->nbins) * sizeof(uint64_t);
-    CK(cudaMemsetAsync(hist, 0, hbytes, s), "cudaMemsetAsync(hist)");
-    cudaError_t e = launch_histogram(exit_ptrs(ex), ex->n, n_items, bins->nbins, x_lo, dx,
-                                     (unsigned long long *)hist, s);
-    if (e != cudaSuccess) return cuda_fail(e, "histogram kernel launch");
-    return spectrum_of_hist(its, lis, bins->nbins, x_lo, dx, hist, J, sigma, ibuf, istage, lbuf, lstage, s);
-}
-
-// Eq. 4 per item from a histogram already in device memory (the second half of run_spectrum).
-static cosmica_status spectrum_of_hist(const std::vector<SpecItem> &its, const cosmica_lis *lis, uint32_t nbins,
-                                       double x_lo, double dx, const uint64_t *hist, double *J, double *sigma,
-                                       DevBuf &ibuf, Staging &istage, DevBuf &lbuf, Staging &lstage, cudaStream_t s)
-{
-    const uint32_t n_items = (uint32_t)its.size();
-    cosmica_status st = ibuf.reserve(n_items * sizeof(SpecItem));
-    if (st != COSMICA_OK) return st;
-    st = istage.reserve(n_items * sizeof(SpecItem));
-    if (st != COSMICA_OK) return st;
-    std::memcpy(istage.h, its.data(), n_items * sizeof(SpecItem));
-    st = istage.upload(ibuf.d, n_items * sizeof(SpecItem), s);
-    if (st != COSMICA_OK) return st;
-    int kind; const double *lnT, *lnJ; uint32_t ln;
-    st = upload_lis(lis, lbuf, lstage, s, &kind, &lnT, &lnJ, &ln);
-    if (st != COSMICA_OK) return st;
-    cudaError_t e = launch_spectrum((const unsigned long long *)hist, n_items, nbins, x_lo, dx,
-                                    (const SpecItem *)ibuf.d, kind, lnT, lnJ, ln, J, sigma, s);
-    if (e != cudaSuccess) return cuda_fail(e, "spectrum kernel launch");
-    return COSMICA_OK;
+    return spectrum_of(ex, si, lis, bins->nbins, x_lo, dx, hist, J, sigma, ibuf, istage, lbuf, lstage, s);
 }
 
 extern "C" cosmica_status cosmica_spectrum(const cosmica_exit_states *exit, const cosmica_species *species,
@@ -735,13 +757,14 @@ extern "C" cosmica_status cosmica_spectrum(const cosmica_exit_states *exit, cons
     cosmica_status st = check_species(species);
     if (st != COSMICA_OK) return st;
     if (n_energies > 0 && !T_in) return fail(COSMICA_ERR_INVALID, "T_in is NULL");
-    std::vector<SpecItem> its(n_energies);
-    for (uint32_t e = 0; e < n_energies; ++e)
-        its[e] = SpecItem{T_in[e], (double)species->A, (double)species->Z, species->m0_GeV};
+    SpecItems si;
+    si.its.reserve(n_energies);
+    uint32_t number = UINT32_MAX;
+    for (uint32_t e = 0; e < n_energies; ++e) si.add(T_in[e], *species, number);
     // scratch of the calling thread: the spectrum call carries no handle
     thread_local DevBuf ibuf, lbuf;
     thread_local Staging istage, lstage;
-    return run_spectrum(exit, its, lis, bins, J_out, sigma_out, hist_out, ibuf, istage, lbuf, lstage,
+    return run_spectrum(exit, si, lis, bins, J_out, sigma_out, hist_out, ibuf, istage, lbuf, lstage,
                         (cudaStream_t)stream);
 }
 
@@ -766,26 +789,34 @@ extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *e
     cudaStream_t s = (cudaStream_t)stream;
     thread_local DevBuf buf, lbuf;
     thread_local Staging stage, lstage;
+    // items, prefix sums of the particles and of the chunks; behind them the chunks' partial sums
+    const uint32_t per = unbinned_per_thread(total, num_sms());
     const size_t b_items = align_up(n_energies * sizeof(SpecItem), 256);
-    const size_t bytes = b_items + (n_energies + 1) * sizeof(uint64_t);
-    st = buf.reserve(bytes);
-    if (st != COSMICA_OK) return st;
+    const size_t b_pre = align_up((n_energies + 1) * sizeof(uint64_t), 256);
+    const size_t bytes = b_items + 2 * b_pre;
     st = stage.reserve(bytes);
     if (st != COSMICA_OK) return st;
     SpecItem *hi = (SpecItem *)stage.h;
     uint64_t *hp = (uint64_t *)((char *)stage.h + b_items);
-    hp[0] = 0;
+    uint64_t *hc = (uint64_t *)((char *)stage.h + b_items + b_pre);
+    hp[0] = hc[0] = 0;
     for (uint32_t e = 0; e < n_energies; ++e) {
-        hi[e] = SpecItem{T_in[e], (double)species->A, (double)species->Z, species->m0_GeV};
+        hi[e] = SpecItem{T_in[e], (double)species->A, (double)species->Z, species->m0_GeV, 0u, 0u};
         hp[e + 1] = hp[e] + n_per_energy[e];
+        hc[e + 1] = hc[e] + unbinned_chunks(n_per_energy[e], per);
     }
+    const uint64_t n_chunks = hc[n_energies];
+    st = buf.reserve(bytes + n_chunks * unbinned_partial_bytes());
+    if (st != COSMICA_OK) return st;
     st = stage.upload(buf.d, bytes, s);
     if (st != COSMICA_OK) return st;
     int kind; const double *lnT, *lnJ; uint32_t ln;
     st = upload_lis(lis, lbuf, lstage, s, &kind, &lnT, &lnJ, &ln);
     if (st != COSMICA_OK) return st;
-    cudaError_t e = launch_spectrum_unbinned(exit_ptrs(exit), (const uint64_t *)((char *)buf.d + b_items), n_energies,
-                                             (const SpecItem *)buf.d, formulation, kind, lnT, lnJ, ln, J_out,
+    char *d = (char *)buf.d;
+    cudaError_t e = launch_spectrum_unbinned(exit_ptrs(exit), (const uint64_t *)(d + b_items),
+                                             (const uint64_t *)(d + b_items + b_pre), n_chunks, per, d + bytes,
+                                             n_energies, (const SpecItem *)d, formulation, kind, lnT, lnJ, ln, J_out,
                                              sigma_out, s);
     return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "unbinned spectrum launch");
 }
@@ -1003,6 +1034,19 @@ extern "C" cosmica_status cosmica_batch_run(cosmica_batch *b, const cosmica_work
     return COSMICA_OK;
 }
 
+static cosmica_status batch_spec_items(const cosmica_batch *b, const cosmica_work_item *items, uint32_t n_items,
+                                       SpecItems &si)
+{
+    si.its.reserve(n_items);
+    std::vector<uint32_t> number(b->species.size(), UINT32_MAX);
+    for (uint32_t i = 0; i < n_items; ++i) {
+        const uint32_t k = items[i].species_idx;
+        if (k >= b->species.size()) return fail(COSMICA_ERR_INVALID, "species index out of range");
+        si.add(items[i].T_GeVn, b->species[k], number[k]);
+    }
+    return COSMICA_OK;
+}
+
 extern "C" cosmica_status cosmica_batch_spectrum(cosmica_batch *b, const cosmica_work_item *items,
                                                  uint32_t n_items, const cosmica_exit_states *exit,
                                                  const cosmica_lis *lis, const cosmica_bins *bins, double *J_out,
@@ -1010,13 +1054,10 @@ extern "C" cosmica_status cosmica_batch_spectrum(cosmica_batch *b, const cosmica
 {
     if (!b) return fail(COSMICA_ERR_INVALID, "batch is NULL");
     if (n_items > 0 && !items) return fail(COSMICA_ERR_INVALID, "items is NULL");
-    std::vector<SpecItem> its(n_items);
-    for (uint32_t i = 0; i < n_items; ++i) {
-        if (items[i].species_idx >= b->species.size()) return fail(COSMICA_ERR_INVALID, "species index out of range");
-        const cosmica_species &sp = b->species[items[i].species_idx];
-        its[i] = SpecItem{items[i].T_GeVn, (double)sp.A, (double)sp.Z, sp.m0_GeV};
-    }
-    return run_spectrum(exit, its, lis, bins, J_out, sigma_out, hist_out, b->spec_items, b->spec_stage,
+    SpecItems si;
+    cosmica_status st = batch_spec_items(b, items, n_items, si);
+    if (st != COSMICA_OK) return st;
+    return run_spectrum(exit, si, lis, bins, J_out, sigma_out, hist_out, b->spec_items, b->spec_stage,
                         b->lis_buf, b->lis_stage, (cudaStream_t)stream);
 }
 
@@ -1034,14 +1075,12 @@ extern "C" cosmica_status cosmica_batch_spectrum_hist(cosmica_batch *b, const co
     if (!J_out || !sigma_out || !hist) return fail(COSMICA_ERR_INVALID, "J / sigma / hist must be non-NULL");
     if (!is_device_ptr(J_out) || !is_device_ptr(sigma_out) || !is_device_ptr(hist))
         return fail(COSMICA_ERR_INVALID, "J / sigma / hist must be device memory");
-    std::vector<SpecItem> its(n_items);
-    for (uint32_t i = 0; i < n_items; ++i) {
-        if (items[i].species_idx >= b->species.size()) return fail(COSMICA_ERR_INVALID, "species index out of range");
-        const cosmica_species &sp = b->species[items[i].species_idx];
-        its[i] = SpecItem{items[i].T_GeVn, (double)sp.A, (double)sp.Z, sp.m0_GeV};
-    }
-    return spectrum_of_hist(its, lis, bins->nbins, x_lo, dx, hist, J_out, sigma_out, b->spec_items, b->spec_stage,
-                            b->lis_buf, b->lis_stage, (cudaStream_t)stream);
+    SpecItems si;
+    st = batch_spec_items(b, items, n_items, si);
+    if (st != COSMICA_OK) return st;
+    // the histogram is read only: no exit states, nothing is cleared
+    return spectrum_of(nullptr, si, lis, bins->nbins, x_lo, dx, const_cast<uint64_t *>(hist), J_out, sigma_out,
+                       b->spec_items, b->spec_stage, b->lis_buf, b->lis_stage, (cudaStream_t)stream);
 }
 
 // =============================================================== autotune ==

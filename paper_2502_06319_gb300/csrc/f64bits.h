@@ -80,6 +80,18 @@ COSMICA_HD float pi_minus(uint64_t diff)
 #endif
 }
 
+// the double of a 32-bit count, exact
+COSMICA_HD uint64_t from_u32(uint32_t n)
+{
+    if (n == 0u) return 0ull;
+#if defined(__CUDA_ARCH__)
+    const int sh = __clz(n);
+#else
+    const int sh = __builtin_clz(n);
+#endif
+    return ((uint64_t)(1053 - sh) << 52) + ((uint64_t)(n << sh) << 21);   // the leading one carries into the exponent
+}
+
 // FP64 comparisons on the bits, with b > 0 finite: right for every a but NaN.
 COSMICA_HD bool less(uint64_t a, uint64_t b) { return (int64_t)a < (int64_t)b; }
 // a < 0 or a > b (a = -0 counts as below 0: the caller decides with FP64 comparisons then)

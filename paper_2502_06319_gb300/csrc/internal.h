@@ -97,18 +97,32 @@ inline bool full_model(const cosmica_params &p)
 cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, cudaStream_t s);
 int mixed_max_blocks_per_sm(MixedVariant v, unsigned block, bool compact);
 
-cudaError_t launch_histogram(const ExitPtrs &ex, uint64_t n, uint32_t n_items, uint32_t nbins, double x_lo,
-                             double dx, unsigned long long *hist, cudaStream_t s);
 struct SpecItem {
     double T;                  // GeV/n
     double A, Z, m0;           // species
+    uint32_t sp, pad;          // row of the species in the table of bin weights
 };
+// clears hist[0 .. n_hist) and fills weights [n_sp x nbins] (none for null weights), species s
+// being that of items[sp_item[s]]
+cudaError_t launch_spec_prep(unsigned long long *hist, uint64_t n_hist, const SpecItem *items, const uint32_t *sp_item,
+                             uint32_t n_sp, uint32_t nbins, double x_lo, double dx, int lis_kind, const double *lis_lnT,
+                             const double *lis_lnJ, uint32_t lis_n, double *weights, cudaStream_t s);
+cudaError_t launch_histogram(const ExitPtrs &ex, uint64_t n, uint32_t n_items, uint32_t nbins, double x_lo,
+                             double dx, unsigned long long *hist, int sms, cudaStream_t s);
+// weights: from launch_spec_prep, or null (every item evaluates its own); sums: scratch of
+// n_items x spectrum_sums_bytes()
+size_t spectrum_sums_bytes();
 cudaError_t launch_spectrum(const unsigned long long *hist, uint32_t n_items, uint32_t nbins,
-                            double x_lo, double dx, const SpecItem *items, int lis_kind,
-                            const double *lis_lnT, const double *lis_lnJ, uint32_t lis_n,
+                            double x_lo, double dx, const SpecItem *items, const double *weights, int lis_kind,
+                            const double *lis_lnT, const double *lis_lnJ, uint32_t lis_n, void *sums,
                             double *J, double *sigma, cudaStream_t s);
 
-cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix, uint32_t n_items,
+// unbinned estimator: chunks of `per` x 128 exit states of one item, chunk_prefix their prefix sums over items
+uint32_t unbinned_per_thread(uint64_t n, int sms);
+uint64_t unbinned_chunks(uint64_t n, uint32_t per);
+size_t unbinned_partial_bytes();
+cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix, const uint64_t *chunk_prefix,
+                                     uint64_t n_chunks, uint32_t per, void *partials, uint32_t n_items,
                                      const SpecItem *items, int form, int lis_kind, const double *lis_lnT,
                                      const double *lis_lnJ, uint32_t lis_n, double *J, double *sigma, cudaStream_t s);
 

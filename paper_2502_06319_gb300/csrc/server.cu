@@ -120,7 +120,7 @@ struct cosmica_server {
     unsigned long long *d_hist = nullptr;
     double *d_J = nullptr, *d_S = nullptr;
     SpecItem *d_spec_items = nullptr;
-    DevBuf tables;
+    DevBuf tables, weights;
     Staging stage;
     // pinned read-back of the per-quantum counters
     unsigned long long *h_cursor = nullptr;
@@ -183,16 +183,28 @@ bool cosmica_server::retire(uint64_t ticket, Req &r)
     ExitPtrs ex{arena.r + r.base, arena.th + r.base, arena.ph + r.base, arena.lnP + r.base, arena.s + r.base,
                 arena.steps + r.base, arena.status + r.base, arena.item + r.base};
     std::vector<SpecItem> its(nE);
-    for (uint32_t e = 0; e < nE; ++e) its[e] = SpecItem{r.T[e], (double)r.sp.A, (double)r.sp.Z, r.sp.m0_GeV};
+    for (uint32_t e = 0; e < nE; ++e) its[e] = SpecItem{r.T[e], (double)r.sp.A, (double)r.sp.Z, r.sp.m0_GeV, 0u, 0u};
     r.H.assign((size_t)nE * stride, 0);
     r.J.assign(nE, 0.0);
     r.S.assign(nE, 0.0);
-    cudaError_t e = cudaMemsetAsync(d_hist, 0, (size_t)nE * stride * 8, stream);
+    // bin weights of the request's one species, and its number of an item that has it (0)
+    const size_t b_sums = align_up(nE * spectrum_sums_bytes(), 256);
+    if (weights.reserve(256 + b_sums + (size_t)nb * sizeof(double)) != COSMICA_OK) {
+        set_failed(std::string("server retire: ") + cosmica_last_error());
+        return false;
+    }
+    void *d_sums = (char *)weights.d + 256;
+    double *d_w = (double *)((char *)weights.d + 256 + b_sums);
+    cudaError_t e = cudaMemsetAsync(weights.d, 0, 256, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_spec_items, its.data(), nE * sizeof(SpecItem),
                                               cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = launch_histogram(ex, r.total, nE, nb, x_lo, dx, d_hist, stream);
     if (e == cudaSuccess)
-        e = launch_spectrum(d_hist, nE, nb, x_lo, dx, d_spec_items, 0, nullptr, nullptr, 0, d_J, d_S, stream);
+        e = launch_spec_prep(d_hist, (uint64_t)nE * stride, d_spec_items, (const uint32_t *)weights.d, 1, nb, x_lo, dx, 0,
+                             nullptr, nullptr, 0, d_w, stream);
+    if (e == cudaSuccess) e = launch_histogram(ex, r.total, nE, nb, x_lo, dx, d_hist, num_sms(), stream);
+    if (e == cudaSuccess)
+        e = launch_spectrum(d_hist, nE, nb, x_lo, dx, d_spec_items, d_w, 0, nullptr, nullptr, 0, d_sums, d_J, d_S,
+                            stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(r.H.data(), d_hist, (size_t)nE * stride * 8, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(r.J.data(), d_J, nE * 8, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(r.S.data(), d_S, nE * 8, cudaMemcpyDeviceToHost, stream);
@@ -383,7 +395,7 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     s->shape = PersistentShape{block, (unsigned)(num_sms() * bps), 0u};
     s->lane_cap = (uint64_t)s->shape.grid * block;
     const size_t fixed = 2 * s->lane_cap * sizeof(Suspended) + kMaxSlots * (sizeof(DevParams) + sizeof(DevSpecies) + 12) +
-                         (size_t)kMaxEnergies * (kMaxBins + 3) * 8 + kMaxEnergies * (16 + sizeof(SpecItem)) + 4096;
+                         (size_t)kMaxEnergies * (kMaxBins + 3) * 8 + kMaxEnergies * 48 + 4096;
     const size_t per = 5 * 8 + 4 + 4 + 1;
     if (mem_budget <= fixed + 256 * per) {
         delete s;
@@ -547,6 +559,7 @@ extern "C" void cosmica_server_destroy(cosmica_server *s)
     if (s->th.joinable()) s->th.join();
     if (s->stream) cudaStreamSynchronize(s->stream);
     s->tables.release();
+    s->weights.release();
     s->stage.release();
     void *dev[] = {s->arena_mem, s->d_prm, s->d_spc, s->d_done, s->d_steps, s->d_susp[0], s->d_susp[1],
                    s->d_nsusp, s->d_cursors, s->d_hist, s->d_J, s->d_S, s->d_spec_items};

@@ -19,6 +19,7 @@ void t_narrow(const uint64_t *u, uint32_t *o, uint8_t *ok, int n)
 { for (int i = 0; i < n; ++i) { ok[i] = narrow_ok((uint32_t)(u[i] >> 32)); o[i] = narrow(u[i]); } }
 void t_pi_minus(const uint64_t *u, float *o, uint8_t *ok, int n)
 { for (int i = 0; i < n; ++i) { uint64_t d = pi_minus_units(u[i]); ok[i] = pi_minus_ok(d); o[i] = ok[i] ? pi_minus(d) : 0.0f; } }
+void t_count(const uint32_t *u, uint64_t *o, int n) { for (int i = 0; i < n; ++i) o[i] = from_u32(u[i]); }
 void t_cmp(const uint64_t *a, const uint64_t *b, uint8_t *l, uint8_t *oc, uint8_t *oh, uint8_t *fin, int n)
 { for (int i = 0; i < n; ++i) { l[i] = less(a[i], b[i]); oc[i] = outside_closed(a[i], b[i]);
     oh[i] = outside_half_open(a[i], b[i]); fin[i] = is_finite(a[i]); } }
@@ -81,6 +82,15 @@ def test_pi_minus(lib):
     assert np.array_equal(ok.astype(bool), d >= 2.0 ** -20)
     k = ok.astype(bool)
     assert np.array_equal(o[k], d[k].astype(np.float32))
+
+
+def test_count(lib):
+    rng = np.random.default_rng(5)
+    u = np.concatenate([rng.integers(0, 2 ** 32, 50000, dtype=np.uint64), np.arange(40, dtype=np.uint64),
+                        np.uint64(1) << np.arange(32, dtype=np.uint64), np.array([2 ** 32 - 1], dtype=np.uint64)]).astype(np.uint32)
+    o = np.empty(len(u), np.uint64)
+    lib.t_count(p(u), p(o), len(u))
+    assert np.array_equal(o.view(np.float64), u.astype(np.float64))
 
 
 def test_comparisons(lib):
