@@ -56,6 +56,18 @@ struct alignas(16) F32Params {
     float ts_R, ts_c, ts_ia2, ts_ib2, ts_C, hp_c, hp_ia2, hp_ib2;
 };
 
+// FP64 values of one heliosphere that its step would otherwise form again and again, in the
+// step's own operations (step64.cuh); r_x is the reciprocal of x.
+struct F64Params {
+    double Vs, hdV;            // slow wind (the isotropic model's wind), (fast - slow)/2 [AU/day]
+    double lat_f, dlat, r_dlat, Omega;
+    double hts, r_dts;         // (1 - ts_f)/2
+    double ta, ta2, dmin;      // tan(tilt), its square, sheet half-width floor [rad]
+    double dDen, r_dDen;       // r_L / r denominators: D = P 1e9 / dDen
+    double caDen, r_caDen;     // kappa_A: C_A = beta P 1e9 day / caDen
+    double eps_adv2, sdt_fixed;
+};
+
 struct DevParams {
     // raw values (FP64 step)
     double K0, er, et, B1AU, Vs_kms, Vf_kms, lat_fast_deg, tilt_deg, polarity;
@@ -69,6 +81,7 @@ struct DevParams {
     int32_t precision, pad;
     // derived on the device
     double B0;                 // nT, |B|(1 AU, equator) = B1AU
+    F64Params d;
     F32Params f;
 };
 

@@ -258,7 +258,9 @@ struct Tables {
     uint64_t *prefix = nullptr;
     uint32_t *qitem = nullptr;               // item of each queue slot
     uint64_t *qprefix = nullptr;             // prefix sums in queue order
-    unsigned long long *counters = nullptr;   // [0] cursor, [1] steps
+    unsigned long long *counters = nullptr;   // kLaunchCounters of a launch
+    uint32_t *list = nullptr;                 // paths an FP64 launch leaves to its second kernel
+    uint32_t list_cap = 0;
     uint64_t n_total = 0;
     uint32_t n_items = 0;
 
@@ -271,7 +273,8 @@ struct Tables {
         const size_t b_pre = align_up((nI + 1) * sizeof(uint64_t), 256);
         const size_t b_q = align_up(std::max<size_t>(1, nI) * sizeof(uint32_t), 256);
         const size_t up = b_items + 2 * b_pre + b_q;
-        cosmica_status st = dev.reserve(up + 256);
+        list_cap = fp64_list_entries(num_sms());
+        cosmica_status st = dev.reserve(up + 256 + list_cap * sizeof(uint32_t));
         if (st != COSMICA_OK) return st;
         st = stage.reserve(up);
         if (st != COSMICA_OK) return st;
@@ -292,6 +295,7 @@ struct Tables {
         qprefix = (uint64_t *)(d + b_items + b_pre);
         qitem = (uint32_t *)(d + b_items + 2 * b_pre);
         counters = (unsigned long long *)(d + up);
+        list = (uint32_t *)(d + up + 256);
         n_items = (uint32_t)nI;
         n_total = pre[nI];
         return stage.upload(dev.d, up, s);
@@ -544,12 +548,14 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
         st = m->exit_stage.make(total, ex, out->lw != nullptr);
         if (st != COSMICA_OK) return st;
     }
-    CK(cudaMemsetAsync(m->tab.counters, 0, 2 * sizeof(unsigned long long), s), "cudaMemsetAsync(counters)");
+    CK(cudaMemsetAsync(m->tab.counters, 0, kLaunchCounters * sizeof(unsigned long long), s),
+       "cudaMemsetAsync(counters)");
     LaunchArgs a{m->d_prm, d_sp, m->tab.items, m->tab.prefix, m->tab.n_items, total, ex,
-                 m->tab.counters + 1, m->tab.counters, m->tab.qitem, m->tab.qprefix, m->d_f32};
+                 m->tab.counters + 1, m->tab.counters, m->tab.qitem, m->tab.qprefix, m->d_f32,
+                 m->tab.list, m->tab.list_cap, m->tab.counters + 2};
     cudaError_t e;
     if (m->p.precision == COSMICA_PREC_FP64) {
-        e = launch_propagate_fp64(a, s);
+        e = launch_propagate_fp64(a, fp64_variant(&m->p, 1), num_sms(), s);
     } else {
         const MixedVariant v{m->p.precision, m->p.formulation == 1, m->p.n_shells > 0 || m->p.squashed != 0,
                              full_model(m->p)};
@@ -947,11 +953,13 @@ static cosmica_status batch_launch(cosmica_batch *b, uint64_t total, const ExitP
                                    const cosmica_tuning *tuning, cudaStream_t s)
 {
     LaunchArgs a{b->d_prm, b->d_spc, b->tab.items, b->tab.prefix, b->tab.n_items, total, ex,
-                 b->tab.counters + 1, b->tab.counters, b->tab.qitem, b->tab.qprefix, b->d_f32};
+                 b->tab.counters + 1, b->tab.counters, b->tab.qitem, b->tab.qprefix, b->d_f32,
+                 b->tab.list, b->tab.list_cap, b->tab.counters + 2};
     auto direct = [&]() -> cosmica_status {
-        CK(cudaMemsetAsync(b->tab.counters, 0, 2 * sizeof(unsigned long long), s), "cudaMemsetAsync(counters)");
+        CK(cudaMemsetAsync(b->tab.counters, 0, kLaunchCounters * sizeof(unsigned long long), s),
+       "cudaMemsetAsync(counters)");
         cudaError_t e = (b->precision == COSMICA_PREC_FP64)
-                            ? launch_propagate_fp64(a, s)
+                            ? launch_propagate_fp64(a, fp64_variant(b->params.data(), b->params.size()), num_sms(), s)
                             : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total), s);
         if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
         return COSMICA_OK;

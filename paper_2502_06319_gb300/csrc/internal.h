@@ -24,6 +24,11 @@ struct LaunchArgs {
     const uint32_t *qitem;             // item of each queue slot (null: item order)
     const uint64_t *qprefix;           // prefix sums of particle counts in queue order
     const float *f32;                  // FP32 blocks of the parameter sets, paged field-major (P32)
+    // FP64 path: indices of the paths left to the team kernel, room for list_cap of them, and two
+    // counters (paths ended, paths left); cleared like the cursor
+    uint32_t *list;
+    uint32_t list_cap;
+    unsigned long long *ended;         // [0] ended, [1] left
 };
 
 struct PersistentShape {
@@ -79,7 +84,15 @@ void note_launch();
 
 cudaError_t launch_derive(DevParams *prm, uint32_t n, cudaStream_t s);
 cudaError_t launch_f32_table(const DevParams *prm, uint32_t n, float *table, cudaStream_t s);
-cudaError_t launch_propagate_fp64(const LaunchArgs &a, cudaStream_t s);
+// variant of the FP64 kernels: extended sets (shells, squashed) take the plain step; iso: every set is isotropic
+struct Fp64Variant {
+    bool energy, extended, iso, aniso;   // iso / aniso: some set is (not) isotropic
+};
+// counters of a launch: queue cursor, steps, paths ended, paths left to the team kernel
+constexpr uint32_t kLaunchCounters = 4;
+// most paths the team kernel takes over (32 per SM: eight teams of four lanes on every scheduler)
+inline uint32_t fp64_list_entries(int sms) { return 32u * (uint32_t)sms; }
+cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, cudaStream_t s);
 
 // mixed precision persistent kernel; acc = COSMICA_PREC_MIXED or COSMICA_PREC_MIXED_F64ACC
 // compile-time variant of the mixed kernel a launch needs
@@ -89,6 +102,15 @@ struct MixedVariant {
     bool extended;  // some parameter set of the launch has radial shells or a squashed heliosphere
     bool full;      // every set is the full model: drift and current sheet on, adaptive step
 };
+inline Fp64Variant fp64_variant(const cosmica_params *ps, size_t n)
+{
+    Fp64Variant v{ps[0].formulation == 1, false, false, false};
+    for (size_t i = 0; i < n; ++i) {
+        v.extended = v.extended || ps[i].n_shells > 0 || ps[i].squashed != 0;
+        (ps[i].isotropic ? v.iso : v.aniso) = true;
+    }
+    return v;
+}
 // a set is the full model of the mixed kernels' FULL variant
 inline bool full_model(const cosmica_params &p)
 {

@@ -2,15 +2,20 @@
 // is evaluated exactly as written (no fused multiply-add contraction).
 //
 //   k_derive          per-parameter-set constants (FP64 and the FP32 block)
-//   k_propagate_fp64  the plain FP64 path: one thread per quasi-particle
-//                     (Sec. IV.A), Euler-Maruyama until the path exits
+//   k_propagate64     the FP64 path: one lane per quasi-particle (Sec. IV.A), refilled from
+//                     the work queue, Euler-Maruyama until the path exits (step64.cuh)
+//   k_finish64        the last paths of a launch, or all of a small one: teams of lanes
+//   k_propagate_fp64  sets with radial shells or a squashed heliosphere: one thread per
+//                     quasi-particle, the step as it is defined (model64.cuh)
 //   k_debug_*         coefficient / RNG / elementary-function probes used by
 //                     the tests through cosmica_debug.h
+#include <algorithm>
 #include <cstdint>
 
 #include "common.cuh"
 #include "internal.h"
 #include "model64.cuh"
+#include "step64.cuh"
 
 namespace cosmica {
 
@@ -21,6 +26,31 @@ __global__ void k_derive(DevParams *prm, uint32_t n)
     DevParams &p = prm[i];
     const bool iso = p.isotropic != 0.0;
     p.B0 = iso ? 0.0 : m64::field_B0(p);
+    {
+        // in the operations of model64.cuh
+        F64Params &d = p.d;
+        const double Vs64 = iso ? p.V_const_kms * kDay_s / kAU_km : p.Vs_kms * kDay_s / kAU_km;
+        const double Vf64 = p.Vf_kms * kDay_s / kAU_km;
+        d.Vs = Vs64;
+        d.hdV = iso ? 0.0 : (Vf64 - Vs64) * 0.5;
+        d.lat_f = p.lat_fast_deg * kDeg;
+        d.dlat = p.dlat_deg * kDeg;
+        d.r_dlat = 1.0 / d.dlat;
+        d.Omega = iso ? 0.0 : kTwoPi / p.rot_period;
+        d.hts = (1.0 - p.ts_f) * 0.5;
+        d.r_dts = 1.0 / p.dts;
+        double s64, c64;
+        dm::sincos(p.tilt_deg * kDeg, &s64, &c64);
+        d.ta = s64 / c64;
+        d.ta2 = d.ta * d.ta;
+        d.dmin = p.dcs_min_deg * kDeg;
+        d.dDen = kC_ms * p.B0 * 1e-9 * kAU_m;
+        d.r_dDen = 1.0 / d.dDen;
+        d.caDen = 3.0 * p.B0 * 1e-9 * kAU_m * kAU_m;
+        d.r_caDen = 1.0 / d.caDen;
+        d.eps_adv2 = p.eps_adv * 2.0;
+        d.sdt_fixed = p.dt_fixed > 0.0 ? sqrt(p.dt_fixed) : 0.0;
+    }
     F32Params &f = p.f;
     const double Vs = iso ? p.V_const_kms * kDay_s / kAU_km : p.Vs_kms * kDay_s / kAU_km;
     const double Vf = iso ? Vs : p.Vf_kms * kDay_s / kAU_km;
@@ -124,6 +154,206 @@ __global__ void __launch_bounds__(128) k_propagate_fp64(const DevParams *__restr
     }
 }
 
+// ---- FP64 paths of the models without shells or squashing -----------------------------
+// Bound by the FP64 pipe: a step costs its slots times 64 clocks on the warp's scheduler
+// whatever lanes are active (step64.cuh), so
+//   * one warp per scheduler (one block of 128 per SM) already fills the pipe; lanes whose
+//     path ended take the next one from the queue, most expensive items first;
+//   * once no more than 32 paths per SM are left, every lane stores its path in its own exit
+//     record and k_finish64 takes them over with four lanes a path, which halves the slots of
+//     the step that the launch's slowest paths wait for; a launch that starts with so few
+//     goes there at once, with 16 lanes a path when there are eight paths per SM or fewer.
+// Measured against one thread per path with the plain step: 1e4 isotropic paths 86.8 -> 24.4 ms
+// (10 ms of it in the first kernel), 96 paths of the full model 349 -> 114 ms (52 -> 16.9 us a
+// step; the FP64 pipe 82 % busy), 2.5e4 paths 1384 -> 509 ms; the paths are the same bits.
+struct Path64 {
+    uint64_t g, pid, seed;
+    const DevParams *p;
+    const DevSpecies *dsp;
+    uint32_t out_item, max_steps;
+    s64::Spc sp;
+};
+
+__device__ __forceinline__ void locate64(const LaunchArgs &a, uint32_t it, uint64_t local, Path64 &P, DevItem &item)
+{
+    item = a.items[it];
+    P.g = a.prefix[it] + local;
+    P.pid = item.first_pid + local;
+    P.seed = item.seed;
+    P.p = a.prm + item.param_idx;
+    P.dsp = a.spc + item.species_idx;
+    P.out_item = item.out_item;
+    P.max_steps = (uint32_t)P.p->max_steps;
+    P.sp = s64::make_spc(*P.dsp);
+}
+
+// the path in queue slot q, at its start
+__device__ __forceinline__ void fresh64(const LaunchArgs &a, uint64_t q, Path64 &P, m64::State &x)
+{
+    const uint32_t iq = find_item(a.qprefix, a.n_items, q);
+    DevItem item;
+    locate64(a, a.qitem ? a.qitem[iq] : iq, q - a.qprefix[iq], P, item);
+    m64::init_state(*P.dsp, item.T, item.r0, item.th0, item.ph0, x);
+}
+
+// the path whose state waits in exit record g (EN: lnP's place holds T, which gives lnP)
+template <bool EN>
+__device__ __forceinline__ void stored64(const LaunchArgs &a, uint64_t g, Path64 &P, m64::State &x)
+{
+    const uint32_t it = find_item(a.prefix, a.n_items, g);
+    DevItem item;
+    locate64(a, it, g - a.prefix[it], P, item);
+    m64::init_state(*P.dsp, item.T, item.r0, item.th0, item.ph0, x);
+    x.r = a.out.r[g];
+    x.th = a.out.th[g];
+    x.ph = a.out.ph[g];
+    x.s = a.out.s[g];
+    x.k = a.out.steps[g];
+    x.lnP = a.out.lnP[g];
+    if constexpr (EN) {
+        x.T = x.lnP;
+        x.Lam = -a.out.lw[g];
+        x.lnP = dm::log(P.dsp->A / fabs(P.dsp->Z) * sqrt(x.T * (x.T + 2.0 * P.dsp->m0)));
+    }
+}
+
+template <bool EN>
+__device__ __forceinline__ void store64(const ExitPtrs &out, const Path64 &P, const m64::State &x)
+{
+    const uint64_t g = P.g;
+    out.r[g] = x.r;
+    out.th[g] = x.th;
+    out.ph[g] = x.ph;
+    out.lnP[g] = EN && x.status == COSMICA_PATH_RUNNING ? x.T : x.lnP;
+    out.s[g] = x.s;
+    out.steps[g] = x.k;
+    out.status[g] = (uint8_t)x.status;
+    out.item[g] = P.out_item;
+    if (out.lw) out.lw[g] = -x.Lam;
+}
+
+// ISO: 1 every set is isotropic, 0 none, 2 both occur
+template <int G, int ISO, bool EN>
+__device__ __forceinline__ void step64(const Path64 &P, const double *tab, s64::Team<G> team, const double (&z)[3], bool live,
+                                       m64::State &x)
+{
+    if constexpr (ISO == 2) {
+        // teams of a warp may hold different models: all of them run each form that one of them needs
+        // (its shuffles take the whole warp), and each keeps its own
+        const bool iso = P.p->isotropic != 0.0;
+        if (G == 1 ? iso : __any_sync(0xffffffffu, iso))
+            s64::step<G, true, EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, tab, team, z, live && iso, x);
+        if (G == 1 ? !iso : __any_sync(0xffffffffu, !iso))
+            s64::step<G, false, EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, tab, team, z, live && !iso, x);
+    } else {
+        s64::step<G, ISO == 1, EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, tab, team, z, live, x);
+    }
+}
+
+template <int ISO, bool EN>
+__global__ void __launch_bounds__(128) k_propagate64(LaunchArgs a, uint32_t limit)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    Path64 P;
+    m64::State x;
+    bool active = false, drained = false;
+    uint32_t tick = 0;
+    unsigned long long my_steps = 0;
+    while (true) {
+        const unsigned need = __ballot_sync(0xffffffffu, !active && !drained);
+        if (need) {
+            unsigned long long base = 0;
+            const unsigned leader = __ffs(need) - 1;
+            if (lane == leader) base = atomicAdd(a.cursor, (unsigned long long)__popc(need));
+            base = __shfl_sync(0xffffffffu, base, leader);
+            if (need & (1u << lane)) {
+                const uint64_t q = base + __popc(need & ((1u << lane) - 1u));
+                if (q < a.n_total) {
+                    fresh64(a, q, P, x);
+                    active = true;
+                }
+            }
+            if (base + __popc(need) > a.n_total) drained = true;   // a refused lane never asks again
+        }
+        if (!__any_sync(0xffffffffu, active)) {
+            if (drained) break;
+            continue;
+        }
+        // few enough paths left, all of them taken from the queue: hand them over (asked every 8 steps)
+        if (limit && (++tick & 7u) == 0u) {
+            unsigned few = 0;
+            if (lane == 0)
+                few = a.n_total - *(volatile unsigned long long *)a.ended <= limit &&
+                      *(volatile unsigned long long *)a.cursor >= a.n_total;
+            if (__shfl_sync(0xffffffffu, few, 0)) {
+                if (active) {
+                    store64<EN>(a.out, P, x);
+                    a.list[atomicAdd(a.ended + 1, 1ull)] = (uint32_t)P.g;   // at most `limit` paths are left
+                }
+                break;
+            }
+        }
+        bool end = false;
+        if (active) {
+            double z[3];
+            s64::normals(P.seed, P.pid, x.k, z);
+            step64<1, ISO, EN>(P, nullptr, s64::Team<1>{0}, z, true, x);
+            end = x.status != COSMICA_PATH_RUNNING;
+            if (end) {
+                store64<EN>(a.out, P, x);
+                my_steps += x.k;
+                active = false;
+            }
+        }
+        const unsigned ends = __ballot_sync(0xffffffffu, end);
+        if (limit && ends && lane == 0) atomicAdd(a.ended, (unsigned long long)__popc(ends));
+    }
+    if (a.steps_total) {
+        for (int o = 16; o > 0; o >>= 1) my_steps += __shfl_down_sync(0xffffffffu, my_steps, o);
+        if (lane == 0 && my_steps) atomicAdd(a.steps_total, my_steps);
+    }
+}
+
+// Teams of G lanes; team j of warp w takes entry j * warps + w, so that the schedulers share the
+// paths evenly.  fresh: the queue's paths from their start, else those of the list.
+template <int G, int ISO, bool EN>
+__global__ void __launch_bounds__(128) k_finish64(LaunchArgs a, bool fresh)
+{
+    __shared__ double tab[s64::kFnWords];
+    s64::load_table(tab);
+    __syncthreads();
+    const uint64_t n = fresh ? a.n_total : a.ended[1];
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t warps = gridDim.x * (blockDim.x / 32), warp = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    const s64::Team<G> team{(int)(lane & (G - 1))};
+    unsigned long long my_steps = 0;
+    for (uint64_t first = warp; first < n; first += (uint64_t)warps * (32 / G)) {
+        // a team without a path of its own follows the warp's first one and writes nothing
+        uint64_t i = first + (uint64_t)(lane / G) * warps;
+        bool live = i < n;
+        if (!live) i = first;
+        Path64 P;
+        m64::State x;
+        if (fresh) fresh64(a, i, P, x);
+        else stored64<EN>(a, a.list[i], P, x);
+        double zs[3];          // normals of step (first of the round) + team lane
+        for (uint32_t it = 0; __any_sync(0xffffffffu, live); ++it) {
+            if (it % G == 0) s64::normals(P.seed, P.pid, x.k + (uint32_t)team.l, zs);
+            const int j = (int)(it % G);
+            const double z[3] = {team.get(zs[0], j), team.get(zs[1], j), team.get(zs[2], j)};
+            step64<G, ISO, EN>(P, tab, team, z, live, x);
+            if (live && x.status != COSMICA_PATH_RUNNING) {
+                if (team.l == 0) {
+                    store64<EN>(a.out, P, x);
+                    my_steps += x.k;
+                }
+                live = false;
+            }
+        }
+    }
+    if (a.steps_total && my_steps) atomicAdd(a.steps_total, my_steps);
+}
+
 // ---------------------------------------------------------------- debug --
 __global__ void k_debug_eval64(const DevParams *__restrict__ prm, const DevSpecies *__restrict__ spc,
                                uint32_t n, const double *__restrict__ st, double *__restrict__ out)
@@ -203,14 +433,45 @@ cudaError_t launch_derive(DevParams *prm, uint32_t n, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_propagate_fp64(const LaunchArgs &a, cudaStream_t s)
+template <int ISO, bool EN>
+static cudaError_t launch64(const LaunchArgs &a, int sms, cudaStream_t s)
+{
+    const uint64_t few = (uint64_t)std::min(a.list_cap, fp64_list_entries(sms));
+    const unsigned n_sms = (unsigned)sms;
+    if (a.n_total <= 8ull * n_sms) {
+        // at most two paths per scheduler
+        const unsigned grid = (unsigned)std::min<uint64_t>(n_sms, (a.n_total + 3) / 4);
+        k_finish64<16, ISO, EN><<<grid, 128, 0, s>>>(a, true);
+    } else if (a.n_total <= 32ull * n_sms) {
+        k_finish64<4, ISO, EN><<<n_sms, 128, 0, s>>>(a, true);
+    } else {
+        // the list holds 32-bit indices
+        const uint32_t limit = a.n_total <= 0xFFFFFFFFull ? (uint32_t)few : 0u;
+        // a second warp per scheduler fills the gaps between FP64 instructions, but halves the speed
+        // of a path: taken when the queue keeps both busy for long
+        const unsigned per_sm = a.n_total >= 1024ull * n_sms ? 2 : 1;
+        k_propagate64<ISO, EN><<<n_sms * per_sm, 128, 0, s>>>(a, limit);
+        note_launch();
+        if (!limit) return cudaGetLastError();
+        k_finish64<4, ISO, EN><<<n_sms, 128, 0, s>>>(a, false);
+    }
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, cudaStream_t s)
 {
     if (a.n_total == 0) return cudaSuccess;
     cudaGetLastError();
-    k_propagate_fp64<<<grid_for(a.n_total, 128), 128, 0, s>>>(a.prm, a.spc, a.items, a.prefix, a.n_items,
-                                                             a.n_total, a.out, a.steps_total);
-    note_launch();
-    return cudaGetLastError();
+    if (v.extended) {
+        k_propagate_fp64<<<grid_for(a.n_total, 128), 128, 0, s>>>(a.prm, a.spc, a.items, a.prefix, a.n_items,
+                                                                 a.n_total, a.out, a.steps_total);
+        note_launch();
+        return cudaGetLastError();
+    }
+    if (v.iso && v.aniso) return v.energy ? launch64<2, true>(a, sms, s) : launch64<2, false>(a, sms, s);
+    if (v.iso) return v.energy ? launch64<1, true>(a, sms, s) : launch64<1, false>(a, sms, s);
+    return v.energy ? launch64<0, true>(a, sms, s) : launch64<0, false>(a, sms, s);
 }
 
 cudaError_t launch_debug_eval64(const DevParams *prm, const DevSpecies *spc, uint32_t n, const double *st,

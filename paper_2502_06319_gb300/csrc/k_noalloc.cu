@@ -90,8 +90,7 @@ __global__ void k_noalloc_head(const HeadChunk h)
     for (uint32_t w = i; w < sizeof(DevSpecies) / 4; w += blockDim.x) sd[w] = ss[w];
     if (i == 0) {
         unsigned long long *c = reinterpret_cast<unsigned long long *>(g_noalloc_scratch + kOffCounters);
-        c[0] = 0ull;
-        c[1] = 0ull;
+        for (uint32_t k = 0; k < kLaunchCounters; ++k) c[k] = 0ull;
         reinterpret_cast<uint64_t *>(g_noalloc_scratch + kOffPrefix)[0] = 0ull;
     }
 }
@@ -218,9 +217,11 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
 
     LaunchArgs a{d_prm, d_spc, d_items, d_prefix, n_energies, total,
                  ExitPtrs{out->r, out->th, out->ph, out->lnP, out->s, out->steps, out->status, out->item, out->lw},
-                 d_counters + 1, d_counters, nullptr, d_prefix, d_f32};
+                 d_counters + 1, d_counters, nullptr, d_prefix, d_f32,
+                 // the FP64 path reads no FP32 table: its list of paths takes that region
+                 (uint32_t *)d_f32, (uint32_t)(f32_table_floats(1) * sizeof(float) / sizeof(uint32_t)), d_counters + 2};
     if (params->precision == COSMICA_PREC_FP64) {
-        e = launch_propagate_fp64(a, s);
+        e = launch_propagate_fp64(a, fp64_variant(params, 1), num_sms(), s);
     } else {
         const unsigned block = 128;
         const MixedVariant v{params->precision, params->formulation == 1,
