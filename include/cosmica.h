@@ -378,18 +378,18 @@ typedef struct {
 } cosmica_work_item;
 
 /* Launch shape and scheduling of the persistent kernel.  Passing NULL selects
- * block 128, the most resident blocks, compaction every 64 steps, no graph,
- * most-expensive-first queue order -- except that a launch with fewer than 8
- * particles per resident lane (bound by its slowest paths, which step faster
- * when fewer warps share an SM) takes 4 blocks of 128 per SM.  The same
- * default shapes the launches of cosmica_propagate and
- * cosmica_propagate_orbit. */
+ * block 128, compaction with a look every 64 steps, no graph,
+ * most-expensive-first queue order, and 1 to 4 blocks per SM by the number of
+ * particles (a launch with few of them is bound by its slowest paths, which
+ * step faster when fewer warps share an SM).  The same default shapes the
+ * launches of cosmica_propagate, cosmica_propagate_orbit and
+ * cosmica_propagate_noalloc. */
 typedef struct {
     uint32_t block;           /* threads per block (32..256; 0 = 128)                   */
     uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit)  */
     uint32_t compact_period;  /* once the queue is drained, every this many steps the
-                                 active particles of a block are repacked into its lowest
-                                 warps (0 = never)                                       */
+                                 launch looks whether the particles left fit fewer warps,
+                                 which then take them over (0 = never)                   */
     uint32_t use_graph;       /* 1: replay the launch as a CUDA graph                   */
     uint32_t queue_order;     /* 0: items in the given order; 1: items with the lowest
                                  K0 beta P first (longest paths first); exit records keep

@@ -259,7 +259,7 @@ struct Tables {
     uint32_t *qitem = nullptr;               // item of each queue slot
     uint64_t *qprefix = nullptr;             // prefix sums in queue order
     unsigned long long *counters = nullptr;   // kLaunchCounters of a launch
-    uint32_t *list = nullptr;                 // paths an FP64 launch leaves to its second kernel
+    uint32_t *list = nullptr;                 // paths a kernel of the launch leaves to the next
     uint32_t list_cap = 0;
     uint64_t n_total = 0;
     uint32_t n_items = 0;
@@ -273,8 +273,8 @@ struct Tables {
         const size_t b_pre = align_up((nI + 1) * sizeof(uint64_t), 256);
         const size_t b_q = align_up(std::max<size_t>(1, nI) * sizeof(uint32_t), 256);
         const size_t up = b_items + 2 * b_pre + b_q;
-        list_cap = fp64_list_entries(num_sms());
-        cosmica_status st = dev.reserve(up + 256 + list_cap * sizeof(uint32_t));
+        list_cap = list_entries(pre[nI], num_sms());
+        cosmica_status st = dev.reserve(up + 256 + 2 * (size_t)list_cap * sizeof(uint32_t));
         if (st != COSMICA_OK) return st;
         st = stage.reserve(up);
         if (st != COSMICA_OK) return st;
@@ -359,24 +359,34 @@ int num_sms()
     return n;
 }
 
+// Blocks of 128 (warps per scheduler) of an untuned launch.  More of them raise the rate (4.9, 7.0,
+// 8.0 and 8.3e10 steps/s with 1 to 4 in a long batch), fewer step each path faster (0.36, 0.5, 0.7
+// and 0.9 us a step), and a launch waits for its slowest paths, some ten times the mean.  Measured
+// in paths per lane of one layer (one warp per scheduler), ms with 1 / 2 / 3 / 4 layers:
+// 1.5: 36 / 43 / 49 / 50, 3: 47 / 52 / 58 / 60, 8: 55 / 51 / 55 / 59, 15: 73 / 67 / 71 / 70,
+// 31: 139 / 102 / 96 / 102, 57 (FP64 sums): 1212 / 782 / 666 / 637.
+int untuned_layers(uint64_t n_total, int sms, int max_blocks)
+{
+    const uint64_t layer = (uint64_t)sms * 128u;
+    const int layers = n_total <= 4 * layer ? 1 : n_total <= 20 * layer ? 2 : n_total <= 40 * layer ? 3 : max_blocks;
+    return std::max(1, std::min(layers, max_blocks));
+}
+
 PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_total)
 {
     unsigned block = (t && t->block) ? t->block : 128u;
     const unsigned period = t ? t->compact_period : 64u;
     block = std::min(256u, std::max(32u, block / 32u * 32u));
-    int max_b = mixed_max_blocks_per_sm(v, block, period != 0);
+    int max_b = mixed_max_blocks_per_sm(v, block);
     if (max_b < 1) max_b = 1;
     int bps = (t && t->blocks_per_sm) ? (int)t->blocks_per_sm : max_b;
     if (!t) {
-        // no tuning given: a launch with few particles per resident lane is bound by its slowest
-        // paths, which step faster when fewer warps share an SM (the autotuner picks 16 warps per
-        // SM for 6e5 particles, about 5 per lane, and every resident block from 1.5e6 up)
-        const uint64_t lanes = (uint64_t)num_sms() * (uint64_t)max_b * block;
-        if (n_total < 8ull * lanes) bps = std::max(1, (int)(512u / block));
+        bps = untuned_layers(n_total, num_sms(), max_b);
     }
     bps = std::min(bps, max_b);
     uint64_t grid = (uint64_t)num_sms() * (uint64_t)bps;
-    const uint64_t need = (n_total + block - 1) / block;   // never more blocks than particles
+    // never more warps than paths (the kernel spreads them evenly)
+    const uint64_t need = (n_total + block / 32u - 1) / (block / 32u);
     grid = std::max<uint64_t>(1, std::min(grid, need));
     return PersistentShape{block, (unsigned)grid, period};
 }
@@ -559,7 +569,7 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
     } else {
         const MixedVariant v{m->p.precision, m->p.formulation == 1, m->p.n_shells > 0 || m->p.squashed != 0,
                              full_model(m->p)};
-        e = launch_propagate_mixed(a, v, shape_for(v, nullptr, total), s);
+        e = launch_propagate_mixed(a, v, shape_for(v, nullptr, total), num_sms(), s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
     if (host_out) return ExitStage::copy_back(ex, out, s);
@@ -960,7 +970,7 @@ static cosmica_status batch_launch(cosmica_batch *b, uint64_t total, const ExitP
        "cudaMemsetAsync(counters)");
         cudaError_t e = (b->precision == COSMICA_PREC_FP64)
                             ? launch_propagate_fp64(a, fp64_variant(b->params.data(), b->params.size()), num_sms(), s)
-                            : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total), s);
+                            : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total), num_sms(), s);
         if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
         return COSMICA_OK;
     };
@@ -1205,13 +1215,14 @@ extern "C" cosmica_status cosmica_autotune(cosmica_batch *b, const cosmica_work_
         std::vector<cosmica_tuning> cands;
         for (unsigned blk : blocks) {
             for (unsigned per : periods) {
-                const unsigned maxb = (unsigned)std::max(1, mixed_max_blocks_per_sm(b->variant(), blk, per != 0));
+                const unsigned maxb = (unsigned)std::max(1, mixed_max_blocks_per_sm(b->variant(), blk));
                 // all resident blocks, one fewer, and half: fewer resident warps can win when the
                 // register file or the L1 is the contended resource, or when the tail dominates
                 cands.push_back(cosmica_tuning{blk, maxb, per, 0, 1});
                 if (maxb >= 3) cands.push_back(cosmica_tuning{blk, maxb - 1, per, 0, 1});
                 if (maxb / 2 >= 1 && maxb / 2 != maxb && maxb / 2 != maxb - 1)
                     cands.push_back(cosmica_tuning{blk, maxb / 2, per, 0, 1});
+                if (blk == 128 && maxb > 2) cands.push_back(cosmica_tuning{blk, 1, per, 0, 1});
             }
         }
         for (const cosmica_tuning &t : cands) {

@@ -9,8 +9,8 @@
 // (measured beside Acc<COSMICA_PREC_MIXED_F64ACC> in mixed_state.cuh).
 //
 // Each function gives the bits that the conversion instruction gives (round to nearest
-// even, FP32 subnormals flushed) on the values its *_ok() predicate accepts; the caller
-// converts the rest -- zeros, subnormals, infinities, NaN -- with the instruction.
+// even, FP32 subnormals flushed to zero) on the values it names; none of them branches, so
+// that the step they are part of stays one block.
 #pragma once
 #include <cstdint>
 
@@ -27,45 +27,44 @@ constexpr uint64_t kPiBits = 0x400921FB54442D18ull;      // the double nearest p
 constexpr uint64_t kHalfPiBits = 0x3FF921FB54442D18ull;
 constexpr uint64_t kTwoPiBits = 0x401921FB54442D18ull;
 
-// FP32 -> FP64, exact.  Accepts the normal numbers.
-COSMICA_HD bool widen_ok(uint32_t u) { return (u & 0x7FFFFFFFu) - 0x00800000u < 0x7F000000u; }
+// FP32 -> FP64, exact, for every value (a subnormal one gives zero).
 COSMICA_HD uint64_t widen(uint32_t u)
 {
-    // exponent bias 127 -> 1023: add 896 to the exponent field (bit 20 of the high word)
-    const uint32_t hi = (u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u);
-    return ((uint64_t)hi << 32) | (u << 29);
+    // exponent bias 127 -> 1023: add 896 to the exponent field (bit 20 of the high word), or what
+    // turns 255 into 2047; a zero stays one
+    const uint32_t t = u & 0x7FFFFFFFu;
+    const uint32_t bias = t >= 0x7F800000u ? 0x70000000u : 0x38000000u;
+    const bool none = t < 0x00800000u;
+    const uint32_t hi = (u & 0x80000000u) | (none ? 0u : (t >> 3) + bias);
+    return ((uint64_t)hi << 32) | (none ? 0u : u << 29);
 }
 
-// FP64 -> FP32, round to nearest even.  Accepts 2^-125 <= |x| < 2^127 (no result is
-// subnormal and none overflows); hi = the high word.
-COSMICA_HD bool narrow_ok(uint32_t hi) { return (hi & 0x7FFFFFFFu) - 0x38200000u < 0x0FC00000u; }
+// FP64 -> FP32, round to nearest even, for finite |x| < 2^127 (below 2^-126: zero).
 COSMICA_HD uint32_t narrow(uint64_t x)
 {
     const uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
-    const uint32_t e = (hi & 0x7FFFFFFFu) - 0x38000000u;
-    const uint32_t t = (e << 3) | (lo >> 29);            // truncated result without its sign
+    const uint32_t m = hi & 0x7FFFFFFFu;
+    const uint32_t t = ((m - 0x38000000u) << 3) | (lo >> 29);            // truncated result without its sign
     // the 29 bits below it as a fraction of 2^32: adding 2^31 - 1 + lsb carries exactly when
     // the fraction is above one half, or equal to it with an odd t
     const uint64_t r = (((uint64_t)t << 32) | (uint32_t)(lo << 3)) + (0x7FFFFFFFu + (t & 1u));
-    return (uint32_t)(r >> 32) | (hi & 0x80000000u);
+    return (m < 0x38100000u ? 0u : (uint32_t)(r >> 32)) | (hi & 0x80000000u);
 }
 
 // pi - th as FP32 (the FP64 difference rounded to nearest even), th in [pi/2, pi]: both lie
 // within a factor of two, so the FP64 difference is exact (Sterbenz) and is formed as an
-// integer multiple of 2^-52.  Accepts differences of at least 2^-20; diff = pi_minus_units(th).
+// integer multiple of 2^-52.
 COSMICA_HD uint64_t pi_minus_units(uint64_t th)
 {
     const uint64_t m = (th & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
     return 0x003243F6A8885A30ull - (m << ((uint32_t)(th >> 52) & 1u ? 0 : 1));
 }
-COSMICA_HD bool pi_minus_ok(uint64_t diff) { return (uint32_t)(diff >> 32) != 0u; }
 COSMICA_HD float pi_minus(uint64_t diff)
 {
-    const uint32_t hi = (uint32_t)(diff >> 32);
 #if defined(__CUDA_ARCH__)
-    const int sh = __clz(hi);
+    const int sh = __clzll((long long)(diff | 1u));
 #else
-    const int sh = __builtin_clz(hi | 1u);
+    const int sh = __builtin_clzll(diff | 1u);
 #endif
     const uint64_t n = diff << sh;
     // 32 leading bits, the rest folded into a sticky bit below the rounding position

@@ -121,6 +121,7 @@ inline DevItem make_item(double T, uint64_t first_pid, uint64_t seed, uint32_t p
     return it;
 }
 int num_sms();
+int untuned_layers(uint64_t n_total, int sms, int max_blocks);
 
 }  // namespace host
 }  // namespace cosmica

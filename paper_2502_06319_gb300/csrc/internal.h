@@ -14,7 +14,7 @@ constexpr int kDebugEvalN = 21;   // quantities written per state by the debug e
 struct LaunchArgs {
     const DevParams *prm;
     const DevSpecies *spc;
-    const DevItem *items;
+    DevItem *items;
     const uint64_t *prefix;
     uint32_t n_items;
     uint64_t n_total;
@@ -24,18 +24,30 @@ struct LaunchArgs {
     const uint32_t *qitem;             // item of each queue slot (null: item order)
     const uint64_t *qprefix;           // prefix sums of particle counts in queue order
     const float *f32;                  // FP32 blocks of the parameter sets, paged field-major (P32)
-    // FP64 path: indices of the paths left to the team kernel, room for list_cap of them, and two
-    // counters (paths ended, paths left); cleared like the cursor
+    // indices of the paths one kernel of the launch leaves to the next: two lists of list_cap
+    // (mixed paths use both in turn, the FP64 path the first), and counters cleared like the cursor
     uint32_t *list;
     uint32_t list_cap;
-    unsigned long long *ended;         // [0] ended, [1] left
+    unsigned long long *ended;         // [0] paths ended; then, per kernel, paths left and their cursor
 };
 
 struct PersistentShape {
     unsigned block;
     unsigned grid;
-    unsigned compact_period;   // 0: no block compaction
+    unsigned compact_period;   // steps between looks at the paths left; 0: never handed over
 };
+
+// one kernel of a mixed launch: where its paths come from and where it leaves the last ones
+struct MixedStage {
+    const uint32_t *from;              // null: the launch's queue, else parked paths, *n_from of them
+    const unsigned long long *n_from;
+    unsigned long long *cursor;        // of the source
+    uint32_t *to;
+    unsigned long long *n_to;
+    uint32_t limit;                    // leave the last `limit` paths (0: none)
+    uint32_t period;
+};
+constexpr uint32_t kMixedStages = 4;   // most warps per scheduler that hand over step by step
 
 // ---- continuous-batching server -------------------------------------------
 // fresh particles of one (request, energy) slice, offered to one quantum
@@ -88,8 +100,14 @@ cudaError_t launch_f32_table(const DevParams *prm, uint32_t n, float *table, cud
 struct Fp64Variant {
     bool energy, extended, iso, aniso;   // iso / aniso: some set is (not) isotropic
 };
-// counters of a launch: queue cursor, steps, paths ended, paths left to the team kernel
-constexpr uint32_t kLaunchCounters = 4;
+// counters of a launch: queue cursor, steps, paths ended, and per kernel paths left and their cursor
+constexpr uint32_t kLaunchCounters = 3 + 2 * kMixedStages;
+// entries of each of a launch's two lists: at most kMixedStages - 1 warps per scheduler
+inline uint32_t list_entries(uint64_t n_total, int sms)
+{
+    const uint64_t most = (uint64_t)(kMixedStages - 1) * 128u * (uint64_t)sms;
+    return n_total > 32ull * (uint64_t)sms ? (uint32_t)(n_total < most ? n_total : most) : 0u;
+}
 // most paths the team kernel takes over (32 per SM: eight teams of four lanes on every scheduler)
 inline uint32_t fp64_list_entries(int sms) { return 32u * (uint32_t)sms; }
 cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, cudaStream_t s);
@@ -116,8 +134,8 @@ inline bool full_model(const cosmica_params &p)
 {
     return !p.isotropic && p.drift_on && p.hcs_on && !(p.dt_fixed_day > 0.0);
 }
-cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, cudaStream_t s);
-int mixed_max_blocks_per_sm(MixedVariant v, unsigned block, bool compact);
+cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, int sms, cudaStream_t s);
+int mixed_max_blocks_per_sm(MixedVariant v, unsigned block);
 
 struct SpecItem {
     double T;                  // GeV/n

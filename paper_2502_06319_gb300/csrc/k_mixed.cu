@@ -7,9 +7,12 @@
 // exits writes the exit state and immediately takes the next particle from
 // the queue (refill), so that warps stay full while the queue lasts despite
 // the long tail of exit times.  Lanes needing work in the same step take
-// consecutive particles with one atomic per warp.  The paper's thread-per-
+// consecutive particles with one atomic per warp.  When the queue is empty and
+// the paths left fit a smaller grid, they are handed to another launch of the
+// kernel with one warp per scheduler fewer.  The paper's thread-per-
 // quasi-particle mapping (Sec. IV.A) is kept; its one-launch-per-energy-bin
-// loop (Sec. IV.A, last paragraph) becomes this single launch.
+// loop (Sec. IV.A, last paragraph) becomes this.
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -22,14 +25,24 @@ namespace cosmica {
 
 namespace {
 
-template <int ACC, bool EN>
-__device__ __forceinline__ void start_particle(const LaunchArgs &a, uint64_t q, Lane &L, Acc<ACC> &x,
-                                               EnergyAcc<ACC, EN> &en)
+// ln P0 of every item in place of its T (momentum form; the energy form starts from T): a
+// lane taking a path would otherwise spend some 60 slots of the FP64 pipe on it, 64 clocks each
+// for its whole warp.
+__global__ void k_start_lnP(DevItem *items, const DevSpecies *__restrict__ spc, uint32_t n)
 {
-    // queue slot q -> (item, index within the item); the exit record keeps item order
-    const uint32_t iq = find_item(a.qprefix, a.n_items, q);
-    const uint32_t it = a.qitem ? a.qitem[iq] : iq;
-    const uint64_t local = q - a.qprefix[iq];
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const DevSpecies &sp = spc[items[i].species_idx];
+    const double T = items[i].T;
+    const double P0 = sp.A / fabs(sp.Z) * sqrt(T * (T + 2.0 * sp.m0));
+    items[i].T = log(P0);
+}
+
+// the particle `local` of item `it`, at its start
+template <int ACC, bool EN>
+__device__ __forceinline__ void begin(const LaunchArgs &a, uint32_t it, uint64_t local, Lane &L, Acc<ACC> &x,
+                                      EnergyAcc<ACC, EN> &en)
+{
     const DevItem item = a.items[it];
     const DevParams &p = a.prm[item.param_idx];
     const DevSpecies &sp = a.spc[item.species_idx];
@@ -42,21 +55,39 @@ __device__ __forceinline__ void start_particle(const LaunchArgs &a, uint64_t q, 
     L.item = item.out_item;
     L.k = 0;
     L.max_steps = (uint32_t)p.max_steps;
-    const double T = item.T;
-    const double P0 = sp.A / fabs(sp.Z) * sqrt(T * (T + 2.0 * sp.m0));
-    x.init(item.r0, item.th0, item.ph0, log(P0), p.R_out, p.f.r_in);
-    en.init(T, (float)sp.m0, sp.aoz);
+    // item.T: T of the energy form (whose ln P follows from T), ln P0 of the momentum form
+    x.init(item.r0, item.th0, item.ph0, EN ? 1.0 : item.T, p.R_out, p.f.r_in);
+    if constexpr (EN) en.init(item.T, (float)sp.m0, sp.aoz);
 }
 
-// One Euler-Maruyama step (Eq. 3, Eq. 6) of an active lane, with the normals z0, z1, z2
-// of step L.k (drawn before); true when the path ended (exit record written), else the
-// normals of the next step are left in z0, z1, z2.
+// Entry q of the launch's source: a queue slot (fresh), or a path parked by the launch before.
+template <int ACC, bool EN>
+__device__ __forceinline__ void take(const LaunchArgs &a, const MixedStage &st, uint64_t q, Lane &L, Acc<ACC> &x,
+                                     EnergyAcc<ACC, EN> &en)
+{
+    if (!st.from) {
+        // queue slot -> (item, index within the item); the exit record keeps item order
+        const uint32_t iq = find_item(a.qprefix, a.n_items, q);
+        begin<ACC, EN>(a, a.qitem ? a.qitem[iq] : iq, q - a.qprefix[iq], L, x, en);
+    } else {
+        const uint64_t g = st.from[q];
+        const uint32_t it = find_item(a.prefix, a.n_items, g);
+        begin<ACC, EN>(a, it, g - a.prefix[it], L, x, en);
+        unpark<EN>(a.out, g, x, en);
+        L.k = a.out.steps[g];
+    }
+}
+
+// One Euler-Maruyama step (Eq. 3, Eq. 6) with the normals z0, z1, z2 of step L.k, which become
+// those of the next step: the increments are added and nothing else is looked at.  One block
+// without branches (in the full-model variant), so that the compiler interleaves the
+// generator with the coefficients.
 template <int ACC, bool EN, bool EXT, bool FULL>
-__device__ __forceinline__ bool step(const LaunchArgs &a, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en,
-                                     unsigned long long &my_steps, float &z0, float &z1, float &z2)
+__device__ __forceinline__ void advance(const float *params, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en, float &z0,
+                                        float &z1, float &z2)
 {
     m32::Drift c;
-    const P32<kSetsPerPage> q{L.q};
+    const P32<kSetsPerPage> q{params};
     float fr, fth, fph, lnP, sin_th;
     x.view(fr, fth, fph, lnP, sin_th);
     if constexpr (EN) {
@@ -78,21 +109,33 @@ __device__ __forceinline__ bool step(const LaunchArgs &a, Lane &L, Acc<ACC> &x, 
     } else {
         x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
     }
-    x.boundaries(P32F(q, r_in));
     L.k += 1u;
+    m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
+}
 
+// whether the state after a step needs settle(): a boundary other than the longitude's, an end of
+// the path, or nearly so
+template <int ACC, bool EXT>
+__device__ __forceinline__ bool needs_settling(const float *params, const Lane &L, const Acc<ACC> &x)
+{
+    const P32<kSetsPerPage> q{params};
+    const bool squashed = EXT && P32F(q, sq) != 0.0f;
+    bool calm = x.calm(P32F(q, r_in), !squashed) & (L.k < L.max_steps);
+    if (squashed) calm = calm && !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
+    return !calm;
+}
+
+// Boundaries and the three ends of a path; true when the path ended (exit record written).
+template <int ACC, bool EN, bool EXT>
+__device__ __forceinline__ bool settle(const LaunchArgs &a, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en,
+                                       unsigned long long &my_steps)
+{
+    const P32<kSetsPerPage> q{L.q};
+    x.boundaries(P32F(q, r_in));
     const bool fin = x.finite();
     const bool out = (EXT && P32F(q, sq) != 0.0f) ? m32::outside_squashed(q, x.fr(), x.fth(), x.fph()) : x.exited();
     const bool lim = L.k >= L.max_steps;
-    if (fin & !out & !lim) {     // one rarely taken branch for the three ends of a path
-        // the next step's normals, drawn after this step's arithmetic: the Philox block and
-        // the eval of the coefficients are then never live at the same time (64 instead of
-        // 74 registers in the variant without compaction: 32 resident warps per SM instead
-        // of 24, +2.6 % steps/s on config 3; a lone path's step takes 12 % longer, as the
-        // block no longer hides under the eval's latency)
-        m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
-        return false;
-    }
+    if (fin & !out & !lim) return false;
     const int status = !fin ? COSMICA_PATH_NONFINITE : (out ? COSMICA_PATH_EXIT : COSMICA_PATH_STEP_LIMIT);
     x.write(a.out, L.g);
     if constexpr (EN) {
@@ -109,111 +152,93 @@ __device__ __forceinline__ bool step(const LaunchArgs &a, Lane &L, Acc<ACC> &x, 
     return true;
 }
 
-// Persistent propagation.
-// Phase 1: lanes take particles from the device queue (one atomic per warp for all
-// lanes needing work), step them, write the exit record and refill, until the queue
-// is drained.  Phase 2 (COMPACT): every `period` steps the block meets at a
-// checkpoint; the active particles are counted and, if they occupy more warps than
-// they need, repacked through shared memory into the block's lowest lanes, so that
-// issued warp instructions keep carrying full lanes while the long tail of exit
-// times plays out.  Both phases share one step site (one copy of the step code).
-template <int ACC, bool COMPACT, bool EN, bool EXT, bool FULL>
-__global__ void __launch_bounds__(256) k_propagate_mixed(LaunchArgs a, uint32_t period)
+// Persistent propagation.  Lanes take paths from the source (one atomic per warp for all lanes
+// needing work), step them, write the exit record and refill, until the source is drained.
+// Then, if the launch has a limit, every warp asks every `period` steps how many paths are
+// left, and once they are no more than the limit parks its own for the next launch.
+//
+// The steps run in an inner loop that ends when some lane of the warp has a boundary or an end
+// to see to: one vote and one branch a step.  All lanes of the warp run it, those without a
+// path on whatever they hold (nobody looks at the results).  What bounds it: a warp alone on its
+// scheduler is bound by its ~400 instructions a step and their dependences, four warps by the
+// issue rate.  The loop being one block, the compiler interleaves the generator with the
+// coefficients and keeps the parameter set in registers (114-123 instead of 64, so 16 warps
+// per SM instead of 32).  Measured, against a loop that tested everything every step and drew the
+// normals after the tests: a lone path's step 0.68 -> 0.36 us, a warp's step with four warps per
+// scheduler 1.05 -> 0.93 us, 5.7e6 paths of 4 heliospheres 8.3e10 steps/s, one spectrum of 6e5
+// paths 141 -> 99 ms, 1.8e6 paths of 16 heliospheres 870 -> 694 ms.
+template <int ACC, bool EN, bool EXT, bool FULL>
+__global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedStage st)
 {
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned s_count;
-    __shared__ unsigned s_warp[8];
     const unsigned lane = threadIdx.x & 31u;
-    const unsigned warp = threadIdx.x >> 5;
-    Lane L;
-    Acc<ACC> x;
-    EnergyAcc<ACC, EN> en;
-    bool active = false, drained = false, phase2 = false;
+    Lane L{};
+    Acc<ACC> x{};
+    EnergyAcc<ACC, EN> en{};
+    // lanes that never get a path step an unremarkable state of the first set
+    L.q = a.f32;
+    x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f);
+    en.init(1.0, 1.0f, 1.0f);
+    // a source smaller than the grid is spread evenly over the warps
+    const uint64_t n = st.from ? *st.n_from : a.n_total;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    const bool seat = lane < (n + warps - 1) / warps;
+    bool active = false, drained = n == 0;
     float z0 = 0.0f, z1 = 0.0f, z2 = 0.0f;   // normals of the lane's next step
     unsigned long long my_steps = 0;
-    uint32_t tick = 0;   // phase 1: steps since the last drained check; phase 2: steps since the checkpoint
+    uint32_t room = st.limit ? st.period : 0xFFFFFFFFu;   // steps until the next look at the paths left
 
     while (true) {
-        if (!COMPACT && drained) {
-            // the queue is exhausted (warp-uniform): finish the particles in hand
-            if (!__any_sync(0xffffffffu, active)) break;
-        } else if (!phase2) {
-            const unsigned need = __ballot_sync(0xffffffffu, !active && !drained);
-            if (need) {
-                unsigned long long base = 0;
-                const unsigned leader = __ffs(need) - 1;
-                if (lane == leader) base = atomicAdd(a.cursor, (unsigned long long)__popc(need));
-                base = __shfl_sync(0xffffffffu, base, leader);
-                if (need & (1u << lane)) {
-                    const uint64_t q = base + __popc(need & ((1u << lane) - 1u));
-                    if (q < a.n_total) {
-                        start_particle<ACC, EN>(a, q, L, x, en);
-                        m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
-                        active = true;
-                    } else {
-                        drained = true;
-                    }
+        const unsigned need = __ballot_sync(0xffffffffu, seat && !active && !drained);
+        if (need) {
+            unsigned long long base = 0;
+            const unsigned leader = __ffs(need) - 1;
+            if (lane == leader) base = atomicAdd(st.cursor, (unsigned long long)__popc(need));
+            base = __shfl_sync(0xffffffffu, base, leader);
+            if (need & (1u << lane)) {
+                const uint64_t q = base + __popc(need & ((1u << lane) - 1u));
+                if (q < n) {
+                    take<ACC, EN>(a, st, q, L, x, en);
+                    m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
+                    active = true;
                 }
-                // without compaction a lane that was refused never asks again, so once any lane
-                // of the warp is refused the whole warp can stop asking
-                if (!COMPACT && base + __popc(need) > a.n_total) drained = true;
             }
-            if (COMPACT) {
-                // learn of the drained queue even when no lane of the warp needed work
-                if (++tick >= period) {
-                    tick = 0;
-                    unsigned dq = 0;
-                    if (lane == 0) dq = *(volatile unsigned long long *)a.cursor >= a.n_total;
-                    if (__shfl_sync(0xffffffffu, dq, 0)) drained = true;
+            // a lane that was refused never asks again, so once any lane of the warp is refused the
+            // whole warp can stop asking
+            if (base + __popc(need) > n) drained = true;
+        }
+        if (!__any_sync(0xffffffffu, active)) {
+            if (drained) break;
+            continue;
+        }
+        if (room == 0) {
+            room = st.period;
+            // few enough paths left, all of them taken from the source (drained: a lane was refused)
+            unsigned few = 0;
+            if (drained && lane == 0) few = a.n_total - *(volatile unsigned long long *)a.ended <= st.limit;
+            if (__shfl_sync(0xffffffffu, few, 0)) {
+                if (active) {
+                    park<EN>(a.out, L.g, x, en);
+                    a.out.steps[L.g] = L.k;
+                    a.out.status[L.g] = COSMICA_PATH_RUNNING;
+                    st.to[atomicAdd(st.n_to, 1ull)] = (uint32_t)L.g;   // no more than `limit` paths are left
                 }
-                if (__all_sync(0xffffffffu, drained || active) && __any_sync(0xffffffffu, drained)) {
-                    drained = true;
-                    phase2 = true;
-                    tick = 0;
-                }
+                break;
             }
         }
-        if (COMPACT && phase2) {
-            if (tick == 0) {
-                // checkpoint: every warp of the block arrives here once per epoch
-                if (threadIdx.x == 0) s_count = 0;
-                __syncthreads();
-                const unsigned bal = __ballot_sync(0xffffffffu, active);
-                if (lane == 0) {
-                    s_warp[warp] = __popc(bal);
-                    atomicAdd(&s_count, (unsigned)__popc(bal));
-                }
-                __syncthreads();
-                const unsigned n = s_count;
-                if (n == 0) break;
-                unsigned occupied = 0, before = 0;
-                for (unsigned w = 0; w < (blockDim.x >> 5); ++w) {
-                    occupied += s_warp[w] > 0;
-                    if (w < warp) before += s_warp[w];
-                }
-                if (occupied > (n + 31) / 32) {
-                    Packed<ACC, EN> *pack = reinterpret_cast<Packed<ACC, EN> *>(smem_raw);
-                    if (active) {
-                        const unsigned rank = before + __popc(bal & ((1u << lane) - 1u));
-                        pack[rank].L = L;
-                        pack[rank].x = x;
-                        pack[rank].en = en;
-                    }
-                    __syncthreads();
-                    active = threadIdx.x < n;
-                    if (active) {
-                        L = pack[threadIdx.x].L;
-                        x = pack[threadIdx.x].x;
-                        en = pack[threadIdx.x].en;
-                        m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
-                    }
-                }
-                __syncthreads();
-            }
-            // an idle warp goes straight to the next checkpoint
-            tick = __any_sync(0xffffffffu, active) ? (tick + 1 == period ? 0 : tick + 1) : 0;
+        bool see;
+        while (true) {
+            advance<ACC, EN, EXT, FULL>(L.q, L, x, en, z0, z1, z2);
+            see = active && needs_settling<ACC, EXT>(L.q, L, x);
+            const bool wrap = active && x.phi_out();
+            --room;
+            if (!__any_sync(0xffffffffu, see || wrap || room == 0)) continue;
+            if (wrap && !see) x.wrap_near();
+            if (__any_sync(0xffffffffu, see || room == 0)) break;
         }
-        if (active && step<ACC, EN, EXT, FULL>(a, L, x, en, my_steps, z0, z1, z2)) active = false;
+        const bool end = see && settle<ACC, EN, EXT>(a, L, x, en, my_steps);
+        if (end) active = false;
+        const unsigned ends = __ballot_sync(0xffffffffu, end);
+        if (ends && lane == 0) atomicAdd(a.ended, (unsigned long long)__popc(ends));
     }
     if (a.steps_total) {
         for (int o = 16; o > 0; o >>= 1) my_steps += __shfl_down_sync(0xffffffffu, my_steps, o);
@@ -237,59 +262,75 @@ __global__ void k_debug_eval32(const DevParams *__restrict__ prm, const DevSpeci
 
 }  // namespace
 
-template <int ACC, bool EN>
-static size_t pack_bytes(unsigned block) { return (size_t)block * sizeof(Packed<ACC, EN>); }
-
-// Call fn(acc, compact, energy, extended, full) with each flag as a compile-time constant.
+// Call fn(acc, energy, extended, full) with each flag as a compile-time constant.
 template <class Fn>
-static void visit_variant(MixedVariant v, bool compact, Fn &&fn)
+static void visit_variant(MixedVariant v, Fn &&fn)
 {
     auto on_acc = [&](auto A) {
-        auto on_compact = [&](auto C) {
-            auto on_energy = [&](auto E) {
-                auto on_ext = [&](auto X) {
-                    if (v.full) fn(A, C, E, X, std::true_type{});
-                    else fn(A, C, E, X, std::false_type{});
-                };
-                if (v.extended) on_ext(std::true_type{});
-                else on_ext(std::false_type{});
+        auto on_energy = [&](auto E) {
+            auto on_ext = [&](auto X) {
+                if (v.full) fn(A, E, X, std::true_type{});
+                else fn(A, E, X, std::false_type{});
             };
-            if (v.energy) on_energy(std::true_type{});
-            else on_energy(std::false_type{});
+            if (v.extended) on_ext(std::true_type{});
+            else on_ext(std::false_type{});
         };
-        if (compact) on_compact(std::true_type{});
-        else on_compact(std::false_type{});
+        if (v.energy) on_energy(std::true_type{});
+        else on_energy(std::false_type{});
     };
     if (v.acc == COSMICA_PREC_MIXED_F64ACC) on_acc(std::integral_constant<int, COSMICA_PREC_MIXED_F64ACC>{});
     else on_acc(std::integral_constant<int, COSMICA_PREC_MIXED>{});
 }
 
-int mixed_max_blocks_per_sm(MixedVariant v, unsigned block, bool compact)
+int mixed_max_blocks_per_sm(MixedVariant v, unsigned block)
 {
     int nb = 0;
-    visit_variant(v, compact, [&](auto A, auto C, auto E, auto S, auto F) {
-        constexpr int acc = decltype(A)::value;
-        constexpr bool c = decltype(C)::value, en = decltype(E)::value, sh = decltype(S)::value;
-        constexpr bool fu = decltype(F)::value;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_propagate_mixed<acc, c, en, sh, fu>, (int)block,
-                                                      c ? pack_bytes<acc, en>(block) : 0);
+    visit_variant(v, [&](auto A, auto E, auto S, auto F) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &nb, k_propagate_mixed<decltype(A)::value, decltype(E)::value, decltype(S)::value, decltype(F)::value>,
+            (int)block, 0);
     });
     return nb;
 }
 
-cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, cudaStream_t s)
+// A launch of w warps per scheduler whose queue is empty runs on with ever emptier warps, each
+// step as slow as the w warps make it; handing the last paths to w - 1 full warps per scheduler,
+// and so on down to one, steps them at the speed of those (one warp: 0.36 us a step, four: 0.9).
+cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, int sms, cudaStream_t s)
 {
     if (a.n_total == 0) return cudaSuccess;
     cudaGetLastError();
-    const uint32_t per = shape.compact_period;
-    visit_variant(v, per != 0, [&](auto A, auto C, auto E, auto S, auto F) {
-        constexpr int acc = decltype(A)::value;
-        constexpr bool c = decltype(C)::value, en = decltype(E)::value, sh = decltype(S)::value;
-        constexpr bool fu = decltype(F)::value;
-        k_propagate_mixed<acc, c, en, sh, fu><<<shape.grid, shape.block, c ? pack_bytes<acc, en>(shape.block) : 0, s>>>(
-            a, c ? per : 1u);
-    });
-    note_launch();
+    if (!v.energy) {
+        k_start_lnP<<<(a.n_items + 63) / 64, 64, 0, s>>>(a.items, a.spc, a.n_items);
+        note_launch();
+    }
+    const unsigned block = 128;                          // of the later launches
+    const uint64_t layer = (uint64_t)sms * block;        // one warp per scheduler
+    // layers of the next launch: fewer than this one has, and no more than the list holds paths for
+    uint64_t layers = 0;
+    if (shape.compact_period && a.n_total <= 0xFFFFFFFFull && a.list_cap > 0 && a.n_total > layer) {
+        layers = std::min<uint64_t>(((uint64_t)shape.grid * shape.block + layer - 1) / layer, kMixedStages) - 1;
+        layers = std::min<uint64_t>(layers, std::max<uint64_t>(1, a.list_cap / layer));
+    }
+    MixedStage st{};
+    st.cursor = a.cursor;
+    st.period = shape.compact_period ? shape.compact_period : 64u;
+    for (unsigned stage = 0;; ++stage) {
+        st.limit = (uint32_t)std::min<uint64_t>(layers * layer, a.list_cap);
+        st.to = a.list + (stage & 1u) * (size_t)a.list_cap;
+        st.n_to = a.ended + 1 + 2 * stage;
+        visit_variant(v, [&](auto A, auto E, auto S, auto F) {
+            k_propagate_mixed<decltype(A)::value, decltype(E)::value, decltype(S)::value, decltype(F)::value>
+                <<<shape.grid, stage ? block : shape.block, 0, s>>>(a, st);
+        });
+        note_launch();
+        if (layers == 0) break;
+        shape.grid = (unsigned)(layers * sms);
+        st.from = st.to;
+        st.n_from = st.n_to;
+        st.cursor = st.n_to + 1;
+        --layers;
+    }
     return cudaGetLastError();
 }
 

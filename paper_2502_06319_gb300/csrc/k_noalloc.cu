@@ -61,7 +61,7 @@ constexpr size_t kOffCounters = kOffPrefix + ((kMaxE + 1) * sizeof(uint64_t) + 2
 constexpr size_t kOffF32 = kOffCounters + 256;          // one page of the FP32 parameter table
 constexpr size_t kScratchBytes = kOffF32 + (f32_table_floats(1) * sizeof(float) + 255) / 256 * 256;
 static_assert(kScratchBytes <= 96 * 1024, "the documented size of the static scratch is about 95 KB");
-static_assert(sizeof(DevSpecies) <= 256, "species region");
+static_assert(sizeof(DevSpecies) <= 256 && kLaunchCounters * 8 <= 256, "species and counter regions");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -215,21 +215,27 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
     if (e == cudaSuccess) e = launch_f32_table(d_prm, 1, d_f32, s);
     if (e != cudaSuccess) return cuda_fail(e, "cosmica_propagate_noalloc set-up");
 
+    // paths handed from kernel to kernel: the FP64 path reads no FP32 table and takes that region for
+    // its list, the mixed paths put theirs behind the call's items
+    uint32_t *list = (uint32_t *)d_f32;
+    uint32_t list_cap = (uint32_t)(f32_table_floats(1) * sizeof(float) / sizeof(uint32_t));
+    if (params->precision != COSMICA_PREC_FP64) {
+        list = (uint32_t *)(d_items + n_energies);
+        list_cap = (uint32_t)((kMaxE - n_energies) * sizeof(DevItem) / sizeof(uint32_t) / 2);
+    }
     LaunchArgs a{d_prm, d_spc, d_items, d_prefix, n_energies, total,
                  ExitPtrs{out->r, out->th, out->ph, out->lnP, out->s, out->steps, out->status, out->item, out->lw},
                  d_counters + 1, d_counters, nullptr, d_prefix, d_f32,
-                 // the FP64 path reads no FP32 table: its list of paths takes that region
-                 (uint32_t *)d_f32, (uint32_t)(f32_table_floats(1) * sizeof(float) / sizeof(uint32_t)), d_counters + 2};
+                 list, list_cap, d_counters + 2};
     if (params->precision == COSMICA_PREC_FP64) {
         e = launch_propagate_fp64(a, fp64_variant(params, 1), num_sms(), s);
     } else {
         const unsigned block = 128;
         const MixedVariant v{params->precision, params->formulation == 1,
                              params->n_shells > 0 || params->squashed != 0, full_model(*params)};
-        const int bps = std::max(1, mixed_max_blocks_per_sm(v, block, true));
-        uint64_t grid = (uint64_t)num_sms() * (uint64_t)bps;
-        grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + block - 1) / block));
-        e = launch_propagate_mixed(a, v, PersistentShape{block, (unsigned)grid, 64u}, s);
+        const int bps = untuned_layers(total, num_sms(), mixed_max_blocks_per_sm(v, block));
+        const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms() * (uint64_t)bps, (total + 3) / 4);
+        e = launch_propagate_mixed(a, v, PersistentShape{block, (unsigned)grid, 64u}, num_sms(), s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cosmica_propagate_noalloc launch");
     return COSMICA_OK;

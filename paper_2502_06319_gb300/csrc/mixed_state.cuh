@@ -9,6 +9,14 @@
 
 namespace cosmica {
 
+// FP64 <-> FP32 on the bits (f64bits.h)
+__device__ __forceinline__ uint64_t bits64(double x) { return (uint64_t)__double_as_longlong(x); }
+__device__ __forceinline__ double widen64(float d)
+{
+    return __longlong_as_double((long long)f64bits::widen(__float_as_uint(d)));
+}
+__device__ __forceinline__ float narrow64(double x) { return __uint_as_float(f64bits::narrow(bits64(x))); }
+
 struct Lane {
     const float *q;            // field 0 of the particle's FP32 parameter block (see P32)
     float M2, sq;
@@ -57,10 +65,9 @@ struct Acc<COSMICA_PREC_MIXED> {
     template <bool P>
     __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
     {
-        m32::ff_add(r, dr);
-        m32::ff_add(th, dth);
-        m32::ff_add(ph, dph);
-        if (P) m32::ff_add(lnP, dlnP);
+        m32::ff_add2(r, th, dr, dth);
+        if (P) m32::ff_add2(ph, lnP, dph, dlnP);
+        else m32::ff_add(ph, dph);
         m32::ff_add(s, dt);
     }
     // reflect at r_in, fold theta at the poles, wrap phi; all rare branches
@@ -94,6 +101,27 @@ struct Acc<COSMICA_PREC_MIXED> {
         const double p0 = m32::ff_to_double(ph);
         ph = m32::ff_from_double(p0 - kTwoPi * floor(p0 / kTwoPi));
     }
+    // no boundary but the longitude's, no end and no non-finite value is anywhere near: false
+    // for every state that the rest of boundaries(), exited() or finite() would act on, and for
+    // a few others
+    // (sphere: the outer boundary is r = R_out; a squashed one is tested by its own function)
+    __device__ bool calm(float r_in, bool sphere) const
+    {
+        return (r.hi >= r_in) & (!sphere | (r.hi < Rout.hi)) & (__float_as_uint(th.hi) < __float_as_uint(m32::kPiF)) &
+               (ph.hi > -6.28f) & (ph.hi < 12.56f) & isfinite(lnP.hi + s.hi);
+    }
+    bool __device__ phi_out() const { return !(__float_as_uint(ph.hi) < __float_as_uint(m32::kTwoPiF)); }
+    // wrap_phi() for -6.28 < ph < 12.56, where floor(ph / 2 pi) is -1, 0 or 1.  Paths start at one
+    // longitude, often 0, and cross it again and again at first (one step in ten of a warp over
+    // the paths' lives), so only the three FP64 sums of the definition are left.
+    __device__ void wrap_near()
+    {
+        const double p0 = widen64(ph.hi) + widen64(ph.lo);
+        const double turn = ph.hi < 0.0f ? kTwoPi : (f64bits::less(bits64(p0), f64bits::kTwoPiBits) ? 0.0 : -kTwoPi);
+        const double p = p0 + turn;
+        ph.hi = narrow64(p);
+        ph.lo = narrow64(p - widen64(ph.hi));
+    }
     __device__ bool exited() const { return m32::ff_ge(r, Rout); }
     __device__ bool finite() const { return isfinite(r.hi + th.hi + ph.hi + lnP.hi + s.hi); }
     __device__ void write(const ExitPtrs &out, uint64_t g) const
@@ -106,24 +134,10 @@ struct Acc<COSMICA_PREC_MIXED> {
     }
 };
 
-// FP64 <-> FP32 for the FP64-accumulated state: integer forms (f64bits.h) with the
-// conversion instruction left for the rare values those do not take.
-__device__ __forceinline__ uint64_t bits64(double x) { return (uint64_t)__double_as_longlong(x); }
-__device__ __forceinline__ double widen64(float d)
-{
-    return __longlong_as_double((long long)f64bits::widen(__float_as_uint(d)));
-}
-__device__ __forceinline__ bool widen64_ok(float d) { return f64bits::widen_ok(__float_as_uint(d)); }
-__device__ __forceinline__ float narrow64(double x)
-{
-    return f64bits::narrow_ok((uint32_t)__double2hiint(x)) ? __uint_as_float(f64bits::narrow(bits64(x))) : (float)x;
-}
-
 // FP64 accumulation of FP32 increments.
-// Bound by the FP64 pipe (64 clocks per warp instruction and scheduler): only the sums stay on
-// it; conversions, comparisons and the finiteness test run on the bits (f64bits.h), with one
-// rarely taken branch each for the values that need the instruction.  The results are the
-// same bits.  Measured: 4 heliospheres x 3 species x 30 energies, 1.4e5 paths 738 -> 328 ms;
+// The FP64 pipe takes 64 clocks per warp instruction and scheduler, so only the sums stay on it;
+// conversions, comparisons and the finiteness test run on the bits (f64bits.h).  The results
+// are the same bits.  Measured: 4 heliospheres x 3 species x 30 energies, 1.4e5 paths 738 -> 328 ms;
 // one squashed heliosphere 316 -> 175 ms.
 template <>
 struct Acc<COSMICA_PREC_MIXED_F64ACC> {
@@ -141,30 +155,19 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
         const uint64_t bt = bits64(th);
         const bool north = f64bits::less(bt, f64bits::kHalfPiBits);
         const uint64_t units = f64bits::pi_minus_units(bt);
-        fr = __uint_as_float(f64bits::narrow(bits64(r)));
-        fth = __uint_as_float(f64bits::narrow(bt));
-        fph = __uint_as_float(f64bits::narrow(bits64(ph)));
-        flnP = __uint_as_float(f64bits::narrow(bits64(lnP)));
-        float d = north ? fth : f64bits::pi_minus(units);    // distance to the nearer pole
-        if (!(f64bits::narrow_ok((uint32_t)__double2hiint(r)) & f64bits::narrow_ok((uint32_t)__double2hiint(th)) &
-              f64bits::narrow_ok((uint32_t)__double2hiint(ph)) & f64bits::narrow_ok((uint32_t)__double2hiint(lnP)) &
-              (north | f64bits::pi_minus_ok(units)))) {
-            fr = (float)r; fth = (float)th; fph = (float)ph; flnP = (float)lnP;
-            d = (float)(th < 0.5 * kPi ? th : kPi - th);
-        }
-        sin_th = m32::sin_from_pole_distance(d);
+        fr = narrow64(r);
+        fth = narrow64(th);
+        fph = narrow64(ph);
+        flnP = narrow64(lnP);
+        sin_th = m32::sin_from_pole_distance(north ? fth : f64bits::pi_minus(units));   // of the nearer pole's distance
     }
     // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone)
     template <bool P>
     __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
     {
-        double ar = widen64(dr), ath = widen64(dth), aph = widen64(dph), aP = widen64(dlnP), at = widen64(dt);
-        if (!(widen64_ok(dr) & widen64_ok(dth) & widen64_ok(dph) & (!P | widen64_ok(dlnP)) & widen64_ok(dt))) {
-            ar = (double)dr; ath = (double)dth; aph = (double)dph; aP = (double)dlnP; at = (double)dt;
-        }
-        r += ar; th += ath; ph += aph;
-        if (P) lnP += aP;
-        s += at;
+        r += widen64(dr); th += widen64(dth); ph += widen64(dph);
+        if (P) lnP += widen64(dlnP);
+        s += widen64(dt);
     }
     __device__ void boundaries(float)
     {
@@ -179,6 +182,19 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
             }
             if (ph < 0.0 || ph >= kTwoPi) ph = ph - kTwoPi * floor(ph / kTwoPi);
         }
+    }
+    // as in the compensated state, on the high words
+    __device__ bool calm(float, bool sphere) const
+    {
+        return (__double2hiint(r) > __double2hiint(r_in)) & (__double2hiint(r) < (sphere ? __double2hiint(Rout) : 0x7FF00000)) &
+               ((uint32_t)__double2hiint(th) < (uint32_t)(f64bits::kPiBits >> 32)) &
+               (__double2hiint(ph) < 0x40291EB8) & ((uint32_t)__double2hiint(ph) < 0xC0191EB8u) &
+               f64bits::is_finite(bits64(lnP)) & f64bits::is_finite(bits64(s));
+    }
+    bool __device__ phi_out() const { return f64bits::outside_half_open(bits64(ph), f64bits::kTwoPiBits); }
+    __device__ void wrap_near()
+    {
+        ph += __double2hiint(ph) < 0 ? kTwoPi : (f64bits::less(bits64(ph), f64bits::kTwoPiBits) ? 0.0 : -kTwoPi);
     }
     // (a non-NaN comparison; finite() is asked first)
     __device__ bool exited() const { return !f64bits::less(bits64(r), bits64(Rout)); }
@@ -226,20 +242,71 @@ struct EnergyAcc<COSMICA_PREC_MIXED_F64ACC, true> {
     __device__ float fT() const { return narrow64(T); }
     __device__ void add(float dT, float dLam)
     {
-        double aT = widen64(dT), aL = widen64(dLam);
-        if (!(widen64_ok(dT) & widen64_ok(dLam))) { aT = (double)dT; aL = (double)dLam; }
-        T += aT; Lam += aL;
+        T += widen64(dT);
+        Lam += widen64(dLam);
     }
     __device__ double T64() const { return T; }
     __device__ double lw() const { return -Lam; }
 };
 
-// a lane's complete state, moved through shared memory by block compaction
-template <int ACC, bool EN>
-struct Packed {
-    Lane L;
-    Acc<ACC> x;
-    EnergyAcc<ACC, EN> en;
-};
+// A path between two kernels of one launch: its exact state in its own exit record (float-float
+// pairs and doubles both fill the record's 8-byte fields; the energy form keeps T in ln P's
+// place and the loss integral in the weight's).
+__device__ __forceinline__ double pair_bits(const m32::FF &a) { return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo)); }
+__device__ __forceinline__ m32::FF from_pair_bits(double v)
+{
+    m32::FF a;
+    a.hi = __int_as_float(__double2hiint(v));
+    a.lo = __int_as_float(__double2loint(v));
+    return a;
+}
+template <bool EN>
+__device__ __forceinline__ void park(const ExitPtrs &o, uint64_t g, const Acc<COSMICA_PREC_MIXED> &x,
+                                     const EnergyAcc<COSMICA_PREC_MIXED, EN> &en)
+{
+    o.r[g] = pair_bits(x.r); o.th[g] = pair_bits(x.th); o.ph[g] = pair_bits(x.ph); o.s[g] = pair_bits(x.s);
+    if constexpr (EN) {
+        o.lnP[g] = pair_bits(en.T);
+        o.lw[g] = pair_bits(en.Lam);
+    } else {
+        o.lnP[g] = pair_bits(x.lnP);
+    }
+}
+template <bool EN>
+__device__ __forceinline__ void unpark(const ExitPtrs &o, uint64_t g, Acc<COSMICA_PREC_MIXED> &x,
+                                       EnergyAcc<COSMICA_PREC_MIXED, EN> &en)
+{
+    x.r = from_pair_bits(o.r[g]); x.th = from_pair_bits(o.th[g]); x.ph = from_pair_bits(o.ph[g]); x.s = from_pair_bits(o.s[g]);
+    if constexpr (EN) {
+        en.T = from_pair_bits(o.lnP[g]);
+        en.Lam = from_pair_bits(o.lw[g]);
+    } else {
+        x.lnP = from_pair_bits(o.lnP[g]);
+    }
+}
+template <bool EN>
+__device__ __forceinline__ void park(const ExitPtrs &o, uint64_t g, const Acc<COSMICA_PREC_MIXED_F64ACC> &x,
+                                     const EnergyAcc<COSMICA_PREC_MIXED_F64ACC, EN> &en)
+{
+    o.r[g] = x.r; o.th[g] = x.th; o.ph[g] = x.ph; o.s[g] = x.s;
+    if constexpr (EN) {
+        o.lnP[g] = en.T;
+        o.lw[g] = en.Lam;
+    } else {
+        o.lnP[g] = x.lnP;
+    }
+}
+template <bool EN>
+__device__ __forceinline__ void unpark(const ExitPtrs &o, uint64_t g, Acc<COSMICA_PREC_MIXED_F64ACC> &x,
+                                       EnergyAcc<COSMICA_PREC_MIXED_F64ACC, EN> &en)
+{
+    x.r = o.r[g]; x.th = o.th[g]; x.ph = o.ph[g]; x.s = o.s[g];
+    if constexpr (EN) {
+        en.T = o.lnP[g];
+        en.Lam = o.lw[g];
+    } else {
+        x.lnP = o.lnP[g];
+    }
+}
 
 }  // namespace cosmica

@@ -381,6 +381,39 @@ __device__ __forceinline__ void ff_add(FF &a, float d)
     a.hi = hi;
 }
 
+// Two of them at once in packed FP32 pairs (one issue slot per pair of operations; the
+// same roundings): (a, b) += (da, db).
+__device__ __forceinline__ uint64_t pk(float a, float b)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpk(uint64_t v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t v;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
+{
+    uint64_t v;
+    asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ void ff_add2(FF &a, FF &b, float da, float db)
+{
+    const uint64_t ah = pk(a.hi, b.hi), al = pk(a.lo, b.lo), d = pk(da, db);
+    const uint64_t s = add2(ah, d);
+    const uint64_t bb = sub2(s, ah);
+    const uint64_t err = add2(sub2(ah, sub2(s, bb)), sub2(d, bb));
+    const uint64_t lo = add2(al, err);
+    const uint64_t hi = add2(s, lo);
+    unpk(sub2(lo, sub2(hi, s)), a.lo, b.lo);
+    unpk(hi, a.hi, b.hi);
+}
+
 __device__ __forceinline__ void ff_add_ff(FF &a, float bh, float bl)
 {
     ff_add(a, bh);

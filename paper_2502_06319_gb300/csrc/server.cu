@@ -33,6 +33,18 @@ using namespace cosmica::host;
 
 namespace {
 
+constexpr uint32_t kMaxSlots = 256;
+constexpr uint32_t kMaxEnergies = 256;
+constexpr uint32_t kMaxBins = 8192;
+
+// device counters of the server, read back as one block after each quantum
+struct Control {
+    unsigned long long cursors[2];        // cleared before each quantum, like n_susp
+    unsigned int n_susp, pad;
+    unsigned long long steps[kMaxSlots];
+    unsigned int done[kMaxSlots];
+};
+
 struct Req {
     cosmica_params p;
     cosmica_species sp;
@@ -88,10 +100,6 @@ struct RangeAlloc {
     }
 };
 
-constexpr uint32_t kMaxSlots = 256;
-constexpr uint32_t kMaxEnergies = 256;
-constexpr uint32_t kMaxBins = 8192;
-
 double now_s(std::chrono::steady_clock::time_point t0)
 {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -111,22 +119,15 @@ struct cosmica_server {
     uint64_t arena_cap = 0;
     DevParams *d_prm = nullptr;
     DevSpecies *d_spc = nullptr;
-    unsigned int *d_done = nullptr;
-    unsigned long long *d_steps = nullptr;
     Suspended *d_susp[2] = {nullptr, nullptr};
     uint64_t lane_cap = 0;
-    unsigned int *d_nsusp = nullptr;
-    unsigned long long *d_cursors = nullptr;
+    Control *d_ctl = nullptr;
     unsigned long long *d_hist = nullptr;
     double *d_J = nullptr, *d_S = nullptr;
     SpecItem *d_spec_items = nullptr;
     DevBuf tables, weights;
     Staging stage;
-    // pinned read-back of the per-quantum counters
-    unsigned long long *h_cursor = nullptr;
-    unsigned int *h_nsusp = nullptr;
-    unsigned int *h_done = nullptr;
-    unsigned long long *h_steps = nullptr;
+    Control *h_ctl = nullptr;   // pinned read-back after each quantum
     // host bookkeeping (guarded by mu)
     std::mutex mu;
     std::condition_variable cv_submit, cv_done;
@@ -165,8 +166,8 @@ bool cosmica_server::upload_slot(Req &r)
     cudaError_t e = cudaMemcpyAsync(d_prm + r.slot, &dp, sizeof(dp), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_spc + r.slot, &ds, sizeof(ds), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = launch_derive(d_prm + r.slot, 1, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_done + r.slot, 0, sizeof(unsigned int), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_steps + r.slot, 0, sizeof(unsigned long long), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_ctl->done + r.slot, 0, sizeof(unsigned int), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_ctl->steps + r.slot, 0, sizeof(unsigned long long), stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);   // dp, ds live on this stack frame
     if (e != cudaSuccess) {
         set_failed(std::string("server slot upload: ") + cudaGetErrorString(e));
@@ -284,26 +285,26 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
     a.resume = d_susp[cur];
     a.n_resume = n_resume;
     a.suspend = d_susp[cur ^ 1];
-    a.n_suspend = d_nsusp;
-    a.cursors = d_cursors;
+    a.n_suspend = &d_ctl->n_susp;
+    a.cursors = d_ctl->cursors;
     a.arena = arena;
-    a.req_done = d_done;
-    a.req_steps = d_steps;
+    a.req_done = d_ctl->done;
+    a.req_steps = d_ctl->steps;
     a.budget = budget;
-    cudaError_t e = cudaMemsetAsync(d_cursors, 0, 2 * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_nsusp, 0, sizeof(unsigned int), stream);
-    if (e == cudaSuccess) e = launch_serve(a, precision, ext, full, shape, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_cursor, d_cursors, sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_nsusp, d_nsusp, sizeof(unsigned int), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_done, d_done, kMaxSlots * sizeof(unsigned int), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_steps, d_steps, kMaxSlots * 8, cudaMemcpyDeviceToHost, stream);
+    // no more warps per scheduler than the particles fill: fewer step faster
+    PersistentShape q = shape;
+    const uint64_t layer = (uint64_t)num_sms() * shape.block;
+    q.grid = (unsigned)std::min<uint64_t>(shape.grid, (uint64_t)num_sms() * ((n_fresh + n_resume + layer - 1) / layer));
+    cudaError_t e = cudaMemsetAsync(d_ctl, 0, offsetof(Control, steps), stream);
+    if (e == cudaSuccess) e = launch_serve(a, precision, ext, full, q, stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h_ctl, d_ctl, sizeof(Control), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
         set_failed(std::string("server quantum: ") + cudaGetErrorString(e));
         return false;
     }
     // account the fresh particles this quantum started, in table order
-    uint64_t taken = std::min<uint64_t>(*h_cursor, n_fresh);
+    uint64_t taken = std::min<uint64_t>(h_ctl->cursors[0], n_fresh);
     std::vector<uint64_t> done_tickets;
     {
         std::lock_guard<std::mutex> lk(mu);
@@ -318,16 +319,16 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
         for (auto &kv : reqs) {
             Req &r = kv.second;
             if (r.state != 1) continue;
-            const uint64_t d = h_done[r.slot];
+            const uint64_t d = h_ctl->done[r.slot];
             inflight += r.total - d;
             if (d == r.total) {
-                r.steps = h_steps[r.slot];
+                r.steps = h_ctl->steps[r.slot];
                 done_tickets.push_back(kv.first);
             }
         }
         st.in_flight_particles = inflight;
     }
-    n_resume = *h_nsusp;
+    n_resume = h_ctl->n_susp;
     cur ^= 1;
     for (uint64_t t : done_tickets) {
         Req *r;
@@ -408,21 +409,17 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     A(&s->arena_mem, C * per + 8 * 256);
     A((void **)&s->d_prm, kMaxSlots * sizeof(DevParams));
     A((void **)&s->d_spc, kMaxSlots * sizeof(DevSpecies));
-    A((void **)&s->d_done, kMaxSlots * sizeof(unsigned int));
-    A((void **)&s->d_steps, kMaxSlots * 8);
+    A((void **)&s->d_ctl, sizeof(Control));
     A((void **)&s->d_susp[0], s->lane_cap * sizeof(Suspended));
     A((void **)&s->d_susp[1], s->lane_cap * sizeof(Suspended));
-    A((void **)&s->d_nsusp, sizeof(unsigned int));
-    A((void **)&s->d_cursors, 2 * sizeof(unsigned long long));
     A((void **)&s->d_hist, (size_t)kMaxEnergies * (kMaxBins + 3) * 8);
     A((void **)&s->d_J, kMaxEnergies * 8);
     A((void **)&s->d_S, kMaxEnergies * 8);
     A((void **)&s->d_spec_items, kMaxEnergies * sizeof(SpecItem));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_cursor, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_nsusp, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_done, kMaxSlots * sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_steps, kMaxSlots * 8);
-    if (e == cudaSuccess) e = cudaMemset(s->d_done, 0, kMaxSlots * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_ctl, sizeof(Control));
+    if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, sizeof(Control));
+    // lanes without a particle read slot 0's parameters (no shells: no table index)
+    if (e == cudaSuccess) e = cudaMemset(s->d_prm, 0, kMaxSlots * sizeof(DevParams));
     if (e != cudaSuccess) {
         cosmica_status rs = cuda_fail(e, "server allocation");
         cosmica_server_destroy(s);
@@ -561,13 +558,11 @@ extern "C" void cosmica_server_destroy(cosmica_server *s)
     s->tables.release();
     s->weights.release();
     s->stage.release();
-    void *dev[] = {s->arena_mem, s->d_prm, s->d_spc, s->d_done, s->d_steps, s->d_susp[0], s->d_susp[1],
-                   s->d_nsusp, s->d_cursors, s->d_hist, s->d_J, s->d_S, s->d_spec_items};
+    void *dev[] = {s->arena_mem, s->d_prm, s->d_spc, s->d_ctl, s->d_susp[0], s->d_susp[1], s->d_hist,
+                   s->d_J, s->d_S, s->d_spec_items};
     for (void *p : dev)
         if (p) cudaFree(p);
-    void *hst[] = {s->h_cursor, s->h_nsusp, s->h_done, s->h_steps};
-    for (void *p : hst)
-        if (p) cudaFreeHost(p);
+    if (s->h_ctl) cudaFreeHost(s->h_ctl);
     if (s->stream) cudaStreamDestroy(s->stream);
     delete s;
 }
