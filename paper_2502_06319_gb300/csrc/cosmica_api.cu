@@ -567,8 +567,9 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
     if (m->p.precision == COSMICA_PREC_FP64) {
         e = launch_propagate_fp64(a, fp64_variant(&m->p, 1), num_sms(), s);
     } else {
-        const MixedVariant v{m->p.precision, m->p.formulation == 1, m->p.n_shells > 0 || m->p.squashed != 0,
-                             full_model(m->p)};
+        Extensions ext;
+        ext.add(m->p);
+        const MixedVariant v{m->p.precision, m->p.formulation == 1, ext.kind(), full_model(m->p)};
         e = launch_propagate_mixed(a, v, shape_for(v, nullptr, total), num_sms(), s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
@@ -842,13 +843,13 @@ struct cosmica_batch {
     std::vector<cosmica_params> params;
     std::vector<cosmica_species> species;
     int precision = 0;
-    bool extended = false;     // some parameter set has radial shells or a squashed heliosphere
+    Extensions ext;            // radial shells and squashed heliospheres among the parameter sets
     bool full = true;          // every parameter set is the full model (see full_model)
     DevParams *d_prm = nullptr;
     const float *d_f32 = nullptr;   // paged field-major FP32 blocks (inside the d_prm allocation)
     DevSpecies *d_spc = nullptr;
     Tables tab;
-    MixedVariant variant() const { return MixedVariant{precision, params[0].formulation == 1, extended, full}; }
+    MixedVariant variant() const { return MixedVariant{precision, params[0].formulation == 1, ext.kind(), full}; }
     ExitStage exit_stage;
     DevBuf spec_items, lis_buf;
     Staging spec_stage, lis_stage;
@@ -901,7 +902,7 @@ extern "C" cosmica_status cosmica_batch_create(const cosmica_params *params, uin
     b->species.assign(species, species + n_species);
     b->precision = params[0].precision;
     for (uint32_t i = 0; i < n_params; ++i) {
-        b->extended = b->extended || params[i].n_shells > 0 || params[i].squashed != 0;
+        b->ext.add(params[i]);
         b->full = b->full && full_model(params[i]);
     }
     cosmica_status st = upload_params(params, n_params, &b->d_prm, &b->d_f32);
@@ -1127,7 +1128,7 @@ extern "C" cosmica_status cosmica_autotune(cosmica_batch *b, const cosmica_work_
     int size_class = 0;
     while ((n_all >> size_class) > 1) ++size_class;
     // the kernel variant (energy form, shells) has its own registers, hence its own best shape
-    const int variant = (b->params[0].formulation == 1 ? 1 : 0) | (b->extended ? 2 : 0) | (b->full ? 4 : 0);
+    const int variant = (b->params[0].formulation == 1 ? 1 : 0) | (b->full ? 2 : 0) | b->ext.kind() * 4;
     const auto key = std::make_tuple(dev, b->precision, drift, ts, size_class, variant);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);

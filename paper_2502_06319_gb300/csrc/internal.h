@@ -88,9 +88,28 @@ struct ServeArgs {
     uint32_t budget;               // steps per lane per quantum
 };
 
-// full: every resident request is the full model (the variant without uniform branches)
-cudaError_t launch_serve(const ServeArgs &a, int acc, bool ext, bool full, PersistentShape shape, cudaStream_t s);
-int serve_max_blocks_per_sm(int acc, bool ext, bool full, unsigned block);
+// ext: Extensions::kind() of the resident requests; full: every one is the full model (the variant
+// without uniform branches)
+cudaError_t launch_serve(const ServeArgs &a, int acc, int ext, bool full, PersistentShape shape, cudaStream_t s);
+int serve_max_blocks_per_sm(int acc, int ext, bool full, unsigned block);
+
+// extensions of a launch's parameter sets
+struct Extensions {
+    bool shells = false, no_shells = false, squashed = false, round = false;   // some set has (has not) ...
+    void add(const cosmica_params &p)
+    {
+        (p.n_shells > 0 ? shells : no_shells) = true;
+        (p.squashed != 0 ? squashed : round) = true;
+    }
+    // 0 none, 1 shells in every set, 2 every set squashed, 3 anything else (m32::kExt...)
+    int kind() const
+    {
+        if (!shells && !squashed) return 0;
+        if (!no_shells && !squashed) return 1;
+        if (!shells && !round) return 2;
+        return 3;
+    }
+};
 
 void note_launch();
 
@@ -117,7 +136,7 @@ cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, c
 struct MixedVariant {
     int acc;        // COSMICA_PREC_MIXED or COSMICA_PREC_MIXED_F64ACC
     bool energy;    // energy formulation (Eq. 1) instead of the momentum form
-    bool extended;  // some parameter set of the launch has radial shells or a squashed heliosphere
+    int extended;   // Extensions::kind() of the launch's parameter sets
     bool full;      // every set is the full model: drift and current sheet on, adaptive step
 };
 inline Fp64Variant fp64_variant(const cosmica_params *ps, size_t n)

@@ -82,7 +82,7 @@ __device__ __forceinline__ void take(const LaunchArgs &a, const MixedStage &st, 
 // those of the next step: the increments are added and nothing else is looked at.  One block
 // without branches (in the full-model variant), so that the compiler interleaves the
 // generator with the coefficients.
-template <int ACC, bool EN, bool EXT, bool FULL>
+template <int ACC, bool EN, int EXT, bool FULL>
 __device__ __forceinline__ void advance(const float *params, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en, float &z0,
                                         float &z1, float &z2)
 {
@@ -115,25 +115,25 @@ __device__ __forceinline__ void advance(const float *params, Lane &L, Acc<ACC> &
 
 // whether the state after a step needs settle(): a boundary other than the longitude's, an end of
 // the path, or nearly so
-template <int ACC, bool EXT>
+template <int ACC, int EXT>
 __device__ __forceinline__ bool needs_settling(const float *params, const Lane &L, const Acc<ACC> &x)
 {
     const P32<kSetsPerPage> q{params};
-    const bool squashed = EXT && P32F(q, sq) != 0.0f;
+    const bool squashed = m32::is_squashed<EXT>(q);
     bool calm = x.calm(P32F(q, r_in), !squashed) & (L.k < L.max_steps);
-    if (squashed) calm = calm && !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
+    if (squashed) calm &= !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
     return !calm;
 }
 
 // Boundaries and the three ends of a path; true when the path ended (exit record written).
-template <int ACC, bool EN, bool EXT>
+template <int ACC, bool EN, int EXT>
 __device__ __forceinline__ bool settle(const LaunchArgs &a, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en,
                                        unsigned long long &my_steps)
 {
     const P32<kSetsPerPage> q{L.q};
     x.boundaries(P32F(q, r_in));
     const bool fin = x.finite();
-    const bool out = (EXT && P32F(q, sq) != 0.0f) ? m32::outside_squashed(q, x.fr(), x.fth(), x.fph()) : x.exited();
+    const bool out = m32::is_squashed<EXT>(q) ? m32::outside_squashed(q, x.fr(), x.fth(), x.fph()) : x.exited();
     const bool lim = L.k >= L.max_steps;
     if (fin & !out & !lim) return false;
     const int status = !fin ? COSMICA_PATH_NONFINITE : (out ? COSMICA_PATH_EXIT : COSMICA_PATH_STEP_LIMIT);
@@ -167,7 +167,7 @@ __device__ __forceinline__ bool settle(const LaunchArgs &a, Lane &L, Acc<ACC> &x
 // normals after the tests: a lone path's step 0.68 -> 0.36 us, a warp's step with four warps per
 // scheduler 1.05 -> 0.93 us, 5.7e6 paths of 4 heliospheres 8.3e10 steps/s, one spectrum of 6e5
 // paths 141 -> 99 ms, 1.8e6 paths of 16 heliospheres 870 -> 694 ms.
-template <int ACC, bool EN, bool EXT, bool FULL>
+template <int ACC, bool EN, int EXT, bool FULL>
 __global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedStage st)
 {
     const unsigned lane = threadIdx.x & 31u;
@@ -254,7 +254,7 @@ __global__ void k_debug_eval32(const DevParams *__restrict__ prm, const DevSpeci
     if (i >= n) return;
     float dbg[kDebugEvalN];
     m32::Drift c;
-    m32::eval<true, false, 1>(P32<1>{reinterpret_cast<const float *>(&prm[0].f)}, spc[0].aoz_m0_sq, spc[0].sgnq,
+    m32::eval<m32::kExtAny, false, 1>(P32<1>{reinterpret_cast<const float *>(&prm[0].f)}, spc[0].aoz_m0_sq, spc[0].sgnq,
                               (float)st[4 * i], (float)st[4 * i + 1], m32::sin_theta_f64(st[4 * i + 1]),
                               (float)st[4 * i + 2], (float)st[4 * i + 3], c, dbg);
     for (int j = 0; j < kDebugEvalN; ++j) out[(size_t)i * kDebugEvalN + j] = dbg[j];
@@ -272,8 +272,10 @@ static void visit_variant(MixedVariant v, Fn &&fn)
                 if (v.full) fn(A, E, X, std::true_type{});
                 else fn(A, E, X, std::false_type{});
             };
-            if (v.extended) on_ext(std::true_type{});
-            else on_ext(std::false_type{});
+            if (v.extended == m32::kExtNone) on_ext(std::integral_constant<int, m32::kExtNone>{});
+            else if (v.extended == m32::kExtShells) on_ext(std::integral_constant<int, m32::kExtShells>{});
+            else if (v.extended == m32::kExtSquashed) on_ext(std::integral_constant<int, m32::kExtSquashed>{});
+            else on_ext(std::integral_constant<int, m32::kExtAny>{});
         };
         if (v.energy) on_energy(std::true_type{});
         else on_energy(std::false_type{});

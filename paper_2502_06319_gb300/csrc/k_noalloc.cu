@@ -231,8 +231,9 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
         e = launch_propagate_fp64(a, fp64_variant(params, 1), num_sms(), s);
     } else {
         const unsigned block = 128;
-        const MixedVariant v{params->precision, params->formulation == 1,
-                             params->n_shells > 0 || params->squashed != 0, full_model(*params)};
+        Extensions ext;
+        ext.add(*params);
+        const MixedVariant v{params->precision, params->formulation == 1, ext.kind(), full_model(*params)};
         const int bps = untuned_layers(total, num_sms(), mixed_max_blocks_per_sm(v, block));
         const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms() * (uint64_t)bps, (total + 3) / 4);
         e = launch_propagate_mixed(a, v, PersistentShape{block, (unsigned)grid, 64u}, num_sms(), s);

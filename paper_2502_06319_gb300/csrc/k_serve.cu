@@ -65,12 +65,12 @@ struct ServeLane {
     uint64_t exit_idx;
 };
 
-// EXT: some resident request has radial shells or a squashed heliosphere (the
-// extended model; compile-time, as in the batched kernel).  FULL: every resident
+// EXT: which extensions the resident requests have (compile-time, as in the batched
+// kernel).  FULL: every resident
 // request is the full model (drift and current sheet on, adaptive step), so the step
 // carries no uniform branch on those switches (the same DAG as the batched kernel's
 // full-model variant).
-template <int ACC, bool EXT, bool FULL>
+template <int ACC, int EXT, bool FULL>
 __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
 {
     const unsigned lane = threadIdx.x & 31u;
@@ -170,9 +170,9 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
             x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
             S.L.k += 1u;
             m32::normals(S.L.seed, S.L.pid, S.L.k, z0, z1, z2);
-            const bool squashed = EXT && P32F(q, sq) != 0.0f;
+            const bool squashed = m32::is_squashed<EXT>(q);
             bool calm = x.calm(P32F(q, r_in), !squashed) & (S.L.k < S.L.max_steps);
-            if (squashed) calm = calm && !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
+            if (squashed) calm &= !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
             see = active && !calm;
             const bool wrap = active && x.phi_out();
             ++used;
@@ -184,8 +184,7 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
         if (see) {
             x.boundaries(P32F(q, r_in));
             const bool fin = x.finite();
-            const bool out = (EXT && P32F(q, sq) != 0.0f) ? m32::outside_squashed(q, x.fr(), x.fth(), x.fph())
-                                                           : x.exited();
+            const bool out = m32::is_squashed<EXT>(q) ? m32::outside_squashed(q, x.fr(), x.fth(), x.fph()) : x.exited();
             const bool lim = S.L.k >= S.L.max_steps;
             if (!(fin & !out & !lim)) {
                 const int status = !fin ? COSMICA_PATH_NONFINITE : (out ? COSMICA_PATH_EXIT : COSMICA_PATH_STEP_LIMIT);
@@ -222,21 +221,23 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
 
 // Call fn(acc, extended, full) with each flag as a compile-time constant.
 template <class Fn>
-static void visit_serve(int acc, bool ext, bool full, Fn &&fn)
+static void visit_serve(int acc, int ext, bool full, Fn &&fn)
 {
     auto on_acc = [&](auto A) {
         auto on_ext = [&](auto X) {
             if (full) fn(A, X, std::true_type{});
             else fn(A, X, std::false_type{});
         };
-        if (ext) on_ext(std::true_type{});
-        else on_ext(std::false_type{});
+        if (ext == m32::kExtNone) on_ext(std::integral_constant<int, m32::kExtNone>{});
+        else if (ext == m32::kExtShells) on_ext(std::integral_constant<int, m32::kExtShells>{});
+        else if (ext == m32::kExtSquashed) on_ext(std::integral_constant<int, m32::kExtSquashed>{});
+        else on_ext(std::integral_constant<int, m32::kExtAny>{});
     };
     if (acc == COSMICA_PREC_MIXED_F64ACC) on_acc(std::integral_constant<int, COSMICA_PREC_MIXED_F64ACC>{});
     else on_acc(std::integral_constant<int, COSMICA_PREC_MIXED>{});
 }
 
-int serve_max_blocks_per_sm(int acc, bool ext, bool full, unsigned block)
+int serve_max_blocks_per_sm(int acc, int ext, bool full, unsigned block)
 {
     int nb = 0;
     visit_serve(acc, ext, full, [&](auto A, auto X, auto F) {
@@ -247,7 +248,7 @@ int serve_max_blocks_per_sm(int acc, bool ext, bool full, unsigned block)
     return nb;
 }
 
-cudaError_t launch_serve(const ServeArgs &a, int acc, bool ext, bool full, PersistentShape shape, cudaStream_t s)
+cudaError_t launch_serve(const ServeArgs &a, int acc, int ext, bool full, PersistentShape shape, cudaStream_t s)
 {
     cudaGetLastError();
     visit_serve(acc, ext, full, [&](auto A, auto X, auto F) {

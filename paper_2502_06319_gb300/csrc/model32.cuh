@@ -58,20 +58,23 @@ __device__ __forceinline__ void shell_weights(const P32<ST> &q, float r, int &a,
 {
     const int n = (int)P32F(q, n_sh);
     const int k = min(max((int)(r * P32F(q, sh_inv_dr)), 0), n - 1);
-    float x = 0.0f;
-    a = k;
-    b = k;
     const float lo_edge = (float)k * P32F(q, sh_dr);
     const float hi_edge = (float)(k + 1) * P32F(q, sh_dr);
-    if (k >= 1 && r < lo_edge + P32F(q, sh_w)) {
-        a = k - 1;
-        x = (r - (lo_edge - P32F(q, sh_w))) * P32F(q, sh_inv_2w);
-    } else if (k + 1 <= n - 1 && r > hi_edge - P32F(q, sh_w)) {
-        b = k + 1;
-        x = (r - (hi_edge - P32F(q, sh_w))) * P32F(q, sh_inv_2w);
-    }
+    const bool in_lo = (k >= 1) & (r < lo_edge + P32F(q, sh_w));
+    const bool in_hi = !in_lo & (k + 1 <= n - 1) & (r > hi_edge - P32F(q, sh_w));
+    a = in_lo ? k - 1 : k;
+    b = in_hi ? k + 1 : k;
+    const float from = (in_lo ? lo_edge : hi_edge) - P32F(q, sh_w);
+    const float x = (in_lo | in_hi) ? (r - from) * P32F(q, sh_inv_2w) : 0.0f;
     S = x * x * fmaf(-2.0f, x, 3.0f);
     dS = 6.0f * x * (1.0f - x) * P32F(q, sh_inv_2w);
+}
+
+constexpr int kExtNone = 0, kExtShells = 1, kExtSquashed = 2, kExtAny = 3;
+template <int EXT, uint32_t ST>
+__device__ __forceinline__ bool is_squashed(const P32<ST> &q)
+{
+    return EXT == kExtSquashed || (EXT == kExtAny && P32F(q, sq) != 0.0f);
 }
 
 // Coefficients at (r, th, ph, lnP).  q: FP32 constants of the heliosphere (read through P32).
@@ -133,17 +136,20 @@ __device__ __forceinline__ float sin_theta_f64(double th)
     return sin_from_pole_distance((float)d);
 }
 
-// EXT: the parameter sets of the launch may have radial shells or a squashed
-// heliosphere (compile-time, so that launches of the basic model carry none of
-// that code or its registers).  FULL: every set of the launch is the full model
-// (drift and current sheet on, adaptive step); the uniform branches on those
-// switches then vanish and the step is one long branch-free block, which the
+// EXT: which extensions the parameter sets of the launch have (compile-time, so that
+// launches of the basic model carry none of that code or its registers): kExtNone, or all
+// of them radial shells (kExtShells), all of them a squashed heliosphere (kExtSquashed),
+// or any mixture, tested set by set (kExtAny): the first three leave the step one block
+// without branches.  Measured against kExtAny: 2e5 paths through 15 shells 110 -> 80 ms, a
+// lone path of the energy form in a squashed heliosphere 0.62 -> 0.41 us a step.  FULL: every
+// set of the launch is the full model (drift and current sheet on, adaptive step); the
+// uniform branches on those switches then vanish and the step is one long branch-free block, which the
 // compiler schedules with more instruction-level parallelism (the latency of a
 // lone path is what bounds the end of a launch).
 // sin_th: sin(theta) accurate relative to itself near the poles (the caller derives
 // it from the compensated state, see sin_from_pole_distance); cos theta is taken
 // from the SFU, whose absolute error is harmless in cot theta.
-template <bool EXT, bool FULL, uint32_t ST>
+template <int EXT, bool FULL, uint32_t ST>
 __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float r, float th, float sin_th,
                                      float ph, float lnP, Drift &o, float *dbg = nullptr)
 {
@@ -176,7 +182,7 @@ __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float
     // and dg = -0 exactly, which leave every later value as the branch would (measured:
     // +2.6 % steps/s on config 3, +2.4 % on config 2, which has no shock)
     float g = 1.0f, dg = 0.0f, dg_dth = 0.0f, dg_dph = 0.0f;
-    const bool squashed = EXT && P32F(q, sq) != 0.0f;
+    const bool squashed = is_squashed<EXT>(q);
     if (FULL || P32F(q, ts_drop) != 0.0f) {
         float Rts = P32F(q, R_ts), dR_dmu = 0.0f, dmu_dth = 0.0f, dmu_dph = 0.0f;
         if (squashed) {
@@ -196,7 +202,7 @@ __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float
 
     // radial shells: K0 and the sheet tilt of the shell holding r (the single-region
     // tilt is read where the sheet needs it, so that it is not live before)
-    const bool shells = EXT && P32F(q, n_sh) != 0.0f;
+    const bool shells = EXT == kExtShells || (EXT == kExtAny && P32F(q, n_sh) != 0.0f);
     float K0 = P32F(q, K0), dK0 = 0.0f, sh_ta = 0.0f, sh_ta2 = 0.0f, dta = 0.0f;
     if (shells) {
         int a, b;

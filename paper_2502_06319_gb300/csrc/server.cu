@@ -240,14 +240,14 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
     std::vector<ServeItem> its;
     std::vector<uint64_t> pre(1, 0);
     std::vector<std::pair<uint64_t, uint32_t>> owner;   // (ticket, energy) per item
-    bool ext = false;   // a resident request has radial shells or a squashed heliosphere
+    Extensions ext;
     bool full = true;   // every resident request is the full model
     {
         std::lock_guard<std::mutex> lk(mu);
         for (auto &kv : reqs) {
             Req &r = kv.second;
             if (r.state != 1) continue;
-            ext = ext || r.p.n_shells > 0 || r.p.squashed != 0;
+            ext.add(r.p);
             full = full && full_model(r.p);
             for (uint32_t e = 0; e < r.T.size(); ++e) {
                 const uint64_t left = r.n[e] - r.started[e];
@@ -296,7 +296,7 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
     const uint64_t layer = (uint64_t)num_sms() * shape.block;
     q.grid = (unsigned)std::min<uint64_t>(shape.grid, (uint64_t)num_sms() * ((n_fresh + n_resume + layer - 1) / layer));
     cudaError_t e = cudaMemsetAsync(d_ctl, 0, offsetof(Control, steps), stream);
-    if (e == cudaSuccess) e = launch_serve(a, precision, ext, full, q, stream);
+    if (e == cudaSuccess) e = launch_serve(a, precision, ext.kind(), full, q, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_ctl, d_ctl, sizeof(Control), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
@@ -392,7 +392,7 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     // sized for the full model's kernel (the common case); a variant with fewer resident
     // blocks (extended heliosphere, or a model without drift or sheet) starts its extra
     // blocks as others finish, and they take whatever work is left
-    const int bps = std::max(1, serve_max_blocks_per_sm(precision, false, true, block));
+    const int bps = std::max(1, serve_max_blocks_per_sm(precision, 0, true, block));
     s->shape = PersistentShape{block, (unsigned)(num_sms() * bps), 0u};
     s->lane_cap = (uint64_t)s->shape.grid * block;
     const size_t fixed = 2 * s->lane_cap * sizeof(Suspended) + kMaxSlots * (sizeof(DevParams) + sizeof(DevSpecies) + 12) +
@@ -407,9 +407,11 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
     auto A = [&](void **p, size_t n) { if (e == cudaSuccess) e = cudaMalloc(p, n); };
     A(&s->arena_mem, C * per + 8 * 256);
-    A((void **)&s->d_prm, kMaxSlots * sizeof(DevParams));
-    A((void **)&s->d_spc, kMaxSlots * sizeof(DevSpecies));
-    A((void **)&s->d_ctl, sizeof(Control));
+    // counters, parameter sets and species of the slots in one block
+    const size_t b_ctl = align_up(sizeof(Control), 256), b_prm = align_up(kMaxSlots * sizeof(DevParams), 256);
+    A((void **)&s->d_ctl, b_ctl + b_prm + kMaxSlots * sizeof(DevSpecies));
+    s->d_prm = (DevParams *)((char *)s->d_ctl + b_ctl);
+    s->d_spc = (DevSpecies *)((char *)s->d_prm + b_prm);
     A((void **)&s->d_susp[0], s->lane_cap * sizeof(Suspended));
     A((void **)&s->d_susp[1], s->lane_cap * sizeof(Suspended));
     A((void **)&s->d_hist, (size_t)kMaxEnergies * (kMaxBins + 3) * 8);
@@ -417,9 +419,8 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     A((void **)&s->d_S, kMaxEnergies * 8);
     A((void **)&s->d_spec_items, kMaxEnergies * sizeof(SpecItem));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_ctl, sizeof(Control));
-    if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, sizeof(Control));
-    // lanes without a particle read slot 0's parameters (no shells: no table index)
-    if (e == cudaSuccess) e = cudaMemset(s->d_prm, 0, kMaxSlots * sizeof(DevParams));
+    // lanes without a particle read slot 0's parameters (zero: no shells, so no table index)
+    if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, b_ctl + sizeof(DevParams));
     if (e != cudaSuccess) {
         cosmica_status rs = cuda_fail(e, "server allocation");
         cosmica_server_destroy(s);
@@ -558,7 +559,7 @@ extern "C" void cosmica_server_destroy(cosmica_server *s)
     s->tables.release();
     s->weights.release();
     s->stage.release();
-    void *dev[] = {s->arena_mem, s->d_prm, s->d_spc, s->d_ctl, s->d_susp[0], s->d_susp[1], s->d_hist,
+    void *dev[] = {s->arena_mem, s->d_ctl, s->d_susp[0], s->d_susp[1], s->d_hist,
                    s->d_J, s->d_S, s->d_spec_items};
     for (void *p : dev)
         if (p) cudaFree(p);
