@@ -125,10 +125,8 @@ constexpr uint32_t kLaunchCounters = 3 + 2 * kMixedStages;
 inline uint32_t list_entries(uint64_t n_total, int sms)
 {
     const uint64_t most = (uint64_t)(kMixedStages - 1) * 128u * (uint64_t)sms;
-    return n_total > 32ull * (uint64_t)sms ? (uint32_t)(n_total < most ? n_total : most) : 0u;
+    return n_total > 8ull * (uint64_t)sms ? (uint32_t)(n_total < most ? n_total : most) : 0u;
 }
-// most paths the team kernel takes over (32 per SM: eight teams of four lanes on every scheduler)
-inline uint32_t fp64_list_entries(int sms) { return 32u * (uint32_t)sms; }
 cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, cudaStream_t s);
 
 // mixed precision persistent kernel; acc = COSMICA_PREC_MIXED or COSMICA_PREC_MIXED_F64ACC

@@ -4,7 +4,9 @@
 //   k_derive          per-parameter-set constants (FP64 and the FP32 block)
 //   k_propagate64     the FP64 path: one lane per quasi-particle (Sec. IV.A), refilled from
 //                     the work queue, Euler-Maruyama until the path exits (step64.cuh)
-//   k_finish64        the last paths of a launch, or all of a small one: teams of lanes
+//   k_finish64, k_quad64
+//                     the last paths of a launch, or all of a small one: teams of lanes,
+//                     then the four warps of a block
 //   k_propagate_fp64  sets with radial shells or a squashed heliosphere: one thread per
 //                     quasi-particle, the step as it is defined (model64.cuh)
 //   k_debug_*         coefficient / RNG / elementary-function probes used by
@@ -15,6 +17,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "model64.cuh"
+#include "quad64.cuh"
 #include "step64.cuh"
 
 namespace cosmica {
@@ -161,11 +164,15 @@ __global__ void __launch_bounds__(128) k_propagate_fp64(const DevParams *__restr
 //     path ended take the next one from the queue, most expensive items first;
 //   * once no more than 32 paths per SM are left, every lane stores its path in its own exit
 //     record and k_finish64 takes them over with four lanes a path, which halves the slots of
-//     the step that the launch's slowest paths wait for; a launch that starts with so few
-//     goes there at once, with 16 lanes a path when there are eight paths per SM or fewer.
-// Measured against one thread per path with the plain step: 1e4 isotropic paths 86.8 -> 24.4 ms
-// (10 ms of it in the first kernel), 96 paths of the full model 349 -> 114 ms (52 -> 16.9 us a
-// step; the FP64 pipe 82 % busy), 2.5e4 paths 1384 -> 509 ms; the paths are the same bits.
+//     the step that the launch's slowest paths wait for;
+//   * once no more than 8 per SM are left, k_quad64 takes them over with the four warps of a
+//     block for up to eight paths (quad64.cuh), which halves the slots on the longest warp again.
+// A launch that starts with so few paths starts there.  (A mixture of isotropic and other sets
+// stays with k_finish64.)
+// Measured against one thread per path with the plain step: a step of the full model 52 us, 29 in
+// k_propagate64 (a lane a path), 17.4 in k_finish64 (477 slots, the FP64 pipe 84 % busy), 10.4 in
+// k_quad64 (250 slots on its longest warp); 1e4 isotropic paths 86.8 -> 23.2 ms, 2.5e4 paths of the
+// full model 1385 -> 352 ms.  The paths are the same bits.
 struct Path64 {
     uint64_t g, pid, seed;
     const DevParams *p;
@@ -315,17 +322,21 @@ __global__ void __launch_bounds__(128) k_propagate64(LaunchArgs a, uint32_t limi
 }
 
 // Teams of G lanes; team j of warp w takes entry j * warps + w, so that the schedulers share the
-// paths evenly.  fresh: the queue's paths from their start, else those of the list.
+// paths evenly.  from: null for the queue's paths from their start, else *n_from indices of
+// stored paths.  The last `limit` paths are left to the next kernel (if every path has a team of
+// its own: a path that waits for one cannot be left).
 template <int G, int ISO, bool EN>
-__global__ void __launch_bounds__(128) k_finish64(LaunchArgs a, bool fresh)
+__global__ void __launch_bounds__(128) k_finish64(LaunchArgs a, const uint32_t *from, const unsigned long long *n_from,
+                                                  uint32_t *to, unsigned long long *n_to, uint32_t limit)
 {
     __shared__ double tab[s64::kFnWords];
     s64::load_table(tab);
     __syncthreads();
-    const uint64_t n = fresh ? a.n_total : a.ended[1];
+    const uint64_t n = from ? *n_from : a.n_total;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = gridDim.x * (blockDim.x / 32), warp = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const s64::Team<G> team{(int)(lane & (G - 1))};
+    const bool hand_over = limit != 0 && n <= (uint64_t)warps * (32 / G);
     unsigned long long my_steps = 0;
     for (uint64_t first = warp; first < n; first += (uint64_t)warps * (32 / G)) {
         // a team without a path of its own follows the warp's first one and writes nothing
@@ -334,22 +345,113 @@ __global__ void __launch_bounds__(128) k_finish64(LaunchArgs a, bool fresh)
         if (!live) i = first;
         Path64 P;
         m64::State x;
-        if (fresh) fresh64(a, i, P, x);
-        else stored64<EN>(a, a.list[i], P, x);
+        if (!from) fresh64(a, i, P, x);
+        else stored64<EN>(a, from[i], P, x);
         double zs[3];          // normals of step (first of the round) + team lane
         for (uint32_t it = 0; __any_sync(0xffffffffu, live); ++it) {
+            if (hand_over && it % 16 == 15) {
+                unsigned few = 0;
+                if (lane == 0) few = a.n_total - *(volatile unsigned long long *)a.ended <= limit;
+                if (__shfl_sync(0xffffffffu, few, 0)) {
+                    if (live && team.l == 0) {
+                        store64<EN>(a.out, P, x);
+                        to[atomicAdd(n_to, 1ull)] = (uint32_t)P.g;   // no more than `limit` paths are left
+                    }
+                    break;
+                }
+            }
             if (it % G == 0) s64::normals(P.seed, P.pid, x.k + (uint32_t)team.l, zs);
             const int j = (int)(it % G);
             const double z[3] = {team.get(zs[0], j), team.get(zs[1], j), team.get(zs[2], j)};
             step64<G, ISO, EN>(P, tab, team, z, live, x);
-            if (live && x.status != COSMICA_PATH_RUNNING) {
+            const bool end = live && x.status != COSMICA_PATH_RUNNING;
+            if (end) {
                 if (team.l == 0) {
                     store64<EN>(a.out, P, x);
                     my_steps += x.k;
                 }
                 live = false;
             }
+            const unsigned ends = __ballot_sync(0xffffffffu, end && team.l == 0);
+            if (hand_over && ends && lane == 0) atomicAdd(a.ended, (unsigned long long)__popc(ends));
         }
+    }
+    if (a.steps_total && my_steps) atomicAdd(a.steps_total, my_steps);
+}
+
+// One block of four warps for up to eight paths: team j of every warp holds path
+// j * gridDim.x + blockIdx.x (quad64.cuh).  Shared memory carries the state from warp 0, which
+// owns the paths, to the others.
+template <bool ISO, bool EN>
+__global__ void __launch_bounds__(128, 1) k_quad64(LaunchArgs a, const uint32_t *from, const unsigned long long *n_from)
+{
+    __shared__ s64::QuadShared S;
+    s64::load_table(S.tab);
+    const uint64_t n = from ? *n_from : a.n_total;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const int tm = (int)(lane >> 2);
+    const s64::Team<4> team{(int)(lane & 3u)};
+    unsigned long long my_steps = 0;
+    for (uint64_t first = blockIdx.x; first < n; first += (uint64_t)gridDim.x * s64::kQuadTeams) {
+        // a team without a path of its own follows the block's first one and writes nothing
+        uint64_t i = first + (uint64_t)tm * gridDim.x;
+        bool live = i < n;
+        if (!live) i = first;
+        Path64 P;
+        m64::State x;
+        if (!from) fresh64(a, i, P, x);
+        else stored64<EN>(a, from[i], P, x);
+        const uint32_t k0 = x.k;
+        auto draw = [&](uint32_t batch) {      // normals of steps k0 + 4 batch + (0 .. 3)
+            double z[3];
+            s64::normals(P.seed, P.pid, k0 + 4u * batch + (uint32_t)team.l, z);
+            for (int c = 0; c < 3; ++c) S.z[batch & 1u][tm][team.l][c] = z[c];
+        };
+        auto publish = [&](uint32_t it) {       // the state at the beginning of step `it`
+            if (team.l == 0) {
+                double *st = S.st[tm];
+                st[0] = x.r; st[1] = x.th; st[2] = x.ph; st[3] = x.lnP; st[4] = x.T;
+                S.live[it & 1u][tm] = live;
+            }
+        };
+        if (warp == 0) publish(0);
+        if (warp == 3) draw(0);
+        s64::meet(3, 128);
+        for (uint32_t it = 0;; ++it) {
+            int any = 0;
+            for (int j = 0; j < s64::kQuadTeams; ++j) any |= S.live[it & 1u][j];
+            if (!any) break;       // the same answer in all four warps
+            const double *st = S.st[tm];
+            const double *z = S.z[(it >> 2) & 1u][tm][it & 3u];
+            if (warp == 0) {
+                if constexpr (ISO) s64::quad_isotropic<EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, S, team, tm, z, live, x);
+                else s64::quad_chain<EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, S, team, tm, live, x);
+                if (live && x.status != COSMICA_PATH_RUNNING) {
+                    if (team.l == 0) {
+                        store64<EN>(a.out, P, x);
+                        my_steps += x.k;
+                    }
+                    live = false;
+                }
+                publish(it + 1u);
+            } else if (warp == 3) {
+                double g = 1.0, dg = 0.0;
+                if (P.p->R_ts > 0.0) s64::quad_shock(*P.p, st[0], g, dg);
+                if (team.l == 0) {
+                    S.shock[tm][0] = g;
+                    S.shock[tm][1] = dg;
+                }
+                s64::meet(2, 64);
+                if ((it & 3u) == 0u) draw((it >> 2) + 1u);
+                if constexpr (!ISO) s64::meet(3, 128);
+            } else if constexpr (!ISO) {
+                if (warp == 1) s64::quad_drift(*P.p, P.sp, S, team, tm, st[0], st[1], st[3]);
+                else s64::quad_tensor<EN>(*P.p, P.sp, S, team, tm, st[0], st[1], st[3], st[4], z);
+                s64::meet(3, 128);
+            }
+            s64::meet(3, 128);
+        }
+        s64::meet(3, 128);     // before the next round's paths are published
     }
     if (a.steps_total && my_steps) atomicAdd(a.steps_total, my_steps);
 }
@@ -436,26 +538,37 @@ cudaError_t launch_derive(DevParams *prm, uint32_t n, cudaStream_t s)
 template <int ISO, bool EN>
 static cudaError_t launch64(const LaunchArgs &a, int sms, cudaStream_t s)
 {
-    const uint64_t few = (uint64_t)std::min(a.list_cap, fp64_list_entries(sms));
     const unsigned n_sms = (unsigned)sms;
-    if (a.n_total <= 8ull * n_sms) {
-        // at most two paths per scheduler
-        const unsigned grid = (unsigned)std::min<uint64_t>(n_sms, (a.n_total + 3) / 4);
-        k_finish64<16, ISO, EN><<<grid, 128, 0, s>>>(a, true);
-    } else if (a.n_total <= 32ull * n_sms) {
-        k_finish64<4, ISO, EN><<<n_sms, 128, 0, s>>>(a, true);
-    } else {
-        // the list holds 32-bit indices
-        const uint32_t limit = a.n_total <= 0xFFFFFFFFull ? (uint32_t)few : 0u;
+    const uint64_t n = a.n_total, teams = 32ull * n_sms, quads = ISO == 2 ? 0 : 8ull * n_sms;
+    // the lists hold 32-bit indices
+    const uint32_t cap = n <= 0xFFFFFFFFull ? a.list_cap : 0u;
+    const uint32_t *from = nullptr;
+    const unsigned long long *n_from = nullptr;
+    if (n > teams) {
         // a second warp per scheduler fills the gaps between FP64 instructions, but halves the speed
         // of a path: taken when the queue keeps both busy for long
-        const unsigned per_sm = a.n_total >= 1024ull * n_sms ? 2 : 1;
+        const unsigned per_sm = n >= 1024ull * n_sms ? 2 : 1;
+        const uint32_t limit = (uint32_t)std::min<uint64_t>(teams, cap);
         k_propagate64<ISO, EN><<<n_sms * per_sm, 128, 0, s>>>(a, limit);
         note_launch();
         if (!limit) return cudaGetLastError();
-        k_finish64<4, ISO, EN><<<n_sms, 128, 0, s>>>(a, false);
+        from = a.list;
+        n_from = a.ended + 1;
     }
-    note_launch();
+    if (n > quads) {
+        const uint32_t limit = (uint32_t)std::min<uint64_t>(quads, cap);
+        uint32_t *to = a.list + (from ? cap : 0u);
+        unsigned long long *n_to = a.ended + (from ? 3 : 1);
+        k_finish64<4, ISO, EN><<<n_sms, 128, 0, s>>>(a, from, n_from, to, n_to, limit);
+        note_launch();
+        if (!limit) return cudaGetLastError();
+        from = to;
+        n_from = n_to;
+    }
+    if constexpr (ISO != 2) {
+        k_quad64<ISO == 1, EN><<<(unsigned)std::min<uint64_t>(n_sms, n), 128, 0, s>>>(a, from, n_from);
+        note_launch();
+    }
     return cudaGetLastError();
 }
 

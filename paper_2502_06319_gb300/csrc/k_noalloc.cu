@@ -215,10 +215,10 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
     if (e == cudaSuccess) e = launch_f32_table(d_prm, 1, d_f32, s);
     if (e != cudaSuccess) return cuda_fail(e, "cosmica_propagate_noalloc set-up");
 
-    // paths handed from kernel to kernel: the FP64 path reads no FP32 table and takes that region for
-    // its list, the mixed paths put theirs behind the call's items
+    // paths handed from kernel to kernel (two lists): the FP64 path reads no FP32 table and takes that
+    // region for them, the mixed paths put theirs behind the call's items
     uint32_t *list = (uint32_t *)d_f32;
-    uint32_t list_cap = (uint32_t)(f32_table_floats(1) * sizeof(float) / sizeof(uint32_t));
+    uint32_t list_cap = (uint32_t)(f32_table_floats(1) * sizeof(float) / sizeof(uint32_t) / 2);
     if (params->precision != COSMICA_PREC_FP64) {
         list = (uint32_t *)(d_items + n_energies);
         list_cap = (uint32_t)((kMaxE - n_energies) * sizeof(DevItem) / sizeof(uint32_t) / 2);

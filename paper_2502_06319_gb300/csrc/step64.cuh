@@ -25,7 +25,7 @@
 // the active lanes, so a launch with fewer paths than lanes spreads each path's independent
 // operations over G lanes -- polynomials, groups of up to four quotients, reciprocals or
 // square roots, and the normals of G consecutive steps -- and exchanges results by shuffles
-// (a few clocks): about 430 slots a step for G = 4, 400 for G = 16.  Every lane of a team
+// (a few clocks): about 480 slots a step for G = 4.  Every lane of a team
 // holds the whole state, and all 32 lanes of the warp execute every shuffle.
 //
 // Include only from translation units built with -fmad=false.
@@ -369,6 +369,30 @@ __device__ __noinline__ m64::State plain_step(const DevParams &p, const DevSpeci
     return x;
 }
 
+// reflection at r_in and the angles' ranges, by definition
+__device__ __forceinline__ void into_range(const DevParams &p, m64::State &o)
+{
+    if (o.r < p.r_in) o.r = 2.0 * p.r_in - o.r;
+    const double t = o.th - kTwoPi * floor(o.th / kTwoPi);
+    if (t > kPi) {
+        o.th = kTwoPi - t;
+        o.ph = o.ph + kPi;
+    } else {
+        o.th = t;
+    }
+    // floor(ph / 2 pi) is -1 and 1 on [-2 pi, 0) and [2 pi, 4 pi)
+    if (o.ph < 0.0 && o.ph >= -kTwoPi) o.ph = o.ph + kTwoPi;
+    else if (o.ph >= kTwoPi && o.ph < 2.0 * kTwoPi) o.ph = o.ph - kTwoPi;
+    else o.ph = o.ph - kTwoPi * floor(o.ph / kTwoPi);
+}
+
+template <bool EN>
+__device__ __forceinline__ bool finite_state(const m64::State &o)
+{
+    return (!EN | f64bits::is_finite(bits(o.T))) & f64bits::is_finite(bits(o.r)) & f64bits::is_finite(bits(o.th)) &
+           f64bits::is_finite(bits(o.ph)) & f64bits::is_finite(bits(o.lnP)) & f64bits::is_finite(bits(o.s));
+}
+
 // One step of x, m64::em_step's values.  ISO: the spherically symmetric model; EN: the energy
 // form; no shells, not squashed.  z: the step's normals.  Team lanes hold equal states and
 // must all call (shuffles); live = false leaves the state as it was.
@@ -708,27 +732,14 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
     // one rarely taken branch for the reflection and the angles' ranges
     if (f64bits::less(bits(o.r), bits(p.r_in)) | f64bits::outside_closed(bits(o.th), f64bits::kPiBits) |
         f64bits::outside_half_open(bits(o.ph), f64bits::kTwoPiBits)) {
-        if (o.r < p.r_in) o.r = 2.0 * p.r_in - o.r;
-        const double t = o.th - kTwoPi * floor(o.th / kTwoPi);
-        if (t > kPi) {
-            o.th = kTwoPi - t;
-            o.ph = o.ph + kPi;
-        } else {
-            o.th = t;
-        }
-        // floor(ph / 2 pi) is -1 and 1 on [-2 pi, 0) and [2 pi, 4 pi)
-        if (o.ph < 0.0 && o.ph >= -kTwoPi) o.ph = o.ph + kTwoPi;
-        else if (o.ph >= kTwoPi && o.ph < 2.0 * kTwoPi) o.ph = o.ph - kTwoPi;
-        else o.ph = o.ph - kTwoPi * floor(o.ph / kTwoPi);
+        into_range(p, o);
     }
     o.s = x.s + dt;
     o.k = x.k + 1u;
     o.r_old = r;
     o.status = !lt(o.r, p.R_out) ? COSMICA_PATH_EXIT : (o.k >= max_steps ? COSMICA_PATH_STEP_LIMIT : COSMICA_PATH_RUNNING);
-    const bool fin = (!EN | f64bits::is_finite(bits(o.T))) & f64bits::is_finite(bits(o.r)) & f64bits::is_finite(bits(o.th)) & f64bits::is_finite(bits(o.ph)) &
-                     f64bits::is_finite(bits(o.lnP)) & f64bits::is_finite(bits(o.s));
     if (live) {
-        if (fin & !odd_range) x = o;
+        if (finite_state<EN>(o) & !odd_range) x = o;
         else x = plain_step(p, dsp, seed, pid, x);
     }
 }

@@ -1,5 +1,5 @@
 """The FP64 path's kernels against the oracle, bit for bit: sizes on both sides of every switch between them
-(16 or 4 lanes a path, a lane a path with the queue, the hand-over of the last paths), the models each form of
+(four warps or four lanes a path, a lane a path with the queue, the hand-overs of the last paths), the models each form of
 the step covers, starts that leave its range, and batches that mix isotropic and anisotropic sets."""
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ from paper_2502_06319_gb300 import workloads as W
 from tests.gpu_util import gpu_run, torch
 
 pytestmark = pytest.mark.gpu
-SM = 152
+SM = 152        # 8 and 32 paths per SM are the switches between kernels
 
 MODELS = {
     "isotropic": dict(W.config0().params),
@@ -36,7 +36,7 @@ def same(got, ref, with_lw=False):
 @pytest.mark.parametrize("form", [0, 1])
 @pytest.mark.parametrize("model", list(MODELS))
 def test_models(orc, model, form):
-    """A few paths to their end (teams of 16), and many for some steps (a lane a path, teams of 4)."""
+    """A few paths to their end (four warps), and many for some steps (a lane a path, teams of four lanes)."""
     p = dict(MODELS[model], formulation=float(form))
     for n, T, steps in (([3, 2], [5.0, 60.0], 1e8), ([5000, 2001], [0.3, 20.0], 150), ([1500], [2.0], 150)):
         job = W.Job(dict(p, max_steps=steps), W.HELIUM4 if form else W.PROTON, T, n, seed=11)
