@@ -79,11 +79,12 @@ __device__ __forceinline__ void take(const LaunchArgs &a, const MixedStage &st, 
 }
 
 // One Euler-Maruyama step (Eq. 3, Eq. 6) with the normals z0, z1, z2 of step L.k, which become
-// those of the next step: the increments are added and nothing else is looked at.  One block
-// without branches (in the full-model variant), so that the compiler interleaves the
-// generator with the coefficients.
+// those of the next step: the increments are added and nothing else is done.  True when the new
+// state has to be looked at (a boundary, an end of the path, or nearly so).  One block without
+// branches (in the full-model variant), so that the compiler interleaves the generator with the
+// coefficients.
 template <int ACC, bool EN, int EXT, bool FULL>
-__device__ __forceinline__ void advance(const float *params, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en, float &z0,
+__device__ __forceinline__ bool advance(const float *params, Lane &L, Acc<ACC> &x, EnergyAcc<ACC, EN> &en, float &z0,
                                         float &z1, float &z2)
 {
     m32::Drift c;
@@ -105,12 +106,14 @@ __device__ __forceinline__ void advance(const float *params, Lane &L, Acc<ACC> &
         const float T = en.fT();
         const float alpha = __fdividef(T + 2.0f * en.m0, T + en.m0);
         en.add(c.dlnP * alpha * T * c.dt, c.dlnP * fmaf(c.beta, c.beta, 1.0f) * c.dt);
-        x.template add<false>(dr, dth, dph, 0.0f, c.dt);
-    } else {
-        x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
     }
+    const bool squashed = m32::is_squashed<EXT>(q);
+    bool calm = x.template add<!EN>(fr, fth, fph, dr, dth, dph, EN ? 0.0f : c.dlnP * c.dt, c.dt, P32F(q, r_in), !squashed);
     L.k += 1u;
+    calm &= L.k < L.max_steps;
+    if (squashed) calm &= !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
     m32::normals(L.seed, L.pid, L.k, z0, z1, z2);
+    return !calm;
 }
 
 // whether the state after a step needs settle(): a boundary other than the longitude's, an end of
@@ -227,12 +230,11 @@ __global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedS
         }
         bool see;
         while (true) {
-            advance<ACC, EN, EXT, FULL>(L.q, L, x, en, z0, z1, z2);
-            see = active && needs_settling<ACC, EXT>(L.q, L, x);
-            const bool wrap = active && x.phi_out();
+            const bool look = advance<ACC, EN, EXT, FULL>(L.q, L, x, en, z0, z1, z2);
             --room;
-            if (!__any_sync(0xffffffffu, see || wrap || room == 0)) continue;
-            if (wrap && !see) x.wrap_near();
+            if (!__any_sync(0xffffffffu, (active && look) || room == 0)) continue;
+            see = active && look && needs_settling<ACC, EXT>(L.q, L, x);
+            if (active && look && !see && x.phi_out()) x.wrap_near();
             if (__any_sync(0xffffffffu, see || room == 0)) break;
         }
         const bool end = see && settle<ACC, EN, EXT>(a, L, x, en, my_steps);

@@ -167,17 +167,18 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
             const float dr = fmaf(c.Ar_tot, c.dt, c.l00 * z0 * sdt);
             const float dth = fmaf(c.dth_drift, c.dt, c.l11 * z1 * sdt * c.inv_r);
             const float dph = fmaf(c.dph_drift, c.dt, fmaf(c.l20, z0, c.l22 * z2) * sdt * c.inv_rs);
-            x.template add<true>(dr, dth, dph, c.dlnP * c.dt, c.dt);
-            S.L.k += 1u;
-            m32::normals(S.L.seed, S.L.pid, S.L.k, z0, z1, z2);
             const bool squashed = m32::is_squashed<EXT>(q);
-            bool calm = x.calm(P32F(q, r_in), !squashed) & (S.L.k < S.L.max_steps);
+            bool calm = x.template add<true>(fr, fth, fph, dr, dth, dph, c.dlnP * c.dt, c.dt, P32F(q, r_in), !squashed);
+            S.L.k += 1u;
+            calm &= S.L.k < S.L.max_steps;
             if (squashed) calm &= !m32::outside_squashed(q, x.fr(), x.fth(), x.fph());
-            see = active && !calm;
-            const bool wrap = active && x.phi_out();
+            m32::normals(S.L.seed, S.L.pid, S.L.k, z0, z1, z2);
             ++used;
-            if (!__any_sync(0xffffffffu, see || wrap || used == a.budget)) continue;
-            if (wrap && !see) x.wrap_near();
+            const bool look = active && !calm;
+            if (!__any_sync(0xffffffffu, look || used == a.budget)) continue;
+            see = look && (!x.calm(P32F(q, r_in), !squashed) || S.L.k >= S.L.max_steps ||
+                           (squashed && m32::outside_squashed(q, x.fr(), x.fth(), x.fph())));
+            if (look && !see && x.phi_out()) x.wrap_near();
             if (__any_sync(0xffffffffu, see || used == a.budget)) break;
         }
 

@@ -61,14 +61,18 @@ struct Acc<COSMICA_PREC_MIXED> {
         fr = r.hi; fth = th.hi; fph = ph.hi; flnP = lnP.hi;
         sin_th = m32::sin_from_pole_distance(pole_distance());
     }
-    // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone)
+    // Adds a step's increments (to the state whose view was fr, fth, fph); true when nothing has to
+    // be looked at: no boundary, end or non-finite value is near.
+    // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone);
+    // sphere: the outer boundary is r = R_out (a squashed one is tested by its own function)
     template <bool P>
-    __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
+    __device__ bool add(float, float, float, float dr, float dth, float dph, float dlnP, float dt, float r_in, bool sphere)
     {
         m32::ff_add2(r, th, dr, dth);
         if (P) m32::ff_add2(ph, lnP, dph, dlnP);
         else m32::ff_add(ph, dph);
         m32::ff_add(s, dt);
+        return calm(r_in, sphere) & !phi_out();
     }
     // reflect at r_in, fold theta at the poles, wrap phi; all rare branches
     __device__ void boundaries(float r_in)
@@ -104,13 +108,12 @@ struct Acc<COSMICA_PREC_MIXED> {
     // no boundary but the longitude's, no end and no non-finite value is anywhere near: false
     // for every state that the rest of boundaries(), exited() or finite() would act on, and for
     // a few others
-    // (sphere: the outer boundary is r = R_out; a squashed one is tested by its own function)
     __device__ bool calm(float r_in, bool sphere) const
     {
         return (r.hi >= r_in) & (!sphere | (r.hi < Rout.hi)) & (__float_as_uint(th.hi) < __float_as_uint(m32::kPiF)) &
                (ph.hi > -6.28f) & (ph.hi < 12.56f) & isfinite(lnP.hi + s.hi);
     }
-    bool __device__ phi_out() const { return !(__float_as_uint(ph.hi) < __float_as_uint(m32::kTwoPiF)); }
+    __device__ bool phi_out() const { return !(__float_as_uint(ph.hi) < __float_as_uint(m32::kTwoPiF)); }
     // wrap_phi() for -6.28 < ph < 12.56, where floor(ph / 2 pi) is -1, 0 or 1.  Paths start at one
     // longitude, often 0, and cross it again and again at first (one step in ten of a warp over
     // the paths' lives), so only the three FP64 sums of the definition are left.
@@ -137,14 +140,18 @@ struct Acc<COSMICA_PREC_MIXED> {
 // FP64 accumulation of FP32 increments.
 // The FP64 pipe takes 64 clocks per warp instruction and scheduler, so only the sums stay on it;
 // conversions, comparisons and the finiteness test run on the bits (f64bits.h).  The results
-// are the same bits.  Measured: 4 heliospheres x 3 species x 30 energies, 1.4e5 paths 738 -> 328 ms;
-// one squashed heliosphere 316 -> 175 ms.
+// are the same bits.  Measured: 1.4e5 paths of 4 heliospheres 738 -> 328 ms by the integer
+// forms, 781 -> 181 ms with the step as one block whose vote does not wait for the sums (a lone
+// path's step 2.16 -> 0.53 us).
 template <>
 struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     double r, th, ph, lnP, s, Rout, r_in;
+    float r_lo, r_hi;      // a little inside (r_in, R_out), see add()
     __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in_f)
     {
         r = r0; th = th0; ph = ph0; lnP = lnP0; s = 0.0; Rout = R_out; r_in = (double)r_in_f;
+        r_lo = r_in_f * 1.000001f;
+        r_hi = (float)R_out * 0.999999f;
     }
     __device__ float fr() const { return narrow64(r); }
     __device__ float fth() const { return narrow64(th); }
@@ -161,13 +168,20 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
         flnP = narrow64(lnP);
         sin_th = m32::sin_from_pole_distance(north ? fth : f64bits::pi_minus(units));   // of the nearer pole's distance
     }
-    // P: the form accumulates lnP (the energy form integrates T instead and leaves lnP alone)
+    // As in the compensated state.  The FP64 sums take 64 clocks each, one after the other, so the
+    // step's vote does not wait for them: it looks at the FP32 sums, whose error (two roundings,
+    // under 2.4e-7 of r and of 2 pi) is far inside the margins, and the sums' finiteness follows
+    // from that of the increments.  theta first: the next step's longest chain starts from it.
     template <bool P>
-    __device__ void add(float dr, float dth, float dph, float dlnP, float dt)
+    __device__ bool add(float fr, float fth, float fph, float dr, float dth, float dph, float dlnP, float dt, float, bool sphere)
     {
-        r += widen64(dr); th += widen64(dth); ph += widen64(dph);
+        const float nr = fr + dr, nth = fth + dth, nph = fph + dph;
+        const bool still = (nr > r_lo) & (!sphere | (nr < r_hi)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
+                           (nph < 6.28317f) & isfinite(dlnP + dt);
+        th += widen64(dth); r += widen64(dr);
         if (P) lnP += widen64(dlnP);
-        s += widen64(dt);
+        ph += widen64(dph); s += widen64(dt);
+        return still;
     }
     __device__ void boundaries(float)
     {
@@ -191,7 +205,7 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
                (__double2hiint(ph) < 0x40291EB8) & ((uint32_t)__double2hiint(ph) < 0xC0191EB8u) &
                f64bits::is_finite(bits64(lnP)) & f64bits::is_finite(bits64(s));
     }
-    bool __device__ phi_out() const { return f64bits::outside_half_open(bits64(ph), f64bits::kTwoPiBits); }
+    __device__ bool phi_out() const { return f64bits::outside_half_open(bits64(ph), f64bits::kTwoPiBits); }
     __device__ void wrap_near()
     {
         ph += __double2hiint(ph) < 0 ? kTwoPi : (f64bits::less(bits64(ph), f64bits::kTwoPiBits) ? 0.0 : -kTwoPi);
