@@ -359,12 +359,12 @@ int num_sms()
     return n;
 }
 
-// Blocks of 128 (warps per scheduler) of an untuned launch.  More of them raise the rate (4.9, 7.0,
-// 8.0 and 8.3e10 steps/s with 1 to 4 in a long batch), fewer step each path faster (0.36, 0.5, 0.7
-// and 0.9 us a step), and a launch waits for its slowest paths, some ten times the mean.  Measured
-// in paths per lane of one layer (one warp per scheduler), ms with 1 / 2 / 3 / 4 layers:
-// 1.5: 36 / 43 / 49 / 50, 3: 47 / 52 / 58 / 60, 8: 55 / 51 / 55 / 59, 15: 73 / 67 / 71 / 70,
-// 31: 139 / 102 / 96 / 102, 57 (FP64 sums): 1212 / 782 / 666 / 637.
+// Blocks of 128 (warps per scheduler) of an untuned launch.  More of them raise the rate, fewer
+// step each path faster (0.3 us a step alone, 0.9 us with four), and a launch waits for its
+// slowest paths, some ten times the mean.  Measured in paths per lane of one layer (one warp per
+// scheduler), ms with 1 / 2 / 3 / 4 layers: 1.5: 36 / 43 / 49 / 50, 3: 47 / 52 / 58 / 60,
+// 8: 55 / 51 / 55 / 59, 15: 73 / 67 / 71 / 70, 31: 127 / 96 / 93 / 99,
+// 57 (FP64 sums): 1074 / 720 / 629 / 630.
 int untuned_layers(uint64_t n_total, int sms, int max_blocks)
 {
     const uint64_t layer = (uint64_t)sms * 128u;

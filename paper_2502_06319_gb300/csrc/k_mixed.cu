@@ -167,9 +167,9 @@ __device__ __forceinline__ bool settle(const LaunchArgs &a, Lane &L, Acc<ACC> &x
 // issue rate.  The loop being one block, the compiler interleaves the generator with the
 // coefficients and keeps the parameter set in registers (114-123 instead of 64, so 16 warps
 // per SM instead of 32).  Measured, against a loop that tested everything every step and drew the
-// normals after the tests: a lone path's step 0.68 -> 0.36 us, a warp's step with four warps per
-// scheduler 1.05 -> 0.93 us, 5.7e6 paths of 4 heliospheres 8.3e10 steps/s, one spectrum of 6e5
-// paths 141 -> 99 ms, 1.8e6 paths of 16 heliospheres 870 -> 694 ms.
+// normals after the tests: a lone path's step 0.68 -> 0.30 us (375 instructions), a warp's step
+// with four warps per scheduler 1.05 -> 0.87 us, one spectrum of 6e5 paths 143 -> 93 ms, 1.8e6
+// paths of 16 heliospheres 869 -> 657 ms (8.5e10 steps/s).
 template <int ACC, bool EN, int EXT, bool FULL>
 __global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedStage st)
 {
@@ -299,7 +299,7 @@ int mixed_max_blocks_per_sm(MixedVariant v, unsigned block)
 
 // A launch of w warps per scheduler whose queue is empty runs on with ever emptier warps, each
 // step as slow as the w warps make it; handing the last paths to w - 1 full warps per scheduler,
-// and so on down to one, steps them at the speed of those (one warp: 0.36 us a step, four: 0.9).
+// and so on down to one, steps them at the speed of those (one warp: 0.3 us a step, four: 0.9).
 cudaError_t launch_propagate_mixed(const LaunchArgs &a, MixedVariant v, PersistentShape shape, int sms, cudaStream_t s)
 {
     if (a.n_total == 0) return cudaSuccess;

@@ -38,14 +38,16 @@ template <>
 __device__ __forceinline__ void save(const Acc<COSMICA_PREC_MIXED> &x, Suspended &s)
 {
     s.f[0] = x.r.hi; s.f[1] = x.r.lo; s.f[2] = x.th.hi; s.f[3] = x.th.lo; s.f[4] = x.ph.hi;
-    s.f[5] = x.ph.lo; s.f[6] = x.lnP.hi; s.f[7] = x.lnP.lo; s.f[8] = x.s.hi; s.f[9] = x.s.lo;
+    const m32::FF P = x.Ps.first(), t = x.Ps.second();
+    s.f[5] = x.ph.lo; s.f[6] = P.hi; s.f[7] = P.lo; s.f[8] = t.hi; s.f[9] = t.lo;
 }
 template <>
 __device__ __forceinline__ void load(Acc<COSMICA_PREC_MIXED> &x, const Suspended &s, const DevParams &p)
 {
     x.init(p.r0, p.th0, p.ph0, 0.0, p.R_out, p.f.r_in);
     x.r.hi = s.f[0]; x.r.lo = s.f[1]; x.th.hi = s.f[2]; x.th.lo = s.f[3]; x.ph.hi = s.f[4];
-    x.ph.lo = s.f[5]; x.lnP.hi = s.f[6]; x.lnP.lo = s.f[7]; x.s.hi = s.f[8]; x.s.lo = s.f[9];
+    x.ph.lo = s.f[5];
+    x.Ps.set(m32::FF{s.f[6], s.f[7]}, m32::FF{s.f[8], s.f[9]});
 }
 template <>
 __device__ __forceinline__ void save(const Acc<COSMICA_PREC_MIXED_F64ACC> &x, Suspended &s)

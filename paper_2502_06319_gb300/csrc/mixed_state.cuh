@@ -30,7 +30,8 @@ struct Acc;
 // compensated FP32 state
 template <>
 struct Acc<COSMICA_PREC_MIXED> {
-    m32::FF r, th, ph, lnP, s;
+    m32::FF r, th, ph;
+    m32::FF2 Ps;   // lnP and s, the two that no boundary touches, as packed pairs
     m32::FF Rout;
     float r_in2;   // 2 r_in
     __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in)
@@ -38,8 +39,7 @@ struct Acc<COSMICA_PREC_MIXED> {
         r = m32::ff_from_double(r0);
         th = m32::ff_from_double(th0);
         ph = m32::ff_from_double(ph0);
-        lnP = m32::ff_from_double(lnP0);
-        s.hi = 0.0f; s.lo = 0.0f;
+        Ps.set(m32::ff_from_double(lnP0), m32::FF{0.0f, 0.0f});
         Rout = m32::ff_from_double(R_out);
         r_in2 = 2.0f * r_in;
     }
@@ -58,7 +58,7 @@ struct Acc<COSMICA_PREC_MIXED> {
     // r, theta, phi, lnP and sin(theta) as the step reads them
     __device__ void view(float &fr, float &fth, float &fph, float &flnP, float &sin_th) const
     {
-        fr = r.hi; fth = th.hi; fph = ph.hi; flnP = lnP.hi;
+        fr = r.hi; fth = th.hi; fph = ph.hi; flnP = Ps.first().hi;
         sin_th = m32::sin_from_pole_distance(pole_distance());
     }
     // Adds a step's increments (to the state whose view was fr, fth, fph); true when nothing has to
@@ -68,10 +68,10 @@ struct Acc<COSMICA_PREC_MIXED> {
     template <bool P>
     __device__ bool add(float, float, float, float dr, float dth, float dph, float dlnP, float dt, float r_in, bool sphere)
     {
-        m32::ff_add2(r, th, dr, dth);
-        if (P) m32::ff_add2(ph, lnP, dph, dlnP);
-        else m32::ff_add(ph, dph);
-        m32::ff_add(s, dt);
+        m32::ff_add(r, dr);
+        m32::ff_add(th, dth);
+        m32::ff_add(ph, dph);
+        m32::ff_add2(Ps, P ? dlnP : 0.0f, dt);
         return calm(r_in, sphere) & !phi_out();
     }
     // reflect at r_in, fold theta at the poles, wrap phi; all rare branches
@@ -111,7 +111,7 @@ struct Acc<COSMICA_PREC_MIXED> {
     __device__ bool calm(float r_in, bool sphere) const
     {
         return (r.hi >= r_in) & (!sphere | (r.hi < Rout.hi)) & (__float_as_uint(th.hi) < __float_as_uint(m32::kPiF)) &
-               (ph.hi > -6.28f) & (ph.hi < 12.56f) & isfinite(lnP.hi + s.hi);
+               (ph.hi > -6.28f) & (ph.hi < 12.56f) & isfinite(Ps.first().hi + Ps.second().hi);
     }
     __device__ bool phi_out() const { return !(__float_as_uint(ph.hi) < __float_as_uint(m32::kTwoPiF)); }
     // wrap_phi() for -6.28 < ph < 12.56, where floor(ph / 2 pi) is -1, 0 or 1.  Paths start at one
@@ -126,14 +126,14 @@ struct Acc<COSMICA_PREC_MIXED> {
         ph.lo = narrow64(p - widen64(ph.hi));
     }
     __device__ bool exited() const { return m32::ff_ge(r, Rout); }
-    __device__ bool finite() const { return isfinite(r.hi + th.hi + ph.hi + lnP.hi + s.hi); }
+    __device__ bool finite() const { return isfinite(r.hi + th.hi + ph.hi + Ps.first().hi + Ps.second().hi); }
     __device__ void write(const ExitPtrs &out, uint64_t g) const
     {
         out.r[g] = m32::ff_to_double(r);
         out.th[g] = m32::ff_to_double(th);
         out.ph[g] = m32::ff_to_double(ph);
-        out.lnP[g] = m32::ff_to_double(lnP);
-        out.s[g] = m32::ff_to_double(s);
+        out.lnP[g] = m32::ff_to_double(Ps.first());
+        out.s[g] = m32::ff_to_double(Ps.second());
     }
 };
 
@@ -278,24 +278,24 @@ template <bool EN>
 __device__ __forceinline__ void park(const ExitPtrs &o, uint64_t g, const Acc<COSMICA_PREC_MIXED> &x,
                                      const EnergyAcc<COSMICA_PREC_MIXED, EN> &en)
 {
-    o.r[g] = pair_bits(x.r); o.th[g] = pair_bits(x.th); o.ph[g] = pair_bits(x.ph); o.s[g] = pair_bits(x.s);
+    o.r[g] = pair_bits(x.r); o.th[g] = pair_bits(x.th); o.ph[g] = pair_bits(x.ph);
+    o.s[g] = pair_bits(x.Ps.second());
     if constexpr (EN) {
         o.lnP[g] = pair_bits(en.T);
         o.lw[g] = pair_bits(en.Lam);
     } else {
-        o.lnP[g] = pair_bits(x.lnP);
+        o.lnP[g] = pair_bits(x.Ps.first());
     }
 }
 template <bool EN>
 __device__ __forceinline__ void unpark(const ExitPtrs &o, uint64_t g, Acc<COSMICA_PREC_MIXED> &x,
                                        EnergyAcc<COSMICA_PREC_MIXED, EN> &en)
 {
-    x.r = from_pair_bits(o.r[g]); x.th = from_pair_bits(o.th[g]); x.ph = from_pair_bits(o.ph[g]); x.s = from_pair_bits(o.s[g]);
+    x.r = from_pair_bits(o.r[g]); x.th = from_pair_bits(o.th[g]); x.ph = from_pair_bits(o.ph[g]);
+    x.Ps.set(EN ? x.Ps.first() : from_pair_bits(o.lnP[g]), from_pair_bits(o.s[g]));
     if constexpr (EN) {
         en.T = from_pair_bits(o.lnP[g]);
         en.Lam = from_pair_bits(o.lw[g]);
-    } else {
-        x.lnP = from_pair_bits(o.lnP[g]);
     }
 }
 template <bool EN>

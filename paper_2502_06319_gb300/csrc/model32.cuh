@@ -34,10 +34,26 @@ constexpr float kTwoPiF = 6.28318530717958648f;
 constexpr float kInvTwoPiF = 0.159154943091895336f;
 constexpr float kSqrt2F = 1.41421356237309505f;
 
+// Factors of a power of two are exact in FP32, so they are folded into constants (here -2 log2 e,
+// -2 ln 2 below, 2/r in eval) without changing a result: eight multiplications a step fewer.
+__device__ __forceinline__ float pow2_approx(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float log2_approx(float x)
+{
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+constexpr float kLog2eF = 1.44269504088896341f, kLn2F = 0.69314718055994531f;
+
 // 1/(1 + e^{-2x}) = (1 + tanh x) / 2, safe for any finite x
 __device__ __forceinline__ float half_one_plus_tanh(float x)
 {
-    return __fdividef(1.0f, 1.0f + __expf(-2.0f * x));
+    return __fdividef(1.0f, 1.0f + pow2_approx(x * (-2.0f * kLog2eF)));
 }
 
 struct Drift {
@@ -166,8 +182,10 @@ __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float
     const float lat = kHalfPiF - th;
     const float sw = half_one_plus_tanh((fabsf(lat) - P32F(q, lat_f)) * P32F(q, inv_dlat));
     const float V = fmaf(P32F(q, dV), sw, P32F(q, Vs));
-    const float sgn_lat = (lat > 0.0f) ? -1.0f : ((lat < 0.0f) ? 1.0f : 0.0f);   // d|lat|/dth
-    const float dV = P32F(q, dV) * 2.0f * sw * (1.0f - sw) * P32F(q, inv_dlat) * sgn_lat;
+    // times d|lat|/dth: -1 north, +1 south, 0 on the equator
+    const float dV_abs = P32F(q, dV) * 2.0f * sw * (1.0f - sw) * P32F(q, inv_dlat);
+    const float dV_sgn = __uint_as_float(__float_as_uint(dV_abs) ^ (~__float_as_uint(lat) & 0x80000000u));
+    const float dV = lat != 0.0f ? dV_sgn : 0.0f;
     const float inv_V = __fdividef(1.0f, V);
 
     // Parker spiral
@@ -226,7 +244,8 @@ __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float
     if (shells) dKpar = fmaf(dK0 * beta * P, g, dKpar);
     const float c2s = fmaf(P32F(q, er), G2 * iq, iq);            // cos^2 + er sin^2
     const float iq2 = iq * iq;
-    const float dc2_dr = -2.0f * G2 * iq2 * inv_r;         // d cos^2 psi / dr
+    const float two_r = 2.0f * inv_r;
+    const float dc2_dr = -G2 * iq2 * two_r;                // d cos^2 psi / dr
     const float sc = Gam * iq;
     const float dsc_dr = Gam * (1.0f - G2) * iq2 * inv_r;
     const float Krr = Kpar * c2s;
@@ -237,7 +256,7 @@ __device__ __forceinline__ void eval(const P32<ST> &q, float M2, float sq, float
     const float dKrp = erm1 * fmaf(dKpar, sc, Kpar * dsc_dr);
 
     // Ito drift (1/sqrt g) d_j (sqrt g K^ij)
-    float Ar = fmaf(2.0f * Krr, inv_r, dKrr);
+    float Ar = fmaf(Krr, two_r, dKrr);
     float Ath = Ktt * cot * inv_r * inv_r;
     const float inv_rs = inv_r * inv_sn;
     float Aph = fmaf(Krp, inv_r, dKrp) * inv_rs;
@@ -356,8 +375,8 @@ __device__ __forceinline__ void normals(uint64_t seed, uint64_t pid, uint32_t k,
     const float u1 = uniform01(w.y);
     const float u2 = uniform01(w.z);
     const float u3 = uniform01(w.w);
-    const float rho0 = sqrtf(-2.0f * __logf(u0));
-    const float rho2 = sqrtf(-2.0f * __logf(u2));
+    const float rho0 = sqrtf(log2_approx(u0) * (-2.0f * kLn2F));
+    const float rho2 = sqrtf(log2_approx(u2) * (-2.0f * kLn2F));
     // angle 2 pi u - pi lies in (-pi, pi], where the SFU sin/cos are accurate;
     // cos(a - pi) = -cos a, sin(a - pi) = -sin a
     float s1, c1, s3, c3;
@@ -408,16 +427,40 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
     asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
     return v;
 }
-__device__ __forceinline__ void ff_add2(FF &a, FF &b, float da, float db)
+// (kept packed: taking pairs apart and putting them together costs the moves that packing saves)
+struct FF2 {
+    uint64_t hi, lo;
+    __device__ __forceinline__ FF first() const
+    {
+        FF a;
+        float unused;
+        unpk(hi, a.hi, unused);
+        unpk(lo, a.lo, unused);
+        return a;
+    }
+    __device__ __forceinline__ FF second() const
+    {
+        FF b;
+        float unused;
+        unpk(hi, unused, b.hi);
+        unpk(lo, unused, b.lo);
+        return b;
+    }
+    __device__ __forceinline__ void set(const FF &a, const FF &b)
+    {
+        hi = pk(a.hi, b.hi);
+        lo = pk(a.lo, b.lo);
+    }
+};
+__device__ __forceinline__ void ff_add2(FF2 &a, float d0, float d1)
 {
-    const uint64_t ah = pk(a.hi, b.hi), al = pk(a.lo, b.lo), d = pk(da, db);
-    const uint64_t s = add2(ah, d);
-    const uint64_t bb = sub2(s, ah);
-    const uint64_t err = add2(sub2(ah, sub2(s, bb)), sub2(d, bb));
-    const uint64_t lo = add2(al, err);
-    const uint64_t hi = add2(s, lo);
-    unpk(sub2(lo, sub2(hi, s)), a.lo, b.lo);
-    unpk(hi, a.hi, b.hi);
+    const uint64_t d = pk(d0, d1);
+    const uint64_t s = add2(a.hi, d);
+    const uint64_t bb = sub2(s, a.hi);
+    const uint64_t err = add2(sub2(a.hi, sub2(s, bb)), sub2(d, bb));
+    const uint64_t lo = add2(a.lo, err);
+    a.hi = add2(s, lo);
+    a.lo = sub2(lo, sub2(a.hi, s));
 }
 
 __device__ __forceinline__ void ff_add_ff(FF &a, float bh, float bl)
