@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(128) k_propagate_fp64(const DevParams *__restr
 // A launch that starts with so few paths starts there.  (A mixture of isotropic and other sets
 // stays with k_finish64.)
 // Measured against one thread per path with the plain step: a step of the full model 52 us, 29 in
-// k_propagate64 (a lane a path), 17.4 in k_finish64 (477 slots, the FP64 pipe 84 % busy), 10.4 in
-// k_quad64 (250 slots on its longest warp); 1e4 isotropic paths 86.8 -> 23.2 ms, 2.5e4 paths of the
+// k_propagate64 (a lane a path), 17.4 in k_finish64 (477 slots, the FP64 pipe 84 % busy), 10.1 in
+// k_quad64 (242 slots on its longest warp); 1e4 isotropic paths 86.8 -> 23.2 ms, 2.5e4 paths of the
 // full model 1385 -> 352 ms.  The paths are the same bits.
 struct Path64 {
     uint64_t g, pid, seed;
@@ -247,7 +247,7 @@ __device__ __forceinline__ void step64(const Path64 &P, const double *tab, s64::
     if constexpr (ISO == 2) {
         // teams of a warp may hold different models: all of them run each form that one of them needs
         // (its shuffles take the whole warp), and each keeps its own
-        const bool iso = P.p->isotropic != 0.0;
+        const bool iso = s64::on(P.p->isotropic);
         if (G == 1 ? iso : __any_sync(0xffffffffu, iso))
             s64::step<G, true, EN>(*P.p, *P.dsp, P.sp, P.seed, P.pid, P.max_steps, tab, team, z, live && iso, x);
         if (G == 1 ? !iso : __any_sync(0xffffffffu, !iso))
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(128, 1) k_quad64(LaunchArgs a, const uint32_t 
                 publish(it + 1u);
             } else if (warp == 3) {
                 double g = 1.0, dg = 0.0;
-                if (P.p->R_ts > 0.0) s64::quad_shock(*P.p, st[0], g, dg);
+                if (s64::positive(P.p->R_ts)) s64::quad_shock(*P.p, st[0], g, dg);
                 if (team.l == 0) {
                     S.shock[tm][0] = g;
                     S.shock[tm][1] = dg;

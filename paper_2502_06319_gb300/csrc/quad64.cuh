@@ -7,7 +7,7 @@
 // step; an exchange through shared memory costs about one slot.
 //
 //   warp 0  wind, sheet phase, sin/cos, atan, tanh of the sheet, drift, step length, update:
-//           the step's serial chain, 250 slots
+//           the step's serial chain, 242 slots
 //   warp 1  sheet width and its gradient, drift geometry, derivatives of the sheet's argument
 //   warp 2  tensor, Ito drift, Cholesky factor, noise
 //   warp 3  normals of the next four steps (one step per lane), termination shock
@@ -81,7 +81,7 @@ __device__ __forceinline__ Head quad_head(const DevParams &p, const Spc &sp, con
     o.dV = 0.0;
     if constexpr (DV) {
         o.dV = quot(d.hdV * (1.0 - t * t), d.dlat, d.r_dlat);
-        o.dV = (lat > 0.0) ? neg_if(o.dV, true) : ((lat < 0.0) ? o.dV : 0.0);
+        o.dV = toward_equator(o.dV, lat);
     }
     return o;
 }
@@ -203,7 +203,7 @@ __device__ __forceinline__ void quad_tensor(const DevParams &p, const Spc &sp, Q
     }
     const double dc2 = q[0], dsc = q[1];
     const double Kbase = p.K0 * H.beta * H.P;
-    const bool shock = p.R_ts > 0.0;
+    const bool shock = positive(p.R_ts);
     meet(2, 64);
     const double g = S.shock[tm][0], dg = S.shock[tm][1];
     const double Kpar = shock ? Kbase * g : Kbase;
@@ -291,7 +291,7 @@ __device__ __forceinline__ void quad_chain(const DevParams &p, const DevSpecies 
         const double b = exp_in(scale2<1>(uabs)) + 1.0;
         t = 1.0 - quot(2.0, b, recip(b));
     }
-    const bool hcs = p.hcs_on != 0.0, drift = p.drift_on != 0.0;
+    const bool hcs = on(p.hcs_on), drift = on(p.drift_on);
     const double h = hcs ? neg_if(t, __double2hiint(u) < 0) : 1.0;
     const double w = hcs ? 1.0 - h * h : 0.0;
     meet(3, 128);
@@ -311,7 +311,7 @@ __device__ __forceinline__ void quad_chain(const DevParams &p, const DevSpecies 
                      b[4] = {r, r, r, 1.0}, yy[4] = {H.y_r, H.y_r, H.y_r, 1.0};
         team.quot4(n, b, yy, q);
     }
-    const bool s = sp.negative != (p.polarity < 0.0);
+    const bool s = sp.negative != (__double2hiint(p.polarity) < 0);
     const double vd0 = drift ? neg_if(q[0], s) : 0.0, vd1 = drift ? neg_if(q[1], s) : 0.0, vd2 = drift ? neg_if(q[2], s) : 0.0;
 
     // step length
@@ -322,11 +322,11 @@ __device__ __forceinline__ void quad_chain(const DevParams &p, const DevSpecies 
         const double n[4] = {te[7], te[8], go[9], 0.0}, b[4] = {den, te[9], te[11], 1.0}, yy[4] = {recip(den), te[10], te[12], 1.0};
         team.quot4(n, b, yy, q);
     }
-    if (te[7] < dt * den) dt = q[0];
-    if (q[1] < dt) dt = q[1];
-    if (hcs && drift && q[2] < dt) dt = q[2];
-    if (dt < p.dt_min) dt = p.dt_min;
-    if (p.dt_fixed > 0.0) dt = p.dt_fixed;
+    if (lt(te[7], dt * den)) dt = q[0];
+    if (lt(q[1], dt)) dt = q[1];
+    if (hcs && drift && lt(q[2], dt)) dt = q[2];
+    if (lt(dt, p.dt_min)) dt = p.dt_min;
+    if (positive(p.dt_fixed)) dt = p.dt_fixed;
     const double sdt = sqrt(dt);
 
     // update: lanes 0 to 3 take r, theta, phi, ln P
@@ -379,7 +379,7 @@ __device__ __forceinline__ void quad_isotropic(const DevParams &p, const DevSpec
     const double beta = q[0], cot = q[1], dlnP = q[2];
     const double Kbase = p.K0 * beta * P;
     meet(2, 64);
-    const bool shock = p.R_ts > 0.0;
+    const bool shock = positive(p.R_ts);
     const double K = shock ? Kbase * S.shock[tm][0] : Kbase;
     const double dK = shock ? Kbase * S.shock[tm][1] : 0.0;
     {
@@ -389,16 +389,16 @@ __device__ __forceinline__ void quad_isotropic(const DevParams &p, const DevSpec
     const double Ar_tot = (dK + q[0]) - V, Ath = q[1];
     const double l = sqrt(scale2<1>(K));
     double dt = p.dt_fixed, sdt = d.sdt_fixed;
-    const bool fixed = p.dt_fixed > 0.0;
+    const bool fixed = positive(p.dt_fixed);
     if (team.any(!fixed)) {
         double a = p.dt_max;
         const double num = d.eps_adv2 * K, den = Ar_tot * Ar_tot, n2 = p.eps_diff * r * r;
         team.recip4(den, K, 1.0, 1.0, y2);
         const double n[4] = {num, n2, 0.0, 0.0}, b[4] = {den, K, 1.0, 1.0}, yy[4] = {y2[0], y2[1], 1.0, 1.0};
         team.quot4(n, b, yy, q);
-        if (num < a * den) a = q[0];
-        if (q[1] < a) a = q[1];
-        if (a < p.dt_min) a = p.dt_min;
+        if (lt(num, a * den)) a = q[0];
+        if (lt(q[1], a)) a = q[1];
+        if (lt(a, p.dt_min)) a = p.dt_min;
         if (!fixed) {
             dt = a;
             sdt = sqrt(a);

@@ -42,6 +42,9 @@ namespace s64 {
 __device__ __forceinline__ uint64_t bits(double x) { return (uint64_t)__double_as_longlong(x); }
 __device__ __forceinline__ double from_bits(uint64_t b) { return __longlong_as_double((long long)b); }
 __device__ __forceinline__ bool lt(double a, double b) { return (int64_t)bits(a) < (int64_t)bits(b); }   // b >= 0, no NaN
+// x > 0 for any x but a NaN, whose answer is no; a switch held as 0.0 or 1.0
+__device__ __forceinline__ bool positive(double x) { return (int64_t)bits(x) > 0 && (int64_t)bits(x) <= 0x7FF0000000000000ll; }
+__device__ __forceinline__ bool on(double x) { return __double2hiint(x) != 0; }
 // x 2^E for normal results; zeros stay zeros
 template <int E>
 __device__ __forceinline__ double scale2(double x)
@@ -393,6 +396,12 @@ __device__ __forceinline__ bool finite_state(const m64::State &o)
            f64bits::is_finite(bits(o.ph)) & f64bits::is_finite(bits(o.lnP)) & f64bits::is_finite(bits(o.s));
 }
 
+// |dV/dth| with the sign of d|lat|/dth, zero on the equator
+__device__ __forceinline__ double toward_equator(double dV, double lat)
+{
+    return (bits(lat) << 1) == 0 ? 0.0 : neg_if(dV, __double2hiint(lat) >= 0);
+}
+
 // One step of x, m64::em_step's values.  ISO: the spherically symmetric model; EN: the energy
 // form; no shells, not squashed.  z: the step's normals.  Team lanes hold equal states and
 // must all call (shuffles); live = false leaves the state as it was.
@@ -403,7 +412,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
 {
     const F64Params &d = p.d;
     const double r = x.r, th = x.th;
-    const bool shock = p.R_ts > 0.0;
+    const bool shock = positive(p.R_ts);
     double y4[4], q4[4], q5[4], q6[4];
 
     // shock and wind arguments
@@ -459,7 +468,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
         const double t = neg_if(wnear ? 1.0 - q4[2] : 1.0, __double2hiint(wa) < 0);
         V = d.Vs + d.hdV * (1.0 + t);
         dV = quot(d.hdV * (1.0 - t * t), d.dlat, d.r_dlat);
-        dV = (lat > 0.0) ? neg_if(dV, true) : ((lat < 0.0) ? dV : 0.0);
+        dV = toward_equator(dV, lat);
     }
     // termination shock
     double g = 1.0, dg = 0.0;
@@ -480,6 +489,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
 
     double K00, K11, K22, K02 = 0.0, Ar, Ath, Aph = 0.0, l00, l11, l22, l20 = 0.0, dlnP;
     double vd0 = 0.0, vd1 = 0.0, vd2 = 0.0, delta = 0.0, y_rs;
+    bool sheet = false;          // its width limits the step
     if constexpr (ISO) {
         K00 = K11 = K22 = Kpar;
         team.recip4(rr, r3, rs, 1.0, y4);
@@ -511,7 +521,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
         const double phs = x.ph + q4[1];
         odd_range |= !lt(phs, 1e6);
         double sphs = 0.0, cphs = 0.0;
-        const bool hcs = p.hcs_on != 0.0, any_hcs = team.any(hcs);
+        const bool hcs = on(p.hcs_on), any_hcs = team.any(hcs);
         if (any_hcs) {
             if constexpr (G == 1) sincos_in(phs, sphs, cphs);
             else team.sincos(tab, phs, sphs, cphs);
@@ -524,7 +534,8 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
         }
         const double c2 = q4[0], s2 = q4[1], sc = q4[2], dGam_dr = q4[3];
         const double m1 = 1.0 - G2, r2G = rr * Gam;
-        const bool drift = p.drift_on != 0.0;
+        const bool drift = on(p.drift_on);
+        sheet = hcs && drift;
         {
             const double n[4] = {neg_if(scale2<1>(Gam) * dGam_dr, true), dGam_dr * m1, neg_if(scale2<1>(r2G * dGam_dth), true),
                                  r * Gam * (3.0 + G2)},
@@ -651,7 +662,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
                 team.quot4(n, b, y, q4);
             }
             if (drift) {
-                const bool s = sp.negative != (p.polarity < 0.0);
+                const bool s = sp.negative != (__double2hiint(p.polarity) < 0);
                 vd0 = neg_if(q4[0], s);
                 vd1 = neg_if(q4[1], s);
                 vd2 = neg_if(q4[2], s);
@@ -661,34 +672,33 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
 
     // step length
     const double Ar_tot = Ar - V - vd0;
-    const bool fixed = p.dt_fixed > 0.0;
+    const bool fixed = positive(p.dt_fixed);
     double dt = p.dt_fixed, sdt = d.sdt_fixed;
     if (team.any(!fixed)) {
         dt = p.dt_max;
         const double num = d.eps_adv2 * K00, den = Ar_tot * Ar_tot, n2 = p.eps_diff * r * r;
-        const bool sheet = delta > 0.0 && p.drift_on != 0.0;
         const double rd = r * delta, n3 = sheet ? p.eps_diff * rd * rd : 0.0;
         if constexpr (G == 1) {
-            if (num < dt * den) dt = quot(num, den, recip(den));
+            if (lt(num, dt * den)) dt = quot(num, den, recip(den));
             // a quotient can be below dt only if its numerator is not above dt times the denominator
             // (by the high words, with one unit of slack)
             if (__double2hiint(n2) <= __double2hiint(dt * K00) + 1) {
                 const double t2 = quot(n2, K00, recip(K00));
-                if (t2 < dt) dt = t2;
+                if (lt(t2, dt)) dt = t2;
             }
             if (sheet && __double2hiint(n3) <= __double2hiint(dt * K11) + 1) {
                 const double t3 = quot(n3, K11, recip(K11));
-                if (t3 < dt) dt = t3;
+                if (lt(t3, dt)) dt = t3;
             }
         } else {
             team.recip4(den, K00, K11, 1.0, y4);
             const double n[4] = {num, n2, n3, 0.0}, b[4] = {den, K00, K11, 1.0}, y[4] = {y4[0], y4[1], y4[2], 1.0};
             team.quot4(n, b, y, q4);
-            if (num < dt * den) dt = q4[0];
-            if (q4[1] < dt) dt = q4[1];
-            if (sheet && q4[2] < dt) dt = q4[2];
+            if (lt(num, dt * den)) dt = q4[0];
+            if (lt(q4[1], dt)) dt = q4[1];
+            if (sheet && lt(q4[2], dt)) dt = q4[2];
         }
-        if (dt < p.dt_min) dt = p.dt_min;
+        if (lt(dt, p.dt_min)) dt = p.dt_min;
         if (fixed) dt = p.dt_fixed;
         else sdt = sqrt(dt);
     }
