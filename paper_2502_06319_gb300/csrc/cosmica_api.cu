@@ -807,7 +807,7 @@ extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *e
     thread_local DevBuf buf, lbuf;
     thread_local Staging stage, lstage;
     // items, prefix sums of the particles and of the chunks; behind them the chunks' partial sums
-    const uint32_t per = unbinned_per_thread(total, num_sms());
+    const uint32_t per = unbinned_per_thread(n_per_energy, n_energies, num_sms());
     const size_t b_items = align_up(n_energies * sizeof(SpecItem), 256);
     const size_t b_pre = align_up((n_energies + 1) * sizeof(uint64_t), 256);
     const size_t bytes = b_items + 2 * b_pre;

@@ -175,7 +175,7 @@ cudaError_t launch_spectrum(const unsigned long long *hist, uint32_t n_items, ui
                             double *J, double *sigma, cudaStream_t s);
 
 // unbinned estimator: chunks of `per` x 128 exit states of one item, chunk_prefix their prefix sums over items
-uint32_t unbinned_per_thread(uint64_t n, int sms);
+uint32_t unbinned_per_thread(const uint32_t *n_per_item, uint32_t n_items, int sms);
 uint64_t unbinned_chunks(uint64_t n, uint32_t per);
 size_t unbinned_partial_bytes();
 cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix, const uint64_t *chunk_prefix,

@@ -358,23 +358,23 @@ __global__ void __launch_bounds__(kSpecThreads) k_spectrum(const unsigned long l
 }
 
 // ---- unbinned Eq. 4 ---------------------------------------------------------------
-//   momentum form: summand P0^2 J_LIS(T_ex) / P_ex^2
-//   energy form:   summand beta0 J_LIS(T_ex) exp(lw) / beta_ex  (lw = -sum L ds)
-// pref = P0^2 or beta0.  FP64-pipe bound, so the analytic spectrum is taken with one pow and
+//   momentum form: P0^2 times the mean of J_LIS(T_ex) / P_ex^2
+//   energy form:   beta0 times the mean of J_LIS(T_ex) exp(lw) / beta_ex  (lw = -sum L ds)
+// FP64-pipe bound, so the analytic spectrum is taken with one pow and
 // one division: T^-2.7 / (1 + T^-3.7) = T / (T^3.7 + 1) wherever neither form leaves the range.
-__device__ double unbinned_summand(const SpecItem &it, int form, double pref, double lnP, double lw, int lis_kind,
+__device__ double unbinned_summand(const SpecItem &it, int form, double lnP, double lw, int lis_kind,
                                    const double *lnT, const double *lnJ, uint32_t lis_n)
 {
     const double P = exp(lnP);
     const double pn = P * (fabs(it.Z) / it.A);
     const double En = sqrt(pn * pn + it.m0 * it.m0);
     const double T = pn * pn / (En + it.m0);
-    double num = pref, den;
+    double num, den;
     if (lis_kind == 0 && T > 1e-30 && T < 1e30) {
-        num *= T;
+        num = T;
         den = pow(T, 3.7) + 1.0;
     } else {
-        num *= lis_value(lis_kind, T, lnT, lnJ, lis_n);
+        num = lis_value(lis_kind, T, lnT, lnJ, lis_n);
         den = 1.0;
     }
     if (form == 0) return num / (den * (P * P));
@@ -404,26 +404,29 @@ __global__ void __launch_bounds__(kUnbThreads) k_unbinned_chunks(ExitPtrs ex, co
     const uint32_t e = find_item(chunk_prefix, n_items, blockIdx.x);
     const SpecItem it = items[e];
     const uint64_t lo = prefix[e] + (blockIdx.x - chunk_prefix[e]) * ((uint64_t)per * kUnbThreads), hi = prefix[e + 1];
-    const double P0 = it.A / fabs(it.Z) * sqrt(it.T * (it.T + 2.0 * it.m0));
-    double pref = P0 * P0;
-    if (form != 0) {
-        const double pn0 = P0 * (fabs(it.Z) / it.A);
-        pref = pn0 / sqrt(pn0 * pn0 + it.m0 * it.m0);
-    }
     double s1 = 0.0, s2 = 0.0;
     uint32_t have = 0;       // which of the thread's states are EXIT paths
 #pragma unroll 1
     for (uint32_t k = 0; k < per; ++k) {
         const uint64_t g = lo + (uint64_t)k * kUnbThreads + threadIdx.x;
         if (g < hi && ex.status[g] == COSMICA_PATH_EXIT) {
-            const double f = unbinned_summand(it, form, pref, ex.lnP[g], ex.lw ? ex.lw[g] : 0.0, lis_kind, lnT, lnJ, lis_n);
+            const double f = unbinned_summand(it, form, ex.lnP[g], ex.lw ? ex.lw[g] : 0.0, lis_kind, lnT, lnJ, lis_n);
             v[k * kUnbThreads + threadIdx.x] = f;
             s1 += f;
             have |= 1u << k;
         }
     }
-    const double n = block_sum<kUnbThreads>((double)__popc(have), sh);
-    const double mean = block_sum<kUnbThreads>(s1, sh) / n;
+    // the block's scalars by one thread: a division by all four warps is four times its slots
+    __shared__ uint32_t s_n;
+    __shared__ double s_mean;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const uint32_t mine = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(have));
+    if ((threadIdx.x & 31u) == 0) atomicAdd(&s_n, mine);
+    s1 = block_sum<kUnbThreads>(s1, sh);
+    if (threadIdx.x == 0) s_mean = s1 / (double)s_n;
+    __syncthreads();
+    const double mean = s_mean;
     for (uint32_t k = 0; k < per; ++k) {
         if (have & (1u << k)) {
             const double d = v[k * kUnbThreads + threadIdx.x] - mean;
@@ -431,13 +434,14 @@ __global__ void __launch_bounds__(kUnbThreads) k_unbinned_chunks(ExitPtrs ex, co
         }
     }
     s2 = block_sum<kUnbThreads>(s2, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = UnbPartial{n, mean, s2};
+    if (threadIdx.x == 0) part[blockIdx.x] = UnbPartial{(double)s_n, mean, s2};
 }
 
 // One block per item: sum of the chunks' summands and of their squares about the item's mean,
 // m2 + n (mean_chunk - mean)^2, in a fixed order.
 __global__ void __launch_bounds__(kUnbThreads) k_unbinned_items(const UnbPartial *__restrict__ part,
-                                                                const uint64_t *__restrict__ chunk_prefix, double *J,
+                                                                const uint64_t *__restrict__ chunk_prefix,
+                                                                const SpecItem *__restrict__ items, int form, double *J,
                                                                 double *sigma)
 {
     __shared__ double sh[kUnbThreads];
@@ -462,21 +466,44 @@ __global__ void __launch_bounds__(kUnbThreads) k_unbinned_items(const UnbPartial
             J[e] = __longlong_as_double(0x7FF8000000000000ll);
             sigma[e] = __longlong_as_double(0x7FF8000000000000ll);
         } else {
-            J[e] = mu;
-            sigma[e] = (N > 1.0) ? sqrt(S2 / (N - 1.0) / N) : 0.0;
+            const SpecItem it = items[e];
+            const double P0 = it.A / fabs(it.Z) * sqrt(it.T * (it.T + 2.0 * it.m0));
+            double pref = P0 * P0;
+            if (form != 0) {
+                const double pn0 = P0 * (fabs(it.Z) / it.A);
+                pref = pn0 / sqrt(pn0 * pn0 + it.m0 * it.m0);
+            }
+            J[e] = pref * mu;
+            sigma[e] = (N > 1.0) ? pref * sqrt(S2 / (N - 1.0) / N) : 0.0;
         }
     }
 }
 
 }  // namespace
 
-// Chunks of a launch: per exit states a thread, so that every SM's four schedulers get about
-// eight rounds of work (one warp per scheduler already fills the FP64 pipe), at most kUnbPer.
-uint32_t unbinned_per_thread(uint64_t n, int sms)
+uint64_t unbinned_chunks(uint64_t n, uint32_t per)
 {
-    return (uint32_t)std::min<uint64_t>(kUnbPer, std::max<uint64_t>(1, n / ((uint64_t)sms * kUnbThreads * 8)));
+    return (n + (uint64_t)per * kUnbThreads - 1) / ((uint64_t)per * kUnbThreads);
 }
-uint64_t unbinned_chunks(uint64_t n, uint32_t per) { return (n + (uint64_t)per * kUnbThreads - 1) / ((uint64_t)per * kUnbThreads); }
+// Exit states a thread takes (at most kUnbPer): a block of 128 fills the FP64 pipe of its SM's four
+// schedulers, so a launch lasts the largest number of blocks on an SM times a block's work, some
+// 150 slots a state and 60 more for its sums; the size with the shortest such time.  6e5 states of
+// 30 items: 196 us with 8 (600 blocks, 3.95 per SM) against 216 with 7 (685, 4.5 per SM).
+uint32_t unbinned_per_thread(const uint32_t *n_per_item, uint32_t n_items, int sms)
+{
+    uint32_t best = kUnbPer;
+    uint64_t least = UINT64_MAX;
+    for (uint32_t per = 1; per <= kUnbPer; ++per) {
+        uint64_t blocks = 0;
+        for (uint32_t e = 0; e < n_items; ++e) blocks += unbinned_chunks(n_per_item[e], per);
+        const uint64_t cost = (blocks + sms - 1) / sms * (150u * per + 60u);
+        if (cost < least) {
+            least = cost;
+            best = per;
+        }
+    }
+    return best;
+}
 size_t spectrum_sums_bytes() { return sizeof(SpecSums); }
 size_t unbinned_partial_bytes() { return sizeof(UnbPartial); }
 
@@ -493,7 +520,7 @@ cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix,
                                                                      lis_kind, lis_lnT, lis_lnJ, lis_n, part);
         note_launch();
     }
-    k_unbinned_items<<<n_items, kUnbThreads, 0, s>>>(part, chunk_prefix, J, sigma);
+    k_unbinned_items<<<n_items, kUnbThreads, 0, s>>>(part, chunk_prefix, items, form, J, sigma);
     note_launch();
     return cudaGetLastError();
 }
