@@ -738,11 +738,12 @@ static cosmica_status spectrum_of(const cosmica_exit_states *ex, const SpecItems
     void *d_sums = (char *)ibuf.d + up;
     double *d_w = table ? (double *)((char *)ibuf.d + up + b_sums) : nullptr;
     unsigned long long *h = (unsigned long long *)hist;
-    cudaError_t e = launch_spec_prep(h, ex ? (uint64_t)n_items * COSMICA_HIST_STRIDE(nbins) : 0, d_items,
-                                     (const uint32_t *)((const char *)ibuf.d + b_items), n_sp, nbins, x_lo, dx, kind,
-                                     lnT, lnJ, ln, d_w, s);
-    if (e != cudaSuccess) return cuda_fail(e, "spectrum set-up launch");
-    if (ex) e = launch_histogram(exit_ptrs(ex), ex->n, n_items, nbins, x_lo, dx, h, num_sms(), s);
+    const WeightTable wt{d_items, (const uint32_t *)((const char *)ibuf.d + b_items), n_sp, kind, lnT, lnJ, ln, d_w};
+    cudaError_t e = cudaSuccess;
+    if (ex) e = launch_spec_clear(h, (uint64_t)n_items * COSMICA_HIST_STRIDE(nbins), s);
+    if (e != cudaSuccess) return cuda_fail(e, "histogram clear launch");
+    // a given histogram adds no exit states; the table of weights is filled all the same
+    e = launch_histogram(ex ? exit_ptrs(ex) : ExitPtrs{}, ex ? ex->n : 0, n_items, nbins, x_lo, dx, h, wt, num_sms(), s);
     if (e != cudaSuccess) return cuda_fail(e, "histogram kernel launch");
     e = launch_spectrum(h, n_items, nbins, x_lo, dx, d_items, d_w, kind, lnT, lnJ, ln, d_sums, J, sigma, s);
     return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "spectrum kernel launch");

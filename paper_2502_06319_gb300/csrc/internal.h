@@ -159,14 +159,22 @@ struct SpecItem {
     double A, Z, m0;           // species
     uint32_t sp, pad;          // row of the species in the table of bin weights
 };
-// clears hist[0 .. n_hist) and fills weights [n_sp x nbins] (none for null weights), species s
-// being that of items[sp_item[s]]
-cudaError_t launch_spec_prep(unsigned long long *hist, uint64_t n_hist, const SpecItem *items, const uint32_t *sp_item,
-                             uint32_t n_sp, uint32_t nbins, double x_lo, double dx, int lis_kind, const double *lis_lnT,
-                             const double *lis_lnJ, uint32_t lis_n, double *weights, cudaStream_t s);
+// table of bin weights [n_sp x nbins] to fill (none if weights is null), species s being that of
+// items[sp_item[s]]
+struct WeightTable {
+    const SpecItem *items;
+    const uint32_t *sp_item;
+    uint32_t n_sp;
+    int lis_kind;
+    const double *lnT, *lnJ;
+    uint32_t lis_n;
+    double *weights;
+};
+cudaError_t launch_spec_clear(unsigned long long *hist, uint64_t n_hist, cudaStream_t s);
+// adds n exit states to the cleared histogram and fills the table of bin weights
 cudaError_t launch_histogram(const ExitPtrs &ex, uint64_t n, uint32_t n_items, uint32_t nbins, double x_lo,
-                             double dx, unsigned long long *hist, int sms, cudaStream_t s);
-// weights: from launch_spec_prep, or null (every item evaluates its own); sums: scratch of
+                             double dx, unsigned long long *hist, const WeightTable &wt, int sms, cudaStream_t s);
+// weights: from launch_histogram, or null (every item evaluates its own); sums: scratch of
 // n_items x spectrum_sums_bytes()
 size_t spectrum_sums_bytes();
 cudaError_t launch_spectrum(const unsigned long long *hist, uint32_t n_items, uint32_t nbins,

@@ -2,10 +2,11 @@
 // Built with -fmad=false so that the bin of every exit is decided by the
 // same FP64 operations as its definition: b = floor((lnP / ln 10 - x_lo) / dx).
 //
-//   k_spec_prep  clears the histogram and, meanwhile, evaluates the bin weights
-//                w_b = J_LIS(T_b) / P_b^2 once per species and bin
+//   k_spec_clear clears the histogram
 //   k_histogram  blocks of consecutive exit states count into shared memory and add
-//                their nonzero counters to the histogram (integers: deterministic)
+//                their nonzero counters to the histogram (integers: deterministic);
+//                a few more evaluate the bin weights w_b = J_LIS(T_b) / P_b^2 once per
+//                species and bin
 //   k_spectrum_warp, k_spectrum
 //                one warp or one block per item: J = P0^2 (1/N) sum_b c_b w_b (J = f P^2 is
 //                the intensity per unit kinetic energy and f is conserved along
@@ -24,6 +25,45 @@
 namespace cosmica {
 
 namespace {
+
+// ---- local interstellar spectrum ------------------------------------------------
+__device__ double lis_value(int kind, double T, const double *lnT, const double *lnJ, uint32_t m)
+{
+    if (kind == 0) return pow(T, -2.7) / (1.0 + pow(T, -3.7));
+    const double x = log(T);
+    if (x <= lnT[0]) return exp(lnJ[0]);
+    if (x >= lnT[m - 1]) return exp(lnJ[m - 1]);
+    uint32_t lo = 0, hi = m - 1;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (lnT[mid] <= x) lo = mid; else hi = mid;
+    }
+    const double t = (x - lnT[lo]) / (lnT[hi] - lnT[lo]);
+    return exp(lnJ[lo] + t * (lnJ[hi] - lnJ[lo]));
+}
+
+// bin weight w_b = J_LIS(T_b) / P_b^2 at the bin's log-centre
+__device__ double bin_weight(const SpecItem &it, uint32_t b, double x_lo, double dx, int lis_kind, const double *lnT,
+                             const double *lnJ, uint32_t lis_n)
+{
+    const double zoa = fabs(it.Z) / it.A;
+    const double Pb = pow(10.0, x_lo + ((double)b + 0.5) * dx);
+    const double pn = Pb * zoa;
+    const double En = sqrt(pn * pn + it.m0 * it.m0);
+    const double Tb = pn * pn / (En + it.m0);
+    return lis_value(lis_kind, Tb, lnT, lnJ, lis_n) / (Pb * Pb);
+}
+
+// The bin weights of the n_sp species (those of items sp_item[s]), one thread per bin: three pow
+// each, the whole cost of a spectrum when every item evaluated its own.  Called by every thread
+// of the blocks 0, 1, ... that cover n_sp x nbins.
+__device__ __forceinline__ void fill_weights(const WeightTable &w, uint32_t nbins, double x_lo, double dx, uint32_t block)
+{
+    const uint64_t i = (uint64_t)block * blockDim.x + threadIdx.x;
+    if (i >= (uint64_t)w.n_sp * nbins) return;
+    const uint32_t s = (uint32_t)(i / nbins), b = (uint32_t)(i % nbins);
+    w.weights[i] = bin_weight(w.items[w.sp_item[s]], b, x_lo, dx, w.lis_kind, w.lnT, w.lnJ, w.lis_n);
+}
 
 // ---- histogram ---------------------------------------------------------------
 // b = floor((lnP / ln 10 - x_lo) / dx) costs two FP64 divisions (about 20 slots of 64
@@ -97,11 +137,18 @@ constexpr uint32_t kHistWords = 8192;      // 32 KB of counters: 15 rows of 512 
 // was ten times that.
 __global__ void __launch_bounds__(kHistThreads) k_histogram(ExitPtrs ex, uint64_t n, uint32_t n_items, uint32_t nbins,
                                                             BinRule rule, uint32_t rows, uint32_t per,
-                                                            unsigned long long *__restrict__ hist)
+                                                            unsigned long long *__restrict__ hist, WeightTable wt,
+                                                            uint32_t wblocks)
 {
+    // the first blocks fill the table of bin weights meanwhile (some 8 us of dependent pow: with
+    // the clearing, in a launch of their own, the spectrum of 5760 items took 113 us, so 102)
+    if (blockIdx.x < wblocks) {
+        fill_weights(wt, nbins, rule.x_lo, rule.dx, blockIdx.x);
+        return;
+    }
     __shared__ __align__(16) uint32_t cnt[kHistWords];
     const uint32_t stride = nbins + 3u;
-    const uint64_t g0 = (uint64_t)blockIdx.x * (per * kHistThreads);
+    const uint64_t g0 = (uint64_t)(blockIdx.x - wblocks) * (per * kHistThreads);
     const uint32_t words = rows * stride;
     for (uint32_t w = threadIdx.x * 4; w < words; w += kHistThreads * 4)
         *reinterpret_cast<uint4 *>(cnt + w) = make_uint4(0u, 0u, 0u, 0u);   // words <= kHistWords, itself a multiple of 4
@@ -143,34 +190,6 @@ __global__ void __launch_bounds__(kHistThreads) k_histogram(ExitPtrs ex, uint64_
     }
 }
 
-// ---- local interstellar spectrum ------------------------------------------------
-__device__ double lis_value(int kind, double T, const double *lnT, const double *lnJ, uint32_t m)
-{
-    if (kind == 0) return pow(T, -2.7) / (1.0 + pow(T, -3.7));
-    const double x = log(T);
-    if (x <= lnT[0]) return exp(lnJ[0]);
-    if (x >= lnT[m - 1]) return exp(lnJ[m - 1]);
-    uint32_t lo = 0, hi = m - 1;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (lnT[mid] <= x) lo = mid; else hi = mid;
-    }
-    const double t = (x - lnT[lo]) / (lnT[hi] - lnT[lo]);
-    return exp(lnJ[lo] + t * (lnJ[hi] - lnJ[lo]));
-}
-
-// bin weight w_b = J_LIS(T_b) / P_b^2 at the bin's log-centre
-__device__ double bin_weight(const SpecItem &it, uint32_t b, double x_lo, double dx, int lis_kind, const double *lnT,
-                             const double *lnJ, uint32_t lis_n)
-{
-    const double zoa = fabs(it.Z) / it.A;
-    const double Pb = pow(10.0, x_lo + ((double)b + 0.5) * dx);
-    const double pn = Pb * zoa;
-    const double En = sqrt(pn * pn + it.m0 * it.m0);
-    const double Tb = pn * pn / (En + it.m0);
-    return lis_value(lis_kind, Tb, lnT, lnJ, lis_n) / (Pb * Pb);
-}
-
 template <int NT>
 __device__ double block_sum(double v, double *sh)
 {
@@ -188,26 +207,12 @@ __device__ double block_sum(double v, double *sh)
 constexpr int kSpecThreads = 256;
 constexpr uint32_t kPrepThreads = 128;
 
-// The first `wblocks` blocks evaluate the bin weights of the n_sp species (those of items
-// sp_item[s]), one thread per bin -- three pow each, the whole cost of a spectrum when every
-// item evaluated its own -- while the others clear the histogram.
-__global__ void __launch_bounds__(kPrepThreads) k_spec_prep(unsigned long long *__restrict__ hist, uint64_t n_hist,
-                                                            uint32_t wblocks, const SpecItem *__restrict__ items,
-                                                            const uint32_t *__restrict__ sp_item, uint32_t n_sp,
-                                                            uint32_t nbins, double x_lo, double dx, int lis_kind,
-                                                            const double *lnT, const double *lnJ, uint32_t lis_n,
-                                                            double *__restrict__ weights)
+// Clears the histogram: 16-byte stores between an odd first and last counter (the array may
+// start at any counter).
+__global__ void __launch_bounds__(kPrepThreads) k_spec_clear(unsigned long long *__restrict__ hist, uint64_t n_hist)
 {
-    if (blockIdx.x < wblocks) {
-        const uint64_t i = (uint64_t)blockIdx.x * kPrepThreads + threadIdx.x;
-        if (i >= (uint64_t)n_sp * nbins) return;
-        const uint32_t s = (uint32_t)(i / nbins), b = (uint32_t)(i % nbins);
-        weights[i] = bin_weight(items[sp_item[s]], b, x_lo, dx, lis_kind, lnT, lnJ, lis_n);
-        return;
-    }
-    // 16-byte stores between an odd first and last counter (the array may start at any counter)
-    const uint64_t step = (uint64_t)(gridDim.x - wblocks) * kPrepThreads;
-    const uint64_t t = (uint64_t)(blockIdx.x - wblocks) * kPrepThreads + threadIdx.x;
+    const uint64_t step = (uint64_t)gridDim.x * kPrepThreads;
+    const uint64_t t = (uint64_t)blockIdx.x * kPrepThreads + threadIdx.x;
     const uint64_t odd = (reinterpret_cast<uintptr_t>(hist) >> 3) & 1u, pairs = n_hist > odd ? (n_hist - odd) / 2 : 0;
     ulonglong2 *__restrict__ h2 = reinterpret_cast<ulonglong2 *>(hist + odd);
     for (uint64_t i = t; i < pairs; i += step) h2[i] = make_ulonglong2(0ull, 0ull);
@@ -388,8 +393,8 @@ struct UnbPartial {
     double n, mean, m2;     // EXIT paths of the chunk, mean summand, sum of squares about it
 };
 
-// Bound by the FP64 pipe (about 180 slots a state: two exp, a pow, a square root, two divisions).
-// 6e5 states of 30 items: 230 us, against 10 ms with one block per item and two passes.
+// Bound by the FP64 pipe (about 150 slots a state: two exp, a pow, a square root, two divisions).
+// 6e5 states of 30 items: 196 us, against 10 ms with one block per item and two passes.
 // One block per chunk of per x 128 consecutive exit states of one item.  The summands stay
 // in shared memory for the second moment, which is taken about the chunk's own mean (as exact
 // as a second pass over the item, without evaluating anything twice).
@@ -525,33 +530,29 @@ cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix,
     return cudaGetLastError();
 }
 
-cudaError_t launch_spec_prep(unsigned long long *hist, uint64_t n_hist, const SpecItem *items, const uint32_t *sp_item,
-                             uint32_t n_sp, uint32_t nbins, double x_lo, double dx, int lis_kind, const double *lis_lnT,
-                             const double *lis_lnJ, uint32_t lis_n, double *weights, cudaStream_t s)
+cudaError_t launch_spec_clear(unsigned long long *hist, uint64_t n_hist, cudaStream_t s)
 {
-    const uint64_t wblocks = weights ? ((uint64_t)n_sp * nbins + kPrepThreads - 1) / kPrepThreads : 0;
-    const uint64_t zblocks = std::min<uint64_t>(2048, (n_hist + 4 * kPrepThreads - 1) / (4 * kPrepThreads));
-    if (wblocks + zblocks == 0) return cudaSuccess;
+    if (n_hist == 0) return cudaSuccess;
     cudaGetLastError();
-    k_spec_prep<<<(unsigned)(wblocks + zblocks), kPrepThreads, 0, s>>>(hist, n_hist, (uint32_t)wblocks, items, sp_item, n_sp,
-                                                                       nbins, x_lo, dx, lis_kind, lis_lnT, lis_lnJ, lis_n,
-                                                                       weights);
+    const uint64_t blocks = std::min<uint64_t>(2048, (n_hist + 4 * kPrepThreads - 1) / (4 * kPrepThreads));
+    k_spec_clear<<<(unsigned)blocks, kPrepThreads, 0, s>>>(hist, n_hist);
     note_launch();
     return cudaGetLastError();
 }
 
 cudaError_t launch_histogram(const ExitPtrs &ex, uint64_t n, uint32_t n_items, uint32_t nbins, double x_lo,
-                             double dx, unsigned long long *hist, int sms, cudaStream_t s)
+                             double dx, unsigned long long *hist, const WeightTable &wt, int sms, cudaStream_t s)
 {
-    if (n == 0 || n_items == 0) return cudaSuccess;
+    const uint32_t wblocks = wt.weights ? (uint32_t)(((uint64_t)wt.n_sp * nbins + kHistThreads - 1) / kHistThreads) : 0u;
+    if (n_items == 0 || (n == 0 && wblocks == 0)) return cudaSuccess;
     cudaGetLastError();
     // rows of counters that fit (none above 8189 bins: every state then adds to the histogram
     // directly); 1 to 32 states a thread, four blocks per SM first
     const uint32_t rows = nbins <= kHistWords - 3u ? kHistWords / (nbins + 3u) : 0u;
     const uint64_t per = std::min<uint64_t>(32, std::max<uint64_t>(1, n / ((uint64_t)sms * 4 * kHistThreads)));
     const uint64_t blocks = (n + per * kHistThreads - 1) / (per * kHistThreads);
-    k_histogram<<<(unsigned)blocks, kHistThreads, 0, s>>>(ex, n, n_items, nbins, make_rule(x_lo, dx), rows,
-                                                          (uint32_t)per, hist);
+    k_histogram<<<(unsigned)blocks + wblocks, kHistThreads, 0, s>>>(ex, n, n_items, nbins, make_rule(x_lo, dx), rows,
+                                                                    (uint32_t)per, hist, wt, wblocks);
     note_launch();
     return cudaGetLastError();
 }

@@ -199,10 +199,9 @@ bool cosmica_server::retire(uint64_t ticket, Req &r)
     cudaError_t e = cudaMemsetAsync(weights.d, 0, 256, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_spec_items, its.data(), nE * sizeof(SpecItem),
                                               cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-        e = launch_spec_prep(d_hist, (uint64_t)nE * stride, d_spec_items, (const uint32_t *)weights.d, 1, nb, x_lo, dx, 0,
-                             nullptr, nullptr, 0, d_w, stream);
-    if (e == cudaSuccess) e = launch_histogram(ex, r.total, nE, nb, x_lo, dx, d_hist, num_sms(), stream);
+    const WeightTable wt{d_spec_items, (const uint32_t *)weights.d, 1, 0, nullptr, nullptr, 0, d_w};
+    if (e == cudaSuccess) e = launch_spec_clear(d_hist, (uint64_t)nE * stride, stream);
+    if (e == cudaSuccess) e = launch_histogram(ex, r.total, nE, nb, x_lo, dx, d_hist, wt, num_sms(), stream);
     if (e == cudaSuccess)
         e = launch_spectrum(d_hist, nE, nb, x_lo, dx, d_spec_items, d_w, 0, nullptr, nullptr, 0, d_sums, d_J, d_S,
                             stream);
