@@ -361,14 +361,17 @@ int num_sms()
 
 // Blocks of 128 (warps per scheduler) of an untuned launch.  More of them raise the rate, fewer
 // step each path faster (0.3 us a step alone, 0.9 us with four), and a launch waits for its
-// slowest paths, some ten times the mean.  Measured in paths per lane of one layer (one warp per
-// scheduler), ms with 1 / 2 / 3 / 4 layers: 1.5: 36 / 43 / 49 / 50, 3: 47 / 52 / 58 / 60,
-// 8: 55 / 51 / 55 / 59, 15: 73 / 67 / 71 / 70, 31: 127 / 96 / 93 / 99,
-// 57 (FP64 sums): 1074 / 720 / 629 / 630.
+// slowest paths, some ten times the mean, the more so the more heliospheres differ.  Measured in
+// paths per lane of one layer (one warp per scheduler), ms with 1 / 2 / 3 / 4 layers:
+// one heliosphere: 3: 40 / 46 / 50 / 56, 6: 39 / 42, 7: 46 / 43, 15: 65 / 61 / 64 / 65,
+// 20: - / 68 / 76 / 73, 40: - / 119 / 115 / 117; four: 5: 96 / 161 / 180 / 213, 7: 113 / 165,
+// 8: 116 / 141, 10: 133 / 135 / 190 / 202, 20: - / 202 / 206 / 252, 30: - / 273 / 262 / 299,
+// 60: - / 513 / 489 / 488; the same with FP64 sums: 5: 162 / 251, 7: 187 / 259, 10: 218 / 209,
+// 20: - / 298 / 278 / 274, 60: - / 737 / 656 / 645.
 int untuned_layers(uint64_t n_total, int sms, int max_blocks)
 {
     const uint64_t layer = (uint64_t)sms * 128u;
-    const int layers = n_total <= 4 * layer ? 1 : n_total <= 20 * layer ? 2 : n_total <= 40 * layer ? 3 : max_blocks;
+    const int layers = n_total <= 7 * layer ? 1 : n_total <= 20 * layer ? 2 : n_total <= 40 * layer ? 3 : max_blocks;
     return std::max(1, std::min(layers, max_blocks));
 }
 
