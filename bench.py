@@ -17,7 +17,7 @@ throughput the line carries:
   * spectrum_error: the mixed spectra of twelve items of the workload against
     the FP64 CPU oracle's results for the same quasi-particles (stored by
     tests/golden/make_c3_golden.py), per item |dJ|/J and |dJ|/sigma;
-  * fp64_plain: the plain FP64 GPU path (one thread per particle) and the
+  * fp64_plain: the FP64 GPU path and the
     mixed path timed on the same stratified sample of the workload;
   * serving: the continuous-batching server under Poisson request streams at
     0.5x and 0.8x of its measured capacity (p50/p99 latency, spectra/s);

@@ -232,16 +232,16 @@ void cosmica_model_destroy(cosmica_model *model);
 
 /*
  * Propagate quasi-particles backward in time until they leave the heliosphere
- * (Sec. IV.A: one thread per quasi-particle, a propagation kernel evolving
- * each path until a boundary is reached).
+ * (Sec. IV.A: a propagation kernel evolving each path until a boundary is
+ * reached).
  *   species        host, one species for all energies
  *   T_in_GeVn      host [n_energies], kinetic energy per nucleon at the start
  *   n_per_energy   host [n_energies], quasi-particles per energy (0 allowed)
  *   seed           Philox key
  *   out            exit states; out->n must equal sum(n_per_energy); out->item
  *                  receives the energy index
- * Particle g has pid = g.  The FP64 path launches one thread per particle;
- * the mixed paths run the persistent work-queue kernel.
+ * Particle g has pid = g.  All precisions run persistent work-queue kernels
+ * and hand the last paths to kernels with more lanes or fewer warps for them.
  * Errors: INVALID (sizes, null pointers), OOM, CUDA. */
 cosmica_status cosmica_propagate(cosmica_model *model, const cosmica_species *species,
                                  const double *T_in_GeVn, uint32_t n_energies,
@@ -378,7 +378,7 @@ typedef struct {
 } cosmica_work_item;
 
 /* Launch shape and scheduling of the persistent kernel.  Passing NULL selects
- * block 128, compaction with a look every 64 steps, no graph,
+ * block 128, a look every 64 steps whether the last particles fit fewer warps, no graph,
  * most-expensive-first queue order, and 1 to 4 blocks per SM by the number of
  * particles (a launch with few of them is bound by its slowest paths, which
  * step faster when fewer warps share an SM).  The same default shapes the
@@ -444,7 +444,7 @@ cosmica_status cosmica_batch_spectrum_hist(cosmica_batch *batch, const cosmica_w
                                            void *stream);
 
 /* Pick a launch shape for this batch by timing candidate shapes (block size,
- * resident blocks, compaction period) and write the fastest to *best (its
+ * resident blocks, hand-over of the last particles) and write the fastest to *best (its
  * predicted steps/s in *best_rate if not NULL).  Batches of up to ~30 particles
  * per SM thread slot are timed whole; larger ones on two scaled samples of
  * `items` (host; ~10 and ~30 particles per slot), from which each candidate's
@@ -452,7 +452,7 @@ cosmica_status cosmica_batch_spectrum_hist(cosmica_batch *batch, const cosmica_w
  * process per device and configuration class (precision, drift, termination
  * shock, particle count within a factor of two, kernel variant); a cached
  * class returns at once.  Synchronous; uses the batch's own scratch.  An FP64
- * batch needs no tuning and gets block 128 without compaction.  Errors:
+ * batch needs no tuning and gets block 128 and period 0.  Errors:
  * INVALID (NULL batch/best, invalid items, no particles), OOM, CUDA. */
 cosmica_status cosmica_autotune(cosmica_batch *batch, const cosmica_work_item *items,
                                 uint32_t n_items, cosmica_tuning *best, double *best_rate);

@@ -785,8 +785,13 @@ extern "C" cosmica_status cosmica_spectrum(const cosmica_exit_states *exit, cons
     // scratch of the calling thread: the spectrum call carries no handle
     thread_local DevBuf ibuf, lbuf;
     thread_local Staging istage, lstage;
-    return run_spectrum(exit, si, lis, bins, J_out, sigma_out, hist_out, ibuf, istage, lbuf, lstage,
-                        (cudaStream_t)stream);
+    thread_local StreamOrder order;
+    st = order.begin((cudaStream_t)stream);
+    if (st != COSMICA_OK) return st;
+    st = run_spectrum(exit, si, lis, bins, J_out, sigma_out, hist_out, ibuf, istage, lbuf, lstage,
+                      (cudaStream_t)stream);
+    const cosmica_status ordered = order.end((cudaStream_t)stream);   // also after a launch that failed half-way
+    return st != COSMICA_OK ? st : ordered;
 }
 
 extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *exit, const cosmica_species *species,
@@ -810,6 +815,7 @@ extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *e
     cudaStream_t s = (cudaStream_t)stream;
     thread_local DevBuf buf, lbuf;
     thread_local Staging stage, lstage;
+    thread_local StreamOrder order;
     // items, prefix sums of the particles and of the chunks; behind them the chunks' partial sums
     const uint32_t per = unbinned_per_thread(n_per_energy, n_energies, num_sms());
     const size_t b_items = align_up(n_energies * sizeof(SpecItem), 256);
@@ -829,6 +835,8 @@ extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *e
     const uint64_t n_chunks = hc[n_energies];
     st = buf.reserve(bytes + n_chunks * unbinned_partial_bytes());
     if (st != COSMICA_OK) return st;
+    st = order.begin(s);
+    if (st != COSMICA_OK) return st;
     st = stage.upload(buf.d, bytes, s);
     if (st != COSMICA_OK) return st;
     int kind; const double *lnT, *lnJ; uint32_t ln;
@@ -839,7 +847,8 @@ extern "C" cosmica_status cosmica_spectrum_unbinned(const cosmica_exit_states *e
                                              (const uint64_t *)(d + b_items + b_pre), n_chunks, per, d + bytes,
                                              n_energies, (const SpecItem *)d, formulation, kind, lnT, lnJ, ln, J_out,
                                              sigma_out, s);
-    return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "unbinned spectrum launch");
+    st = order.end(s);
+    return e == cudaSuccess ? st : cuda_fail(e, "unbinned spectrum launch");
 }
 
 // =============================================================== batch API ==

@@ -95,6 +95,32 @@ struct Staging {
     }
 };
 
+// Orders the uses of a scratch buffer that belongs to no handle: consecutive calls of a thread may
+// be on different streams, and the partial sums and weights of one must not be overwritten by the
+// next while its kernels run.  A call under capture is ordered by whoever replays it.
+struct StreamOrder {
+    cudaEvent_t ev = nullptr;
+    bool used = false;
+    static bool capturing(cudaStream_t s)
+    {
+        cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+        return cudaStreamIsCapturing(s, &c) != cudaSuccess || c != cudaStreamCaptureStatusNone;
+    }
+    cosmica_status begin(cudaStream_t s)
+    {
+        if (used && !capturing(s)) CK(cudaStreamWaitEvent(s, ev, 0), "cudaStreamWaitEvent(scratch)");
+        return COSMICA_OK;
+    }
+    cosmica_status end(cudaStream_t s)
+    {
+        if (capturing(s)) return COSMICA_OK;
+        if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate(scratch)");
+        CK(cudaEventRecord(ev, s), "cudaEventRecord(scratch)");
+        used = true;
+        return COSMICA_OK;
+    }
+};
+
 size_t align_up(size_t x, size_t a);
 bool is_device_ptr(const void *p);
 cosmica_status check_params(const cosmica_params *p);

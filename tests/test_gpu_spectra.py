@@ -136,3 +136,37 @@ def test_unbinned(counts, form, with_table):
     # a summand carries a few ulp (pow, exp, divisions), a sum of 4e5 positive terms at most 1e-13 more
     np.testing.assert_allclose(J.cpu().numpy(), wJ, rtol=1e-12, equal_nan=True)
     np.testing.assert_allclose(S.cpu().numpy(), wS, rtol=1e-12, equal_nan=True)
+
+
+def test_calls_of_one_thread_on_two_streams():
+    """The scratch of the handle-less calls is one per thread: calls on two streams that nothing else orders
+    give what each gives alone."""
+    import torch
+    rng = np.random.default_rng(5)
+    E, nbins, streams = 40, 2048, [torch.cuda.Stream() for _ in range(2)]
+    T = list(np.exp(rng.uniform(-2.0, 4.0, E)))
+    jobs = []
+    for n in (4000000, 40000):
+        item = np.sort(rng.integers(0, E, n)).astype(np.uint32)
+        out = device_exits(rng.normal(1.0, 1.0, n), np.ones(n, np.uint8), item, -np.abs(rng.normal(0.5, 0.3, n)))
+        jobs.append((out, [int(c) for c in np.bincount(item, minlength=E)]))
+    sp, bins = cz.make_species(W.PROTON), cz.make_bins(0.1, 1000.0, nbins)
+
+    def call(job, stream):
+        out, counts = job
+        r = [torch.empty(E, dtype=torch.float64, device="cuda") for _ in range(4)]
+        H = torch.empty(E * (nbins + 3), dtype=torch.int64, device="cuda")
+        stream.wait_stream(torch.cuda.current_stream())
+        cz.cosmica_spectrum(out, sp, T, bins, r[0], r[1], H, stream=stream)
+        cz.cosmica_spectrum_unbinned(out, sp, T, counts, 1, r[2], r[3], stream=stream)
+        return r + [H]
+
+    alone = []
+    for j in jobs:
+        alone.append(call(j, streams[0]))
+        torch.cuda.synchronize()
+    together = [[call(j, s) for j, s in zip(jobs, streams)] for _ in range(10)]
+    torch.cuda.synchronize()
+    for pair in together:
+        for got, ref in zip(pair, alone):
+            assert all(torch.equal(a, b) for a, b in zip(got, ref))
