@@ -46,7 +46,7 @@ def test_hand_over(model, form, precision):
     """Paths of three energies, some ended by the step limit, others before the first hand-over."""
     p = dict(MODELS[model], formulation=float(form), max_steps=6000.0)
     b = cz.cosmica_batch_create([cz.make_params(p, precision)], [cz.make_species(W.HELIUM4)])
-    for n in (LAYER + 1, 3 * LAYER + 77):
+    for n in (LAYER + 1, 6 * LAYER, 6 * LAYER + 77):
         items = [(0, 0, 30.0, n - n // 3 - 5, 0, 1), (0, 0, 1.0, n // 3, 50, 2), (0, 0, 4.0, 5, 0, 3)]
         ref = run(b, items, cz.cosmica_tuning(128, 0, 0, 0, 0))
         assert len(np.unique(ref["steps"])) > 100
@@ -61,7 +61,7 @@ def test_hand_over(model, form, precision):
 @pytest.mark.parametrize("precision", [cz.PREC_MIXED, cz.PREC_MIXED_F64ACC])
 def test_without_allocation(precision):
     """The fixed scratch holds shorter lists: sizes below, at and above what they hold, against the ordinary entry."""
-    for n in (LAYER, LAYER + 1, 5 * LAYER):
+    for n in (LAYER, LAYER + 1, 5 * LAYER, 8 * LAYER):
         job = W.Job(dict(MODELS["shock"], max_steps=3000), W.PROTON, [2.0, 20.0], [n - 999, 999], seed=5)
         ref, _, m = gpu_run(job, precision=precision)
         m.close()
