@@ -380,7 +380,8 @@ typedef struct {
 /* Launch shape and scheduling of the persistent kernel.  Passing NULL selects
  * block 128, a look every 64 steps whether the last particles fit fewer warps, no graph,
  * most-expensive-first queue order, and 1 to 4 blocks per SM by the number of
- * particles (a launch with few of them is bound by its slowest paths, which
+ * particles and the spread of their expected steps (a launch with few of them is
+ * bound by its slowest paths, which
  * step faster when fewer warps share an SM).  The same default shapes the
  * launches of cosmica_propagate, cosmica_propagate_orbit and
  * cosmica_propagate_noalloc. */
@@ -388,7 +389,8 @@ typedef struct {
     uint32_t block;           /* threads per block (32..256; 0 = 128)                   */
     uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit);
                                  with a compact_period, one of 128 threads at most for up
-                                 to 768 particles per SM, which is then faster          */
+                                 to 768 particles per SM, if an untuned launch takes
+                                 one, which is then faster                              */
     uint32_t compact_period;  /* once the queue is drained, every this many steps the
                                  launch looks whether the particles left fit fewer warps,
                                  which then take them over (0 = never)                   */

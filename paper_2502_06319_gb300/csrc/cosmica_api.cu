@@ -14,6 +14,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <new>
@@ -262,6 +263,7 @@ struct Tables {
     uint32_t *list = nullptr;                 // paths a kernel of the launch leaves to the next
     uint32_t list_cap = 0;
     uint64_t n_total = 0;
+    uint64_t n_long = 0;                      // see cost_order
     uint32_t n_items = 0;
 
     // order: queue order of the items (a permutation of 0..n-1), or empty for item order
@@ -317,21 +319,30 @@ static double start_K0(const cosmica_params &p, double r)
     return p.shell_K0[i];
 }
 
-// Queue order with the longest expected paths first: items sorted by K0 beta0 P0
-// ascending (a smaller diffusion coefficient at the start means more steps).
-std::vector<uint32_t> cost_order(const std::vector<DevItem> &its, const cosmica_params *prm,
-                                 const cosmica_species *spc)
+// K0 beta0 P0 of a path's start: a smaller diffusion coefficient there means more steps
+double start_key(const cosmica_params &p, const cosmica_species &sp, double T, double r0)
+{
+    const double aoz = (double)sp.A / std::fabs((double)sp.Z);
+    const double pn = std::sqrt(T * (T + 2.0 * sp.m0_GeV));
+    const double P = aoz * pn;
+    const double beta = pn / (T + sp.m0_GeV);
+    return start_K0(p, r0) * beta * P;
+}
+
+// Queue order with the longest expected paths first: items sorted by their key, ascending.
+// n_long: particles whose key is within a factor of three of the smallest (see untuned_layers).
+std::vector<uint32_t> cost_order(const std::vector<DevItem> &its, const std::vector<uint64_t> &pre,
+                                 const cosmica_params *prm, const cosmica_species *spc, uint64_t *n_long)
 {
     std::vector<std::pair<double, uint32_t>> key(its.size());
+    double least = std::numeric_limits<double>::infinity();
     for (size_t i = 0; i < its.size(); ++i) {
-        const cosmica_species &sp = spc[its[i].species_idx];
-        const double aoz = (double)sp.A / std::fabs((double)sp.Z);
-        const double T = its[i].T;
-        const double pn = std::sqrt(T * (T + 2.0 * sp.m0_GeV));
-        const double P = aoz * pn;
-        const double beta = pn / (T + sp.m0_GeV);
-        key[i] = {start_K0(prm[its[i].param_idx], its[i].r0) * beta * P, (uint32_t)i};
+        key[i] = {start_key(prm[its[i].param_idx], spc[its[i].species_idx], its[i].T, its[i].r0), (uint32_t)i};
+        if (pre[i + 1] > pre[i]) least = std::min(least, key[i].first);
     }
+    *n_long = 0;
+    for (size_t i = 0; i < its.size(); ++i)
+        if (key[i].first <= 3.0 * least) *n_long += pre[i + 1] - pre[i];
     std::stable_sort(key.begin(), key.end(),
                      [](const std::pair<double, uint32_t> &a, const std::pair<double, uint32_t> &b) {
                          return a.first < b.first;
@@ -359,23 +370,29 @@ int num_sms()
     return n;
 }
 
-// Blocks of 128 (warps per scheduler) of an untuned launch.  More of them raise the rate, fewer
-// step each path faster (0.3 us a step alone, 0.9 us with four), and a launch waits for its
-// slowest paths, some ten times the mean, the more so the more heliospheres differ.  Measured in
-// paths per lane of one layer (one warp per scheduler), ms with 1 / 2 / 3 / 4 layers:
-// one heliosphere: 3: 40 / 46 / 50 / 56, 6: 39 / 42, 7: 46 / 43, 15: 65 / 61 / 64 / 65,
-// 20: - / 68 / 76 / 73, 40: - / 119 / 115 / 117; four: 5: 96 / 161 / 180 / 213, 7: 113 / 165,
-// 8: 116 / 141, 10: 133 / 135 / 190 / 202, 20: - / 202 / 206 / 252, 30: - / 273 / 262 / 299,
-// 60: - / 513 / 489 / 488; the same with FP64 sums: 5: 162 / 251, 7: 187 / 259, 10: 218 / 209,
-// 20: - / 298 / 278 / 274, 60: - / 737 / 656 / 645.
-int untuned_layers(uint64_t n_total, int sms, int max_blocks)
+// Blocks of 128 (warps per scheduler, "layers") of an untuned launch.  More of them raise the rate,
+// fewer step each path faster (0.3 us a step alone, 0.9 us with four), and a launch waits for its
+// slowest paths, some ten times the mean.  Those are among the n_long that are expected to be long
+// (a start key within a factor of three of the smallest).  Where they are few, they all start
+// first, and one layer is enough until the others' work takes longer than the longest path; where
+// most are (one energy, isotropic), the longest may be taken last, so all should start at once.
+// Measured in paths per lane of one layer, ms with 1 / 2 / 3 / 4 layers:
+// 30 energies (n_long 17 %): 3: 40 / 46 / 50 / 56, 6: 39 / 42, 8: 49 / 45 / 48 / 55, 15: 65 / 61 / 64 / 65,
+// 20: - / 68 / 76 / 73, 40: - / 119 / 115 / 117; four heliospheres (6 %): 5: 96 / 161 / 180 / 213,
+// 8: 116 / 141, 10: 133 / 135 / 190 / 202, 20: - / 202 / 206 / 252, 30: - / 273 / 262 / 299, 60: - / 513 /
+// 489 / 488, with FP64 sums 5: 162 / 251, 10: 218 / 209, 60: - / 737 / 656 / 645; one energy (100 %):
+// 1.5: 18 / 19 / 21 / 23, 3: 26 / 24 / 23 / 25, 5: 37 / 32 / 30 / 30, 7: 46 / 38 / 36 / 35; isotropic
+// (100 %): 2: 1.6 / 1.2 / 1.4 / 1.4, 4: 2.3 / 1.8 / 1.6 / 1.6, 7: 3.6 / 2.5 / 2.2 / 2.1.
+int untuned_layers(uint64_t n_total, uint64_t n_long, int sms, int max_blocks)
 {
     const uint64_t layer = (uint64_t)sms * 128u;
-    const int layers = n_total <= 7 * layer ? 1 : n_total <= 20 * layer ? 2 : n_total <= 40 * layer ? 3 : max_blocks;
+    int layers = n_total <= 10 * layer ? 1 : n_total <= 20 * layer ? 2 : n_total <= 40 * layer ? 3 : max_blocks;
+    const int start = (int)std::min<uint64_t>((n_long + layer * 4 / 5) / layer, (uint64_t)max_blocks);
+    layers = std::max(layers, n_long >= n_total / 2 ? start : std::min(start, 2));
     return std::max(1, std::min(layers, max_blocks));
 }
 
-PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_total)
+PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_total, uint64_t n_long)
 {
     unsigned block = (t && t->block) ? t->block : 128u;
     const unsigned period = t ? t->compact_period : 64u;
@@ -383,12 +400,14 @@ PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_to
     int max_b = mixed_max_blocks_per_sm(v, block);
     if (max_b < 1) max_b = 1;
     int bps = (t && t->blocks_per_sm) ? (int)t->blocks_per_sm : max_b;
-    if (!t) bps = untuned_layers(n_total, num_sms(), max_b);
+    const int untuned = untuned_layers(n_total, n_long, num_sms(), max_b);
+    if (!t) bps = untuned;
     // With the hand-over, no shape takes more than one warp per scheduler for up to six paths per
-    // lane: in every case measured (see untuned_layers) that is the fastest, and the launch is on its
-    // way there anyhow.  Four blocks of 128 asked for: 1.5e4 paths of one heliosphere 48.7 -> 31 ms,
-    // 4.8e4 of four 197 -> 98.
-    if (period != 0 && n_total <= 6ull * 128u * (uint64_t)num_sms() && block * (unsigned)std::min(bps, max_b) > 128u) {
+    // lane where an untuned launch takes one: in every such case measured that is the fastest, and
+    // the launch is on its way there anyhow.  Four blocks of 128 asked for: 1.5e4 paths of one
+    // heliosphere 48.7 -> 31 ms, 4.8e4 of four 197 -> 98.
+    if (period != 0 && untuned == 1 && n_total <= 6ull * 128u * (uint64_t)num_sms() &&
+        block * (unsigned)std::min(bps, max_b) > 128u) {
         block = 128u;
         bps = 1;
     }
@@ -558,7 +577,7 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
     DevSpecies *d_sp = nullptr;
     cosmica_status st = upload_species(m->spc, m->spc_stage, species, 1, s, &d_sp);
     if (st != COSMICA_OK) return st;
-    st = m->tab.build(its, pre, cost_order(its, &m->p, species), s);
+    st = m->tab.build(its, pre, cost_order(its, pre, &m->p, species, &m->tab.n_long), s);
     if (st != COSMICA_OK) return st;
 
     const bool host_out = !is_device_ptr(out->r);
@@ -579,7 +598,7 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
         Extensions ext;
         ext.add(m->p);
         const MixedVariant v{m->p.precision, m->p.formulation == 1, ext.kind(), full_model(m->p)};
-        e = launch_propagate_mixed(a, v, shape_for(v, nullptr, total), num_sms(), s);
+        e = launch_propagate_mixed(a, v, shape_for(v, nullptr, total, m->tab.n_long), num_sms(), s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
     if (host_out) return ExitStage::copy_back(ex, out, s);
@@ -990,13 +1009,13 @@ static cosmica_status batch_launch(cosmica_batch *b, uint64_t total, const ExitP
        "cudaMemsetAsync(counters)");
         cudaError_t e = (b->precision == COSMICA_PREC_FP64)
                             ? launch_propagate_fp64(a, fp64_variant(b->params.data(), b->params.size()), num_sms(), s)
-                            : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total), num_sms(), s);
+                            : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total, b->tab.n_long), num_sms(), s);
         if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
         return COSMICA_OK;
     };
     const bool graph = tuning && tuning->use_graph && s != nullptr;
     if (!graph) return direct();
-    const PersistentShape sh = shape_for(b->variant(), tuning, total);
+    const PersistentShape sh = shape_for(b->variant(), tuning, total, b->tab.n_long);
     cosmica_batch::GraphKey key;
     key.total = total;
     key.n_items = b->tab.n_items;
@@ -1052,8 +1071,9 @@ extern "C" cosmica_status cosmica_batch_run(cosmica_batch *b, const cosmica_work
     }
     if (!valid_exit(out)) return fail(COSMICA_ERR_INVALID, "exit-state arrays must be non-NULL");
     const bool by_cost = tuning ? tuning->queue_order != 0 : true;
-    st = b->tab.build(its, pre, by_cost ? cost_order(its, b->params.data(), b->species.data())
-                                        : std::vector<uint32_t>(), s);
+    std::vector<uint32_t> order = cost_order(its, pre, b->params.data(), b->species.data(), &b->tab.n_long);
+    if (!by_cost) order.clear();
+    st = b->tab.build(its, pre, order, s);
     if (st != COSMICA_OK) return st;
     if (b->params[0].formulation == 1 && !out->lw)
         return fail(COSMICA_ERR_INVALID, "the energy form needs out->lw");

@@ -147,7 +147,8 @@ inline DevItem make_item(double T, uint64_t first_pid, uint64_t seed, uint32_t p
     return it;
 }
 int num_sms();
-int untuned_layers(uint64_t n_total, int sms, int max_blocks);
+int untuned_layers(uint64_t n_total, uint64_t n_long, int sms, int max_blocks);
+double start_key(const cosmica_params &p, const cosmica_species &sp, double T, double r0);
 
 }  // namespace host
 }  // namespace cosmica

@@ -38,6 +38,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstring>
+#include <limits>
 #include <mutex>
 
 #include "common.cuh"
@@ -234,7 +235,13 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
         Extensions ext;
         ext.add(*params);
         const MixedVariant v{params->precision, params->formulation == 1, ext.kind(), full_model(*params)};
-        const int bps = untuned_layers(total, num_sms(), mixed_max_blocks_per_sm(v, block));
+        double least = std::numeric_limits<double>::infinity();
+        for (uint32_t i = 0; i < n_energies; ++i)
+            if (n_per_energy[i]) least = std::min(least, start_key(*params, *species, T_in[i], params->r0_AU));
+        uint64_t n_long = 0;
+        for (uint32_t i = 0; i < n_energies; ++i)
+            if (start_key(*params, *species, T_in[i], params->r0_AU) <= 3.0 * least) n_long += n_per_energy[i];
+        const int bps = untuned_layers(total, n_long, num_sms(), mixed_max_blocks_per_sm(v, block));
         const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms() * (uint64_t)bps, (total + 3) / 4);
         e = launch_propagate_mixed(a, v, PersistentShape{block, (unsigned)grid, 64u}, num_sms(), s);
     }

@@ -70,3 +70,17 @@ def test_without_allocation(precision):
                                      job.n_per_energy, 5, out)
         torch().cuda.synchronize()
         same(out.numpy(), ref, n)
+
+
+@pytest.mark.parametrize("T", [[1.0], [0.1, 1.0, 30.0, 100.0]])
+@pytest.mark.parametrize("per_lane", [1.19, 1.21, 2.5, 3.5, 6.5, 10.01])
+def test_untuned_layers(T, per_lane):
+    """Untuned launches on both sides of the lines between one and four warps per scheduler, all paths expected
+    to be long or few of them, the last energy empty: the single launch's records."""
+    n = int(per_lane * LAYER) // len(T)
+    p = dict(W.params(R_out=10.0), max_steps=800.0)
+    items = [(0, 0, t, n, 0, 4 + i) for i, t in enumerate(T)] + [(0, 0, 0.01, 0, 0, 9)]
+    b = cz.cosmica_batch_create([cz.make_params(p, cz.PREC_MIXED)], [cz.make_species(W.PROTON)])
+    ref = run(b, items, cz.cosmica_tuning(128, 0, 0, 0, 0))
+    same(run(b, items), ref, "untuned")
+    cz.cosmica_batch_destroy(b)
