@@ -152,7 +152,10 @@ __global__ void __launch_bounds__(kHistThreads) k_histogram(ExitPtrs ex, uint64_
     const uint32_t words = rows * stride;
     for (uint32_t w = threadIdx.x * 4; w < words; w += kHistThreads * 4)
         *reinterpret_cast<uint4 *>(cnt + w) = make_uint4(0u, 0u, 0u, 0u);   // words <= kHistWords, itself a multiple of 4
-    const uint32_t row0 = n_items <= rows ? 0u : ex.item[g0];
+    // the block's first item, which comes from the caller and may be any number: with row0 + rows <=
+    // n_items every counted row is one of the histogram's, and a valid item below row0 wraps to at
+    // least 2^32 - row0 > rows
+    const uint32_t row0 = n_items <= rows ? 0u : min(ex.item[g0], n_items - rows);
     __syncthreads();
     constexpr uint32_t U = 4;
     for (uint32_t k = 0; k < per; k += U) {
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(kHistThreads) k_histogram(ExitPtrs ex, uint64_
     }
     __syncthreads();
     for (uint32_t w = threadIdx.x; w < words; w += kHistThreads) {
-        const uint32_t c = cnt[w];      // nonzero only in rows of counted items, all below n_items
+        const uint32_t c = cnt[w];      // nonzero only in rows of valid items
         if (c) atomicAdd(hist + (unsigned long long)row0 * stride + w, (unsigned long long)c);
     }
 }
