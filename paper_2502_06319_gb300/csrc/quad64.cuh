@@ -268,13 +268,13 @@ __device__ __forceinline__ void quad_chain(const DevParams &p, const DevSpecies 
     const F64Params &d = p.d;
     const double r = x.r, th = x.th;
     const Head H = quad_head<false, false>(p, sp, S.tab, team, r, th, x.lnP);
-    bool odd_range = !lt(from_bits(bits(x.lnP) & 0x7FFFFFFFFFFFFFFFull), 700.0);
+    bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);
     double y[4], q[4];
     const double Or = d.Omega * r, rs = r * H.sn;
     team.recip4(H.V, rs, 1.0, 1.0, y);
     const double y_rs = y[1];
     const double phs = x.ph + quot(Or, H.V, y[0]);
-    odd_range |= !lt(phs, 1e6);
+    odd_range |= beyond(phs, kFarAngle);
     double sphs, cphs;
     team.sincos(S.tab, phs, sphs, cphs);
     const double diff = (0.5 * kPi + atan_in(d.ta * sphs)) - th;
@@ -364,7 +364,7 @@ __device__ __forceinline__ void quad_isotropic(const DevParams &p, const DevSpec
 {
     const F64Params &d = p.d;
     const double r = x.r, th = x.th, V = d.Vs;
-    const bool odd_range = !lt(from_bits(bits(x.lnP) & 0x7FFFFFFFFFFFFFFFull), 700.0);
+    const bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);
     double P, unused, sn, cs, y[4], y2[4], q[4];
     team.functions(S.tab, x.lnP, 0.0, th, P, unused, sn, cs);
     const double pn = quot(P, sp.aoz, sp.raoz);

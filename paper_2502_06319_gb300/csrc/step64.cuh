@@ -19,7 +19,8 @@
 //     the uniforms of the normals are integer operations;
 //   * sqrt and the elementary functions keep their operations (detmath64.cuh).
 // Whatever leaves the normal range (a pole hit exactly, an overflow) shows as a non-finite
-// state, and the step is then taken again by m64::em_step from the old state.
+// state, and the step is then taken again by m64::em_step from the old state; so is a step whose
+// ln P or angles are outside what the functions below take (odd_range).
 //
 // G lanes step one path together (G = 1: a lane a path).  The slot cost does not depend on
 // the active lanes, so a launch with fewer paths than lanes spreads each path's independent
@@ -42,6 +43,8 @@ namespace s64 {
 __device__ __forceinline__ uint64_t bits(double x) { return (uint64_t)__double_as_longlong(x); }
 __device__ __forceinline__ double from_bits(uint64_t b) { return __longlong_as_double((long long)b); }
 __device__ __forceinline__ bool lt(double a, double b) { return (int64_t)bits(a) < (int64_t)bits(b); }   // b >= 0, no NaN
+// |x| >= b, or a NaN, for a b whose low word is zero
+__device__ __forceinline__ bool beyond(double x, double b) { return ((uint32_t)__double2hiint(x) & 0x7FFFFFFFu) >= (uint32_t)__double2hiint(b); }
 // x > 0 for any x but a NaN, whose answer is no; a switch held as 0.0 or 1.0
 __device__ __forceinline__ bool positive(double x) { return (int64_t)bits(x) > 0 && (int64_t)bits(x) <= 0x7FF0000000000000ll; }
 __device__ __forceinline__ bool on(double x) { return __double2hiint(x) != 0; }
@@ -148,7 +151,9 @@ __device__ __forceinline__ void quadrant(int k, double sr, double cr, double &sn
     cs = neg_if(odd ? sr : cr, (k + 1) & 2);
 }
 
-// arguments with 0 <= x 2/pi + 1/2 < 2^20 (angles here are nonnegative and below a few hundred)
+// angles beyond this take the plain step: ifloor wants |x 2/pi + 1/2| < 2^20.  A start longitude is any
+// finite number, and a step from beside a pole can throw theta so far that its fold leaves nothing of it.
+constexpr double kFarAngle = 1e6;
 __device__ __forceinline__ double reduce(double x, int &k)
 {
     k = ifloor(x * dm::k2OverPi + 0.5);
@@ -321,7 +326,7 @@ struct Team {
             for (int j = 0; j < 4; ++j) s[j] = get(v, j);
         }
     }
-    // exp(x0), exp(x1), sin(th), cos(th) of nonnegative th: one lane each, one Horner form
+    // exp(x0), exp(x1), sin(th), cos(th): one lane each, one Horner form
     __device__ __forceinline__ void functions(const double *tab, double x0, double x1, double th, double &e0, double &e1,
                                               double &sn, double &cs) const
     {
@@ -433,7 +438,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
     } else {
         team.functions(tab, x.lnP, wnear ? scale2<1>(wabs) : 0.0, th, P, ew, sn, cs);
     }
-    bool odd_range = !lt(from_bits(bits(x.lnP) & 0x7FFFFFFFFFFFFFFFull), 700.0);   // exp, or floor, needs its own cases
+    bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);   // exp, or floor, needs its own cases
     double es = 0.0;
     bool snear = false;
     if (shock) {
@@ -519,7 +524,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
         const double G2 = Gam * Gam, og = 1.0 + G2, gg = og * og;
         const double dGam_dth = Gam * (cot - q4[3]);
         const double phs = x.ph + q4[1];
-        odd_range |= !lt(phs, 1e6);
+        odd_range |= beyond(phs, kFarAngle);
         double sphs = 0.0, cphs = 0.0;
         const bool hcs = on(p.hcs_on), any_hcs = team.any(hcs);
         if (any_hcs) {
