@@ -583,7 +583,7 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
                  m->tab.list, m->tab.list_cap, m->tab.counters + 2};
     cudaError_t e;
     if (m->p.precision == COSMICA_PREC_FP64) {
-        e = launch_propagate_fp64(a, fp64_variant(&m->p, 1), num_sms(), s);
+        e = launch_propagate_fp64(a, fp64_variant(&m->p, 1, species, 1), num_sms(), s);
     } else {
         Extensions ext;
         ext.add(m->p);
@@ -998,7 +998,8 @@ static cosmica_status batch_launch(cosmica_batch *b, uint64_t total, const ExitP
         CK(cudaMemsetAsync(b->tab.counters, 0, kLaunchCounters * sizeof(unsigned long long), s),
        "cudaMemsetAsync(counters)");
         cudaError_t e = (b->precision == COSMICA_PREC_FP64)
-                            ? launch_propagate_fp64(a, fp64_variant(b->params.data(), b->params.size()), num_sms(), s)
+                            ? launch_propagate_fp64(a, fp64_variant(b->params.data(), b->params.size(), b->species.data(),
+                                                                  b->species.size()), num_sms(), s)
                             : launch_propagate_mixed(a, b->variant(), shape_for(b->variant(), tuning, total, b->tab.n_long), num_sms(), s);
         if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
         return COSMICA_OK;

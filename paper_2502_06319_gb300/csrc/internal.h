@@ -115,9 +115,11 @@ void note_launch();
 
 cudaError_t launch_derive(DevParams *prm, uint32_t n, cudaStream_t s);
 cudaError_t launch_f32_table(const DevParams *prm, uint32_t n, float *table, cudaStream_t s);
-// variant of the FP64 kernels: extended sets (shells, squashed) take the plain step; iso: every set is isotropic
+// variant of the FP64 kernels
 struct Fp64Variant {
-    bool energy, extended, iso, aniso;   // iso / aniso: some set is (not) isotropic
+    bool energy;
+    bool plain;         // some set or species is not one of the fast step's (see fast_step_set): the plain step for all
+    bool iso, aniso;    // some set is (not) isotropic
 };
 // counters of a launch: queue cursor, steps, paths ended, and per kernel paths left and their cursor
 constexpr uint32_t kLaunchCounters = 3 + 2 * kMixedStages;
@@ -137,13 +139,36 @@ struct MixedVariant {
     int extended;   // Extensions::kind() of the launch's parameter sets
     bool full;      // every set is the full model: drift and current sheet on, adaptive step
 };
-inline Fp64Variant fp64_variant(const cosmica_params *ps, size_t n)
+// Sets and species of the FP64 fast step (step64.cuh): no shells, not squashed, and constants between
+// 1e-9 and 1e9 (times and step-rule factors: 1e-12 and 1e12).  With ln P and the angles in the range that
+// the step itself tests, no operand of its divisions then leaves the range for which they are the correctly
+// rounded ones (a shock width of 1e-310 AU, say, has no finite reciprocal).
+inline bool fast_step_set(const cosmica_params &p)
+{
+    auto in = [](double x) { return x >= 1e-9 && x <= 1e9; };
+    auto in12 = [](double x) { return x >= 1e-12 && x <= 1e12; };
+    if (p.n_shells > 0 || p.squashed != 0 || !in(p.K0) || !in(p.r_in_AU) || !in(p.R_out_AU)) return false;
+    if (p.R_ts_AU > 0.0 && !(in(p.R_ts_AU) && in(p.dts_AU) && in(p.ts_K_factor))) return false;
+    if (p.dt_fixed_day > 0.0) {
+        if (!in12(p.dt_fixed_day)) return false;
+    } else if (!in12(p.dt_min_day) || !in12(p.dt_max_day) || !(p.eps_adv == 0.0 || in12(p.eps_adv)) ||
+               !(p.eps_diff == 0.0 || in12(p.eps_diff))) {
+        return false;
+    }
+    if (p.isotropic) return p.V_const_kms == 0.0 || in(p.V_const_kms);
+    return in(p.kperp_r_frac) && in(p.kperp_th_frac) && in(p.B1AU_nT) && in(p.V_slow_kms) && in(p.V_fast_kms) &&
+           in(p.rot_period_day) && in(p.dlat_deg) && p.lat_fast_deg >= -1e9 && p.lat_fast_deg <= 1e9 &&
+           (!p.hcs_on || in(p.dcs_min_deg));
+}
+inline bool fast_step_species(const cosmica_species &s) { return s.m0_GeV >= 1e-9 && s.m0_GeV <= 1e9; }
+inline Fp64Variant fp64_variant(const cosmica_params *ps, size_t n, const cosmica_species *sp, size_t n_sp)
 {
     Fp64Variant v{ps[0].formulation == 1, false, false, false};
     for (size_t i = 0; i < n; ++i) {
-        v.extended = v.extended || ps[i].n_shells > 0 || ps[i].squashed != 0;
+        v.plain = v.plain || !fast_step_set(ps[i]);
         (ps[i].isotropic ? v.iso : v.aniso) = true;
     }
+    for (size_t i = 0; i < n_sp; ++i) v.plain = v.plain || !fast_step_species(sp[i]);
     return v;
 }
 // a set is the full model of the mixed kernels' FULL variant

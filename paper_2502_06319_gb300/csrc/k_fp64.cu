@@ -7,8 +7,9 @@
 //   k_finish64, k_quad64
 //                     the last paths of a launch, or all of a small one: teams of lanes,
 //                     then the four warps of a block
-//   k_propagate_fp64  sets with radial shells or a squashed heliosphere: one thread per
-//                     quasi-particle, the step as it is defined (model64.cuh)
+//   k_propagate_fp64  sets with radial shells or a squashed heliosphere, or with constants
+//                     outside the fast step's range: one thread per quasi-particle, the step
+//                     as it is defined (model64.cuh)
 //   k_debug_*         coefficient / RNG / elementary-function probes used by
 //                     the tests through cosmica_debug.h
 #include <algorithm>
@@ -576,7 +577,7 @@ cudaError_t launch_propagate_fp64(const LaunchArgs &a, Fp64Variant v, int sms, c
 {
     if (a.n_total == 0) return cudaSuccess;
     cudaGetLastError();
-    if (v.extended) {
+    if (v.plain) {
         k_propagate_fp64<<<grid_for(a.n_total, 128), 128, 0, s>>>(a.prm, a.spc, a.items, a.prefix, a.n_items,
                                                                  a.n_total, a.out, a.steps_total);
         note_launch();

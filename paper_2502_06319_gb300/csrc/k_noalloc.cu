@@ -229,7 +229,7 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
                  d_counters + 1, d_counters, nullptr, d_prefix, d_f32,
                  list, list_cap, d_counters + 2};
     if (params->precision == COSMICA_PREC_FP64) {
-        e = launch_propagate_fp64(a, fp64_variant(params, 1), num_sms(), s);
+        e = launch_propagate_fp64(a, fp64_variant(params, 1, species, 1), num_sms(), s);
     } else {
         const unsigned block = 128;
         Extensions ext;

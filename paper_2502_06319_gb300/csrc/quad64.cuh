@@ -268,7 +268,7 @@ __device__ __forceinline__ void quad_chain(const DevParams &p, const DevSpecies 
     const F64Params &d = p.d;
     const double r = x.r, th = x.th;
     const Head H = quad_head<false, false>(p, sp, S.tab, team, r, th, x.lnP);
-    bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);
+    bool odd_range = beyond(x.lnP, kFarLnP) | odd_theta(th);
     double y[4], q[4];
     const double Or = d.Omega * r, rs = r * H.sn;
     team.recip4(H.V, rs, 1.0, 1.0, y);
@@ -364,7 +364,7 @@ __device__ __forceinline__ void quad_isotropic(const DevParams &p, const DevSpec
 {
     const F64Params &d = p.d;
     const double r = x.r, th = x.th, V = d.Vs;
-    const bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);
+    const bool odd_range = beyond(x.lnP, kFarLnP) | odd_theta(th);
     double P, unused, sn, cs, y[4], y2[4], q[4];
     team.functions(S.tab, x.lnP, 0.0, th, P, unused, sn, cs);
     const double pn = quot(P, sp.aoz, sp.raoz);

@@ -20,7 +20,9 @@
 //   * sqrt and the elementary functions keep their operations (detmath64.cuh).
 // Whatever leaves the normal range (a pole hit exactly, an overflow) shows as a non-finite
 // state, and the step is then taken again by m64::em_step from the old state; so is a step whose
-// ln P or angles are outside what the functions below take (odd_range).
+// ln P or angles are outside the range of what is below (odd_range).  The constants' range is the
+// caller's to test (fast_step_set): comparisons and switches on the bits would let a NaN that a
+// division leaves there pass for a number.
 //
 // G lanes step one path together (G = 1: a lane a path).  The slot cost does not depend on
 // the active lanes, so a launch with fewer paths than lanes spreads each path's independent
@@ -80,6 +82,8 @@ __device__ __forceinline__ double uniform(uint32_t w)
 }
 
 // ---- divisions ---------------------------------------------------------------------
+// b between 2^-1000 and 2^1000, a zero or above 2^-960 in magnitude and the quotient a normal number (or a zero):
+// then nothing underflows.  b = 0 gives a NaN or an infinity.
 __device__ __forceinline__ double recip(double b)
 {
     double y;
@@ -154,6 +158,13 @@ __device__ __forceinline__ void quadrant(int k, double sr, double cr, double &sn
 // angles beyond this take the plain step: ifloor wants |x 2/pi + 1/2| < 2^20.  A start longitude is any
 // finite number, and a step from beside a pole can throw theta so far that its fold leaves nothing of it.
 constexpr double kFarAngle = 1e6;
+// So do P outside e^-40 .. e^40 GV and theta below 2^-100 (or negative): with them, and with the constants in
+// fast_step_set's range, the step's intermediate values stay between about 1e-290 and 1e290 or are zero.
+constexpr double kFarLnP = 40.0, kNearPole = 7.888609052210118e-31;
+__device__ __forceinline__ bool odd_theta(double th)
+{
+    return (uint32_t)(__double2hiint(th) - __double2hiint(kNearPole)) >= (uint32_t)(__double2hiint(kFarAngle) - __double2hiint(kNearPole));
+}
 __device__ __forceinline__ double reduce(double x, int &k)
 {
     k = ifloor(x * dm::k2OverPi + 0.5);
@@ -438,7 +449,7 @@ __device__ __forceinline__ void step(const DevParams &p, const DevSpecies &dsp, 
     } else {
         team.functions(tab, x.lnP, wnear ? scale2<1>(wabs) : 0.0, th, P, ew, sn, cs);
     }
-    bool odd_range = beyond(x.lnP, 700.0) | beyond(th, kFarAngle);   // exp, or floor, needs its own cases
+    bool odd_range = beyond(x.lnP, kFarLnP) | odd_theta(th);
     double es = 0.0;
     bool snear = false;
     if (shock) {
