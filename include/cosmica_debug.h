@@ -50,6 +50,14 @@ cosmica_status cosmica_debug_normals32(uint64_t seed, uint64_t pid0, uint32_t n,
  * 4 tanh, 5 atan) on device arrays x, y of length n. */
 cosmica_status cosmica_debug_fn64(int32_t which, uint32_t n, const double *x, double *y, void *stream);
 
+/* Pieces of the fast FP64 step, which replace IEEE operations and the functions of cosmica_debug_fn64 within
+ * the ranges given: 0 x / b (2^-1000 < b < 2^1000, x zero or above 2^-960, the quotient zero or normal),
+ * 1 floor(x) (|x| < 2^20), 2 (x + 1/2) 2^-32 (x a 32-bit count), 3 2 x (no subnormal x, 2 x finite),
+ * 4 exp (|x| < 700), 5 log (normal x > 0), 6 sin, 7 cos (|x| < 10^6), 8 cos again, its own form, 9 atan
+ * (finite x).  Device arrays x, y of length n, and b for code 0 (else NULL). */
+cosmica_status cosmica_debug_step64(int32_t which, uint32_t n, const double *x, const double *b, double *y,
+                                    void *stream);
+
 /* Coefficients of one step at n states (device double [4 n]: r, th, ph, lnP) for the
  * model's parameter set and `species`; precision 0 = FP64 evaluator, 1 = FP32 evaluator.
  * out: device double [n * COSMICA_DEBUG_EVAL_N]. */

@@ -167,11 +167,12 @@ def lib():
             L.cosmica_debug_normals64.argtypes = [C.c_uint64, C.c_uint64, C.c_uint32, C.c_uint32, P, P]
             L.cosmica_debug_normals32.argtypes = [C.c_uint64, C.c_uint64, C.c_uint32, C.c_uint32, P, P, P]
             L.cosmica_debug_fn64.argtypes = [C.c_int32, C.c_uint32, P, P, P]
+            L.cosmica_debug_step64.argtypes = [C.c_int32, C.c_uint32, P, P, P, P]
             L.cosmica_debug_eval.argtypes = [P, C.POINTER(cosmica_species), C.c_int32, C.c_uint32, P, P, P]
             for name in ("cosmica_model_create", "cosmica_propagate", "cosmica_spectrum", "cosmica_batch_create",
                          "cosmica_batch_run", "cosmica_batch_spectrum", "cosmica_batch_spectrum_hist", "cosmica_autotune", "cosmica_debug_philox",
                          "cosmica_debug_curand_philox", "cosmica_debug_normals64", "cosmica_debug_normals32", "cosmica_debug_fn64",
-                         "cosmica_debug_eval"):
+                         "cosmica_debug_step64", "cosmica_debug_eval"):
                 getattr(L, name).restype = s
             _lib = L
     return _lib
@@ -509,6 +510,14 @@ FN_CODES = {"exp": 0, "log": 1, "sin": 2, "cos": 3, "tanh": 4, "atan": 5}
 
 def cosmica_debug_fn64(name: str, x, y, stream=None):
     _check(lib().cosmica_debug_fn64(FN_CODES[name], x.numel(), _ptr(x), _ptr(y), _stream(stream)))
+
+
+STEP_CODES = {"quotient": 0, "floor": 1, "uniform": 2, "twice": 3, "exp": 4, "log": 5, "sin": 6, "cos": 7,
+              "cos alone": 8, "atan": 9}
+
+
+def cosmica_debug_step64(name: str, x, y, b=None, stream=None):
+    _check(lib().cosmica_debug_step64(STEP_CODES[name], x.numel(), _ptr(x), _ptr(b), _ptr(y), _stream(stream)))
 
 
 def cosmica_debug_eval(model: int, species: cosmica_species, precision: int, states, out, stream=None):

@@ -1336,6 +1336,15 @@ extern "C" cosmica_status cosmica_debug_fn64(int32_t which, uint32_t n, const do
     return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "elementary-function probe");
 }
 
+extern "C" cosmica_status cosmica_debug_step64(int32_t which, uint32_t n, const double *x, const double *b, double *y,
+                                               void *stream)
+{
+    if (which < 0 || which > 9) return fail(COSMICA_ERR_INVALID, "function code %d", which);
+    if (n && (!x || !y || (which == 0 && !b))) return fail(COSMICA_ERR_INVALID, "NULL array");
+    cudaError_t e = launch_debug_step64(which, n, x, b, y, (cudaStream_t)stream);
+    return e == cudaSuccess ? COSMICA_OK : cuda_fail(e, "fast-step probe");
+}
+
 extern "C" cosmica_status cosmica_debug_eval(cosmica_model *m, const cosmica_species *species, int32_t precision,
                                              uint32_t n, const double *states, double *out, void *stream)
 {

@@ -221,6 +221,7 @@ cudaError_t launch_debug_eval64(const DevParams *prm, const DevSpecies *spc, uin
 cudaError_t launch_debug_eval32(const DevParams *prm, const DevSpecies *spc, uint32_t n, const double *st,
                                 double *out, cudaStream_t s);
 cudaError_t launch_debug_fn64(int which, uint32_t n, const double *x, double *y, cudaStream_t s);
+cudaError_t launch_debug_step64(int which, uint32_t n, const double *x, const double *b, double *y, cudaStream_t s);
 cudaError_t launch_debug_normals64(uint64_t seed, uint64_t pid0, uint32_t n, uint32_t step, double *z,
                                    cudaStream_t s);
 cudaError_t launch_debug_normals32(uint64_t seed, uint64_t pid0, uint32_t n, uint32_t step, float *z,

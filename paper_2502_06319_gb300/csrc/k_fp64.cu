@@ -487,6 +487,28 @@ __global__ void k_debug_fn64(int which, uint32_t n, const double *__restrict__ x
     }
 }
 
+// pieces of the fast step (step64.cuh)
+__global__ void k_debug_step64(int which, uint32_t n, const double *__restrict__ x, const double *__restrict__ b,
+                               double *__restrict__ y)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double v = x[i];
+    double s, c;
+    switch (which) {
+    case 0: y[i] = s64::quot(v, b[i], s64::recip(b[i])); break;
+    case 1: y[i] = s64::from_int(s64::ifloor(v)); break;
+    case 2: y[i] = s64::uniform((uint32_t)v); break;
+    case 3: y[i] = s64::scale2<1>(v); break;
+    case 4: y[i] = s64::exp_in(v); break;
+    case 5: y[i] = s64::log_in(v); break;
+    case 6: s64::sincos_in(v, s, c); y[i] = s; break;
+    case 7: s64::sincos_in(v, s, c); y[i] = c; break;
+    case 8: y[i] = s64::cos_in(v); break;
+    default: y[i] = s64::atan_in(v); break;
+    }
+}
+
 __global__ void k_debug_normals64(uint64_t seed, uint64_t pid0, uint32_t n, uint32_t step, double *z)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -603,6 +625,15 @@ cudaError_t launch_debug_fn64(int which, uint32_t n, const double *x, double *y,
     if (n == 0) return cudaSuccess;
     cudaGetLastError();
     k_debug_fn64<<<grid_for(n, 256), 256, 0, s>>>(which, n, x, y);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_debug_step64(int which, uint32_t n, const double *x, const double *b, double *y, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    cudaGetLastError();
+    k_debug_step64<<<grid_for(n, 256), 256, 0, s>>>(which, n, x, b, y);
     note_launch();
     return cudaGetLastError();
 }
