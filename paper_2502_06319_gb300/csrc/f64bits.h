@@ -39,7 +39,8 @@ COSMICA_HD uint64_t widen(uint32_t u)
     return ((uint64_t)hi << 32) | (none ? 0u : u << 29);
 }
 
-// FP64 -> FP32, round to nearest even, for finite |x| < 2^127 (below 2^-126: zero).
+// FP64 -> FP32, round to nearest even, for |x| < 2^128 (below 2^-126: zero); infinite or a NaN from there to
+// 2^129.  Above, and for an infinity or a NaN, a finite number: the caller sees to it that none comes here.
 COSMICA_HD uint32_t narrow(uint64_t x)
 {
     const uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;

@@ -171,12 +171,13 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     // As in the compensated state.  The FP64 sums take 64 clocks each, one after the other, so the
     // step's vote does not wait for them: it looks at the FP32 sums, whose error (two roundings,
     // under 2.4e-7 of r and of 2 pi) is far inside the margins, and the sums' finiteness follows
-    // from that of the increments.  theta first: the next step's longest chain starts from it.
+    // from that of the increments (an infinite r has to be seen here: narrow() makes it 1).
+    // theta first: the next step's longest chain starts from it.
     template <bool P>
     __device__ bool add(float fr, float fth, float fph, float dr, float dth, float dph, float dlnP, float dt, float, bool sphere)
     {
         const float nr = fr + dr, nth = fth + dth, nph = fph + dph;
-        const bool still = (nr > r_lo) & (!sphere | (nr < r_hi)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
+        const bool still = (nr > r_lo) & (nr < (sphere ? r_hi : 1e30f)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
                            (nph < 6.28317f) & isfinite(dlnP + dt);
         th += widen64(dth); r += widen64(dr);
         if (P) lnP += widen64(dlnP);
@@ -256,7 +257,7 @@ struct EnergyAcc<COSMICA_PREC_MIXED_F64ACC, true> {
     __device__ float fT() const { return narrow64(T); }
     __device__ void add(float dT, float dLam)
     {
-        T += widen64(dT);
+        T += widen64(fminf(dT, 3.402823466e38f));   // an infinite T would be 1 to narrow(), 2^128 and more is infinite
         Lam += widen64(dLam);
     }
     __device__ double T64() const { return T; }
