@@ -78,7 +78,8 @@ struct DevParams {
     double n_shells, shell_w;  // radial shells (0: one region), blend half-width [AU]
     double squashed, nose_th, nose_ph, ts_tail, ts_flank, hp_tail, hp_flank;   // nose-squashed surfaces
     double shell_K0[COSMICA_MAX_SHELLS], shell_tilt_deg[COSMICA_MAX_SHELLS];
-    int32_t precision, pad;
+    int32_t precision;
+    float vote_lo;             // derived: f64bits::vote_floor of r_in and the outer boundary's farthest point
     // derived on the device
     double B0;                 // nT, |B|(1 AU, equator) = B1AU
     F64Params d;

@@ -92,6 +92,13 @@ COSMICA_HD uint64_t from_u32(uint32_t n)
     return ((uint64_t)(1053 - sh) << 52) + ((uint64_t)(n << sh) << 21);   // the leading one carries into the exponent
 }
 
+// Bounds for an FP32 sum n = fr + dr, r an FP64 number with the FP32 value fr, 0 <= r <= reach: above the floor
+// and below the ceiling, r + dr is at least r_in and below R.  n is off by up to 2^-24 r and 2^-24 of itself; the
+// first counts where a step from far out ends beside r_in, hence the share of reach.
+COSMICA_HD float vote_floor(float r_in, float reach) { return r_in * 1.000001f + reach * 2.4e-7f; }
+COSMICA_HD float vote_ceiling(float R) { return R * 0.999999f; }
+constexpr float kNoCeiling = 1e30f;      // where another test bounds r: keeps an infinity out
+
 // FP64 comparisons on the bits, with b > 0 finite: right for every a but NaN.
 COSMICA_HD bool less(uint64_t a, uint64_t b) { return (int64_t)a < (int64_t)b; }
 // a < 0 or a > b (a = -0 counts as below 0: the caller decides with FP64 comparisons then)

@@ -30,6 +30,8 @@ __global__ void k_derive(DevParams *prm, uint32_t n)
     DevParams &p = prm[i];
     const bool iso = p.isotropic != 0.0;
     p.B0 = iso ? 0.0 : m64::field_B0(p);
+    // (a spheroid's points are within its tail distance and its flank semi-axis of the Sun, together)
+    p.vote_lo = f64bits::vote_floor((float)p.r_in, (float)(p.squashed != 0.0 ? p.R_out * (1.0 + p.hp_tail + p.hp_flank) : p.R_out));
     {
         // in the operations of model64.cuh
         F64Params &d = p.d;

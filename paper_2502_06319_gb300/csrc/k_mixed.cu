@@ -56,7 +56,7 @@ __device__ __forceinline__ void begin(const LaunchArgs &a, uint32_t it, uint64_t
     L.k = 0;
     L.max_steps = (uint32_t)p.max_steps;
     // item.T: T of the energy form (whose ln P follows from T), ln P0 of the momentum form
-    x.init(item.r0, item.th0, item.ph0, EN ? 1.0 : item.T, p.R_out, p.f.r_in);
+    x.init(item.r0, item.th0, item.ph0, EN ? 1.0 : item.T, p.R_out, p.f.r_in, p.vote_lo);
     if constexpr (EN) en.init(item.T, (float)sp.m0, sp.aoz);
 }
 
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedS
     EnergyAcc<ACC, EN> en{};
     // lanes that never get a path step an unremarkable state of the first set
     L.q = a.f32;
-    x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f);
+    x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f, 0.11f);
     en.init(1.0, 1.0f, 1.0f);
     // a source smaller than the grid is spread evenly over the warps
     const uint64_t n = st.from ? *st.n_from : a.n_total;

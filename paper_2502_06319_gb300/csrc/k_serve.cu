@@ -44,7 +44,7 @@ __device__ __forceinline__ void save(const Acc<COSMICA_PREC_MIXED> &x, Suspended
 template <>
 __device__ __forceinline__ void load(Acc<COSMICA_PREC_MIXED> &x, const Suspended &s, const DevParams &p)
 {
-    x.init(p.r0, p.th0, p.ph0, 0.0, p.R_out, p.f.r_in);
+    x.init(p.r0, p.th0, p.ph0, 0.0, p.R_out, p.f.r_in, p.vote_lo);
     x.r.hi = s.f[0]; x.r.lo = s.f[1]; x.th.hi = s.f[2]; x.th.lo = s.f[3]; x.ph.hi = s.f[4];
     x.ph.lo = s.f[5];
     x.Ps.set(m32::FF{s.f[6], s.f[7]}, m32::FF{s.f[8], s.f[9]});
@@ -57,7 +57,7 @@ __device__ __forceinline__ void save(const Acc<COSMICA_PREC_MIXED_F64ACC> &x, Su
 template <>
 __device__ __forceinline__ void load(Acc<COSMICA_PREC_MIXED_F64ACC> &x, const Suspended &s, const DevParams &p)
 {
-    x.init(s.d[0], s.d[1], s.d[2], s.d[3], p.R_out, p.f.r_in);
+    x.init(s.d[0], s.d[1], s.d[2], s.d[3], p.R_out, p.f.r_in, p.vote_lo);
     x.s = s.d[4];
 }
 
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
     Acc<ACC> x{};
     // lanes that never get a particle step an unremarkable state of the first slot
     S.L.q = reinterpret_cast<const float *>(&a.prm[0].f);
-    x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f);
+    x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f, 0.11f);
     // fewer particles than lanes are spread evenly over the warps
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     const bool seat = lane < (a.n_resume + a.n_fresh + warps - 1) / warps;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
                         S.exit_idx = item.exit_idx + off;
                         const double T = item.T;
                         const double P0 = sp.A / fabs(sp.Z) * sqrt(T * (T + 2.0 * sp.m0));
-                        x.init(p.r0, p.th0, p.ph0, log(P0), p.R_out, p.f.r_in);
+                        x.init(p.r0, p.th0, p.ph0, log(P0), p.R_out, p.f.r_in, p.vote_lo);
                         m32::normals(S.L.seed, S.L.pid, S.L.k, z0, z1, z2);
                         active = true;
                     } else {

@@ -34,7 +34,7 @@ struct Acc<COSMICA_PREC_MIXED> {
     m32::FF2 Ps;   // lnP and s, the two that no boundary touches, as packed pairs
     m32::FF Rout;
     float r_in2;   // 2 r_in
-    __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in)
+    __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in, float)
     {
         r = m32::ff_from_double(r0);
         th = m32::ff_from_double(th0);
@@ -147,11 +147,11 @@ template <>
 struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     double r, th, ph, lnP, s, Rout, r_in;
     float r_lo, r_hi;      // a little inside (r_in, R_out), see add()
-    __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in_f)
+    __device__ void init(double r0, double th0, double ph0, double lnP0, double R_out, float r_in_f, float vote_lo)
     {
         r = r0; th = th0; ph = ph0; lnP = lnP0; s = 0.0; Rout = R_out; r_in = (double)r_in_f;
-        r_lo = r_in_f * 1.000001f;
-        r_hi = (float)R_out * 0.999999f;
+        r_lo = vote_lo;
+        r_hi = f64bits::vote_ceiling((float)R_out);
     }
     __device__ float fr() const { return narrow64(r); }
     __device__ float fth() const { return narrow64(th); }
@@ -170,14 +170,14 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     }
     // As in the compensated state.  The FP64 sums take 64 clocks each, one after the other, so the
     // step's vote does not wait for them: it looks at the FP32 sums, whose error (two roundings,
-    // under 2.4e-7 of r and of 2 pi) is far inside the margins, and the sums' finiteness follows
+    // under 2.4e-7 of the largest r and of 2 pi) is inside the margins, and the sums' finiteness follows
     // from that of the increments (an infinite r has to be seen here: narrow() makes it 1).
     // theta first: the next step's longest chain starts from it.
     template <bool P>
     __device__ bool add(float fr, float fth, float fph, float dr, float dth, float dph, float dlnP, float dt, float, bool sphere)
     {
         const float nr = fr + dr, nth = fth + dth, nph = fph + dph;
-        const bool still = (nr > r_lo) & (nr < (sphere ? r_hi : 1e30f)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
+        const bool still = (nr > r_lo) & (nr < (sphere ? r_hi : f64bits::kNoCeiling)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
                            (nph < 6.28317f) & isfinite(dlnP + dt);
         th += widen64(dth); r += widen64(dr);
         if (P) lnP += widen64(dlnP);
