@@ -201,7 +201,7 @@ cudaError_t launch_histogram(const ExitPtrs &ex, uint64_t n, uint32_t n_items, u
                              double dx, unsigned long long *hist, const WeightTable &wt, int sms, cudaStream_t s);
 // weights: from launch_histogram, or null (every item evaluates its own); sums: scratch of
 // n_items x spectrum_sums_bytes()
-size_t spectrum_sums_bytes();
+constexpr size_t spectrum_sums_bytes() { return 24; }
 cudaError_t launch_spectrum(const unsigned long long *hist, uint32_t n_items, uint32_t nbins,
                             double x_lo, double dx, const SpecItem *items, const double *weights, int lis_kind,
                             const double *lis_lnT, const double *lis_lnJ, uint32_t lis_n, void *sums,

@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_spec_clear(unsigned long long 
 struct SpecSums {
     double N, mu, S2;      // EXIT paths in the bins, mean weight, sum of c (w - mu)^2
 };
+static_assert(sizeof(SpecSums) == spectrum_sums_bytes(), "scratch of the callers");
 
 __device__ __forceinline__ void finish_spectrum(const SpecItem &it, double N, double mu, double S2, double *J, double *sigma)
 {
@@ -512,7 +513,6 @@ uint32_t unbinned_per_thread(const uint32_t *n_per_item, uint32_t n_items, int s
     }
     return best;
 }
-size_t spectrum_sums_bytes() { return sizeof(SpecSums); }
 size_t unbinned_partial_bytes() { return sizeof(UnbPartial); }
 
 cudaError_t launch_spectrum_unbinned(const ExitPtrs &ex, const uint64_t *prefix, const uint64_t *chunk_prefix,

@@ -37,6 +37,11 @@ constexpr uint32_t kMaxSlots = 256;
 constexpr uint32_t kMaxEnergies = 256;
 constexpr uint32_t kMaxBins = 8192;
 
+// a retiring request's scratch (see retire): ends of its sums and of its bin weights, and its size
+constexpr size_t kRetireSums = 256 + kMaxEnergies * spectrum_sums_bytes();
+constexpr size_t kRetireWeights = kRetireSums + kMaxBins * sizeof(double);
+constexpr size_t kRetireScratch = kRetireWeights + kMaxEnergies * sizeof(SpecItem);
+
 // device counters of the server, read back as one block after each quantum
 struct Control {
     unsigned long long cursors[2];        // cleared before each quantum, like n_susp
@@ -124,8 +129,7 @@ struct cosmica_server {
     Control *d_ctl = nullptr;
     unsigned long long *d_hist = nullptr;
     double *d_J = nullptr, *d_S = nullptr;
-    SpecItem *d_spec_items = nullptr;
-    DevBuf tables, weights;
+    DevBuf tables;
     Staging stage;
     Control *h_ctl = nullptr;   // pinned read-back after each quantum
     // host bookkeeping (guarded by mu)
@@ -188,18 +192,17 @@ bool cosmica_server::retire(uint64_t ticket, Req &r)
     r.H.assign((size_t)nE * stride, 0);
     r.J.assign(nE, 0.0);
     r.S.assign(nE, 0.0);
-    // bin weights of the request's one species, and its number of an item that has it (0)
-    const size_t b_sums = align_up(nE * spectrum_sums_bytes(), 256);
-    if (weights.reserve(256 + b_sums + (size_t)nb * sizeof(double)) != COSMICA_OK) {
-        set_failed(std::string("server retire: ") + cosmica_last_error());
-        return false;
-    }
-    void *d_sums = (char *)weights.d + 256;
-    double *d_w = (double *)((char *)weights.d + 256 + b_sums);
-    cudaError_t e = cudaMemsetAsync(weights.d, 0, 256, stream);
+    // scratch in the resume list that the last quantum has used up (no more than kRetireScratch): the number of an
+    // item that has the request's one species (0), sums and bin weights, items
+    char *const scratch = (char *)d_susp[cur ^ 1];
+    const uint32_t *d_sp_item = (const uint32_t *)scratch;
+    void *d_sums = scratch + 256;
+    double *d_w = (double *)(scratch + kRetireSums);
+    SpecItem *d_spec_items = (SpecItem *)(scratch + kRetireWeights);
+    cudaError_t e = cudaMemsetAsync(scratch, 0, 256, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_spec_items, its.data(), nE * sizeof(SpecItem),
                                               cudaMemcpyHostToDevice, stream);
-    const WeightTable wt{d_spec_items, (const uint32_t *)weights.d, 1, 0, nullptr, nullptr, 0, d_w};
+    const WeightTable wt{d_spec_items, d_sp_item, 1, 0, nullptr, nullptr, 0, d_w};
     if (e == cudaSuccess) e = launch_spec_clear(d_hist, (uint64_t)nE * stride, stream);
     if (e == cudaSuccess) e = launch_histogram(ex, r.total, nE, nb, x_lo, dx, d_hist, wt, num_sms(), stream);
     if (e == cudaSuccess)
@@ -394,8 +397,10 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     const int bps = std::max(1, serve_max_blocks_per_sm(precision, 0, true, block));
     s->shape = PersistentShape{block, (unsigned)(num_sms() * bps), 0u};
     s->lane_cap = (uint64_t)s->shape.grid * block;
-    const size_t fixed = 2 * s->lane_cap * sizeof(Suspended) + kMaxSlots * (sizeof(DevParams) + sizeof(DevSpecies) + 12) +
-                         (size_t)kMaxEnergies * (kMaxBins + 3) * 8 + kMaxEnergies * 48 + 4096;
+    const size_t b_susp = std::max<size_t>(s->lane_cap * sizeof(Suspended), kRetireScratch);
+    // with 12 KB for what the allocations are rounded up by
+    const size_t fixed = 2 * b_susp + kMaxSlots * (sizeof(DevParams) + sizeof(DevSpecies) + 12) +
+                         (size_t)kMaxEnergies * (kMaxBins + 3) * 8 + kMaxEnergies * 16 + 12288;
     const size_t per = 5 * 8 + 4 + 4 + 1;
     if (mem_budget <= fixed + 256 * per) {
         delete s;
@@ -411,12 +416,11 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     A((void **)&s->d_ctl, b_ctl + b_prm + kMaxSlots * sizeof(DevSpecies));
     s->d_prm = (DevParams *)((char *)s->d_ctl + b_ctl);
     s->d_spc = (DevSpecies *)((char *)s->d_prm + b_prm);
-    A((void **)&s->d_susp[0], s->lane_cap * sizeof(Suspended));
-    A((void **)&s->d_susp[1], s->lane_cap * sizeof(Suspended));
+    A((void **)&s->d_susp[0], b_susp);
+    A((void **)&s->d_susp[1], b_susp);
     A((void **)&s->d_hist, (size_t)kMaxEnergies * (kMaxBins + 3) * 8);
     A((void **)&s->d_J, kMaxEnergies * 8);
     A((void **)&s->d_S, kMaxEnergies * 8);
-    A((void **)&s->d_spec_items, kMaxEnergies * sizeof(SpecItem));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_ctl, sizeof(Control));
     // lanes without a particle read slot 0's parameters (zero: no shells, so no table index)
     if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, b_ctl + sizeof(DevParams));
@@ -556,10 +560,8 @@ extern "C" void cosmica_server_destroy(cosmica_server *s)
     if (s->th.joinable()) s->th.join();
     if (s->stream) cudaStreamSynchronize(s->stream);
     s->tables.release();
-    s->weights.release();
     s->stage.release();
-    void *dev[] = {s->arena_mem, s->d_ctl, s->d_susp[0], s->d_susp[1], s->d_hist,
-                   s->d_J, s->d_S, s->d_spec_items};
+    void *dev[] = {s->arena_mem, s->d_ctl, s->d_susp[0], s->d_susp[1], s->d_hist, s->d_J, s->d_S};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (s->h_ctl) cudaFreeHost(s->h_ctl);
