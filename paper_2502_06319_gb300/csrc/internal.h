@@ -86,6 +86,7 @@ struct ServeArgs {
     unsigned int *req_done;        // per slot
     unsigned long long *req_steps; // per slot
     uint32_t budget;               // steps per lane per quantum
+    uint32_t idle_slot;            // a resident request's: its parameters are stepped by lanes without a particle
 };
 
 // ext: Extensions::kind() of the resident requests; full: every one is the full model (the variant

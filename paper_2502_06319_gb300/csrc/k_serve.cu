@@ -78,8 +78,9 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
     const unsigned lane = threadIdx.x & 31u;
     ServeLane S{};
     Acc<ACC> x{};
-    // lanes that never get a particle step an unremarkable state of the first slot
-    S.L.q = reinterpret_cast<const float *>(&a.prm[0].f);
+    // lanes that never get a particle step an unremarkable state of a resident request (whose set has the
+    // extensions EXT says: a set without shells has no shell to look up)
+    S.L.q = reinterpret_cast<const float *>(&a.prm[a.idle_slot].f);
     x.init(1.0, 1.0, 1.0, 1.0, 2.0, 0.1f, 0.11f);
     // fewer particles than lanes are spread evenly over the warps
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);

@@ -244,12 +244,14 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
     std::vector<std::pair<uint64_t, uint32_t>> owner;   // (ticket, energy) per item
     Extensions ext;
     bool full = true;   // every resident request is the full model
+    uint32_t idle_slot = 0;
     {
         std::lock_guard<std::mutex> lk(mu);
         for (auto &kv : reqs) {
             Req &r = kv.second;
             if (r.state != 1) continue;
             ext.add(r.p);
+            idle_slot = (uint32_t)r.slot;
             full = full && full_model(r.p);
             for (uint32_t e = 0; e < r.T.size(); ++e) {
                 const uint64_t left = r.n[e] - r.started[e];
@@ -293,6 +295,7 @@ bool cosmica_server::quantum(std::vector<uint64_t> &admitted_now)
     a.req_done = d_ctl->done;
     a.req_steps = d_ctl->steps;
     a.budget = budget;
+    a.idle_slot = idle_slot;
     // no more warps per scheduler than the particles fill: fewer step faster
     PersistentShape q = shape;
     const uint64_t layer = (uint64_t)num_sms() * shape.block;
@@ -422,8 +425,7 @@ extern "C" cosmica_status cosmica_server_create(size_t mem_budget, int32_t preci
     A((void **)&s->d_J, kMaxEnergies * 8);
     A((void **)&s->d_S, kMaxEnergies * 8);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&s->h_ctl, sizeof(Control));
-    // lanes without a particle read slot 0's parameters (zero: no shells, so no table index)
-    if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, b_ctl + sizeof(DevParams));
+    if (e == cudaSuccess) e = cudaMemset(s->d_ctl, 0, b_ctl);
     if (e != cudaSuccess) {
         cosmica_status rs = cuda_fail(e, "server allocation");
         cosmica_server_destroy(s);

@@ -1,5 +1,5 @@
-"""Requests of the largest size that retire while others are suspended: their spectra are formed in the server's own
-buffers, beside which the suspended particles wait."""
+"""Requests that retire while others are suspended: the largest ones, whose spectra are formed in the server's own
+buffers beside the suspended particles, and one after which no resident set is of the kind of the freed slot's."""
 import numpy as np
 import pytest
 
@@ -36,3 +36,24 @@ def test_largest_requests_beside_suspended_ones(precision):
         # the same sums in the same order
         assert np.allclose(got[i].J, J, rtol=1e-14, atol=0, equal_nan=True)
         assert np.allclose(got[i].sigma, S, rtol=1e-12, atol=0, equal_nan=True)
+
+
+@pytest.mark.parametrize("precision", [cz.PREC_MIXED, cz.PREC_MIXED_F64ACC])
+def test_shells_after_a_plain_set_in_the_first_slot(precision):
+    """A short request without shells takes the first slot and retires; the few particles of the ones with shells that
+    are left share their warps with lanes that have none."""
+    shells = dict(W.shell_params(W.solar_cycle_series(), 40, n_shells=5, R_ts=30.0, R_out=50.0), max_steps=3e6)
+    cases = [(W.params(R_out=2.0), [50.0], [8]), (shells, [0.5], [37]), (shells, [1.0], [5])]
+    srv = cz.cosmica_server_create(256 << 20, precision, budget_steps=64)
+    reqs = [cz.Request(cz.make_params(p, precision), cz.make_species(W.PROTON), T, n, 9, cz.make_bins(0.1, 1000.0, 32))
+            for p, T, n in cases]
+    tickets = [cz.cosmica_server_submit(srv, q) for q in reqs]
+    got = [cz.Result(1, 32) for _ in reqs]
+    for t, r in zip(tickets, got):
+        cz.cosmica_server_wait(srv, t, r)
+    cz.cosmica_server_destroy(srv)
+    assert got[0].c.t_done < got[1].c.t_done
+    for (p, T, n), r in zip(cases, got):
+        ref, _, m = gpu_run(W.Job(p, W.PROTON, T, n, 9), precision=precision)
+        m.close()
+        assert int(r.steps) == int(ref["steps"].astype(np.int64).sum())
