@@ -387,7 +387,10 @@ typedef struct {
  * cosmica_propagate_noalloc. */
 typedef struct {
     uint32_t block;           /* threads per block (32..256; 0 = 128)                   */
-    uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit)  */
+    uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit);
+                                 with a compact_period, one of 128 threads at most for up
+                                 to 768 particles per SM, if an untuned launch takes
+                                 one, which is then faster                              */
     uint32_t compact_period;  /* once the queue is drained, every this many steps the
                                  launch looks whether the particles left fit fewer warps,
                                  which then take them over (0 = never)                   */

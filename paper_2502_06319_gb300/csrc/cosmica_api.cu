@@ -400,7 +400,17 @@ PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_to
     int max_b = mixed_max_blocks_per_sm(v, block);
     if (max_b < 1) max_b = 1;
     int bps = (t && t->blocks_per_sm) ? (int)t->blocks_per_sm : max_b;
-    if (!t) bps = untuned_layers(n_total, n_long, num_sms(), max_b);
+    const int untuned = untuned_layers(n_total, n_long, num_sms(), max_b);
+    if (!t) bps = untuned;
+    // With the hand-over, no shape takes more than one warp per scheduler for up to six paths per
+    // lane where an untuned launch takes one: in every such case measured that is the fastest, and
+    // the launch is on its way there anyhow.  Four blocks of 128 asked for: 1.5e4 paths of one
+    // heliosphere 48.7 -> 31 ms, 4.8e4 of four 197 -> 98.
+    if (period != 0 && untuned == 1 && n_total <= 6ull * 128u * (uint64_t)num_sms() &&
+        block * (unsigned)std::min(bps, max_b) > 128u) {
+        block = 128u;
+        bps = 1;
+    }
     bps = std::min(bps, max_b);
     uint64_t grid = (uint64_t)num_sms() * (uint64_t)bps;
     // never more warps than paths (the kernel spreads them evenly)
