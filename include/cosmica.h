@@ -387,13 +387,14 @@ typedef struct {
  * cosmica_propagate_noalloc. */
 typedef struct {
     uint32_t block;           /* threads per block (32..256; 0 = 128)                   */
-    uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit);
-                                 with a compact_period, one of 128 threads at most for up
-                                 to 768 particles per SM, if an untuned launch takes
-                                 one, which is then faster                              */
+    uint32_t blocks_per_sm;   /* resident blocks per SM requested (0 = as many as fit) */
     uint32_t compact_period;  /* once the queue is drained, every this many steps the
                                  launch looks whether the particles left fit fewer warps,
-                                 which then take them over (0 = never)                   */
+                                 which then take them over (0 = never).  With a period
+                                 the launch may start there: up to 768 particles per SM run
+                                 with one block of 128 per SM, whatever block and
+                                 blocks_per_sm say, if an untuned launch of them would,
+                                 which is then faster.  With 0 the shape is as given      */
     uint32_t use_graph;       /* 1: replay the launch as a CUDA graph                   */
     uint32_t queue_order;     /* 0: items in the given order; 1: items with the lowest
                                  K0 beta P first (longest paths first); exit records keep
@@ -454,8 +455,8 @@ cosmica_status cosmica_batch_spectrum_hist(cosmica_batch *batch, const cosmica_w
  * `items` (host; ~10 and ~30 particles per slot), from which each candidate's
  * time for the whole batch is extrapolated linearly in the particle count.  Results are cached for the
  * process per device and configuration class (precision, drift, termination
- * shock, particle count within a factor of two, kernel variant); a cached
- * class returns at once.  Synchronous; uses the batch's own scratch.  An FP64
+ * shock, particle count within a factor of two, blocks per SM of an untuned
+ * launch, kernel variant); a cached class returns at once.  Synchronous; uses the batch's own scratch.  An FP64
  * batch needs no tuning and gets block 128 and period 0.  Errors:
  * INVALID (NULL batch/best, invalid items, no particles), OOM, CUDA. */
 cosmica_status cosmica_autotune(cosmica_batch *batch, const cosmica_work_item *items,

@@ -392,31 +392,37 @@ int untuned_layers(uint64_t n_total, uint64_t n_long, int sms, int max_blocks)
     return std::max(1, std::min(layers, max_blocks));
 }
 
-PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_total, uint64_t n_long)
+// The block size, blocks per SM and period that a launch of n_total particles runs with when t asks for a shape
+// (the other fields of *t do not matter).
+// With the hand-over, no shape takes more than one warp per scheduler for up to six paths per lane where an
+// untuned launch takes one: in every such case measured that is the fastest, and the launch is on its way there
+// anyhow.  Four blocks of 128 asked for: 1.5e4 paths of one heliosphere 48.7 ms as asked, 31 as taken, 4.8e4 of
+// four 197 and 98.  A shape without the hand-over is taken as it is.
+cosmica_tuning taken_shape(MixedVariant v, const cosmica_tuning *t, uint64_t n_total, uint64_t n_long)
 {
-    unsigned block = (t && t->block) ? t->block : 128u;
-    const unsigned period = t ? t->compact_period : 64u;
-    block = std::min(256u, std::max(32u, block / 32u * 32u));
-    int max_b = mixed_max_blocks_per_sm(v, block);
-    if (max_b < 1) max_b = 1;
-    int bps = (t && t->blocks_per_sm) ? (int)t->blocks_per_sm : max_b;
+    cosmica_tuning r{};
+    r.block = std::min(256u, std::max(32u, ((t && t->block) ? t->block : 128u) / 32u * 32u));
+    r.compact_period = t ? t->compact_period : 64u;
+    const int max_b = std::max(1, mixed_max_blocks_per_sm(v, r.block));
     const int untuned = untuned_layers(n_total, n_long, num_sms(), max_b);
-    if (!t) bps = untuned;
-    // With the hand-over, no shape takes more than one warp per scheduler for up to six paths per
-    // lane where an untuned launch takes one: in every such case measured that is the fastest, and
-    // the launch is on its way there anyhow.  Four blocks of 128 asked for: 1.5e4 paths of one
-    // heliosphere 48.7 -> 31 ms, 4.8e4 of four 197 -> 98.
-    if (period != 0 && untuned == 1 && n_total <= 6ull * 128u * (uint64_t)num_sms() &&
-        block * (unsigned)std::min(bps, max_b) > 128u) {
-        block = 128u;
+    int bps = !t ? untuned : t->blocks_per_sm ? (int)std::min<uint32_t>(t->blocks_per_sm, (uint32_t)max_b) : max_b;
+    if (r.compact_period != 0 && untuned == 1 && n_total <= 6ull * 128u * (uint64_t)num_sms() &&
+        r.block * (unsigned)bps > 128u) {
+        r.block = 128u;
         bps = 1;
     }
-    bps = std::min(bps, max_b);
-    uint64_t grid = (uint64_t)num_sms() * (uint64_t)bps;
+    r.blocks_per_sm = (uint32_t)bps;
+    return r;
+}
+
+PersistentShape shape_for(MixedVariant v, const cosmica_tuning *t, uint64_t n_total, uint64_t n_long)
+{
+    const cosmica_tuning r = taken_shape(v, t, n_total, n_long);
+    uint64_t grid = (uint64_t)num_sms() * r.blocks_per_sm;
     // never more warps than paths (the kernel spreads them evenly)
-    const uint64_t need = (n_total + block / 32u - 1) / (block / 32u);
+    const uint64_t need = (n_total + r.block / 32u - 1) / (r.block / 32u);
     grid = std::max<uint64_t>(1, std::min(grid, need));
-    return PersistentShape{block, (unsigned)grid, period};
+    return PersistentShape{r.block, (unsigned)grid, r.compact_period};
 }
 
 }  // namespace host
@@ -1145,11 +1151,33 @@ extern "C" cosmica_status cosmica_batch_spectrum_hist(cosmica_batch *b, const co
 // =============================================================== autotune ==
 // Tuned shapes are cached per (device, configuration class): the precision,
 // whether the sets have a drift / a termination shock, the particle count to
-// within a factor of two (it sets the particles per lane, hence the tail), and
-// the kernel variant (energy form, radial shells or squashed heliosphere).
+// within a factor of two (it sets the particles per lane, hence the tail), the
+// warps per scheduler an untuned launch takes (one of a few energies has another
+// tail than one of thirty), and the kernel variant (energy form, radial shells or
+// squashed heliosphere).
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, int>, std::pair<cosmica_tuning, double>> g_tune_cache;
+std::map<std::tuple<int, int, int, int, int, int, int>, std::pair<cosmica_tuning, double>> g_tune_cache;
+
+// n_long of a list of items (see cost_order); items that batch_items would refuse count for nothing
+uint64_t items_n_long(const cosmica_batch *b, const cosmica_work_item *items, uint32_t n_items)
+{
+    std::vector<std::pair<double, uint64_t>> keys;
+    double least = std::numeric_limits<double>::infinity();
+    for (uint32_t i = 0; i < n_items && items; ++i) {
+        const cosmica_work_item &w = items[i];
+        if (!w.n || w.param_idx >= b->params.size() || w.species_idx >= b->species.size() || !(w.T_GeVn > 0.0)) continue;
+        const cosmica_params &p = b->params[w.param_idx];
+        const bool own = w.r0_AU != 0.0;
+        if (own && !valid_start(p, w.r0_AU, w.th0_rad, w.ph0_rad)) continue;
+        keys.emplace_back(start_key(p, b->species[w.species_idx], w.T_GeVn, own ? w.r0_AU : p.r0_AU), w.n);
+        least = std::min(least, keys.back().first);
+    }
+    uint64_t n = 0;
+    for (const auto &k : keys)
+        if (k.first <= 3.0 * least) n += k.second;
+    return n;
+}
 }  // namespace
 
 extern "C" cosmica_status cosmica_autotune(cosmica_batch *b, const cosmica_work_item *items, uint32_t n_items,
@@ -1169,7 +1197,9 @@ extern "C" cosmica_status cosmica_autotune(cosmica_batch *b, const cosmica_work_
     while ((n_all >> size_class) > 1) ++size_class;
     // the kernel variant (energy form, shells) has its own registers, hence its own best shape
     const int variant = (b->params[0].formulation == 1 ? 1 : 0) | (b->full ? 2 : 0) | b->ext.kind() * 4;
-    const auto key = std::make_tuple(dev, b->precision, drift, ts, size_class, variant);
+    const uint64_t n_long = items_n_long(b, items, n_items);
+    const int layers = untuned_layers(n_all, n_long, num_sms(), std::max(1, mixed_max_blocks_per_sm(b->variant(), 128u)));
+    const auto key = std::make_tuple(dev, b->precision, drift, ts, size_class, variant, layers);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -1254,16 +1284,24 @@ extern "C" cosmica_status cosmica_autotune(cosmica_batch *b, const cosmica_work_
         const unsigned blocks[] = {128, 256};
         const unsigned periods[] = {0, 64};
         std::vector<cosmica_tuning> cands;
+        // a shape that the whole batch would not run with stands for the one it would; one candidate each
+        auto add = [&](unsigned blk, unsigned bps, unsigned per) {
+            const cosmica_tuning asked{blk, bps, per, 0, 1};
+            cosmica_tuning t = taken_shape(b->variant(), &asked, n_full, n_long);
+            t.queue_order = 1;
+            for (const cosmica_tuning &c : cands)
+                if (c.block == t.block && c.blocks_per_sm == t.blocks_per_sm && c.compact_period == t.compact_period) return;
+            cands.push_back(t);
+        };
         for (unsigned blk : blocks) {
             for (unsigned per : periods) {
                 const unsigned maxb = (unsigned)std::max(1, mixed_max_blocks_per_sm(b->variant(), blk));
                 // all resident blocks, one fewer, and half: fewer resident warps can win when the
                 // register file or the L1 is the contended resource, or when the tail dominates
-                cands.push_back(cosmica_tuning{blk, maxb, per, 0, 1});
-                if (maxb >= 3) cands.push_back(cosmica_tuning{blk, maxb - 1, per, 0, 1});
-                if (maxb / 2 >= 1 && maxb / 2 != maxb && maxb / 2 != maxb - 1)
-                    cands.push_back(cosmica_tuning{blk, maxb / 2, per, 0, 1});
-                if (blk == 128 && maxb > 2) cands.push_back(cosmica_tuning{blk, 1, per, 0, 1});
+                add(blk, maxb, per);
+                if (maxb >= 3) add(blk, maxb - 1, per);
+                if (maxb / 2 >= 1) add(blk, maxb / 2, per);
+                if (blk == 128) add(blk, 1, per);
             }
         }
         for (const cosmica_tuning &t : cands) {
