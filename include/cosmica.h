@@ -177,9 +177,12 @@ typedef struct {
 } cosmica_species;
 
 /* Exit states, one entry per quasi-particle, structure of arrays.  Entry g is
- * the g-th particle in work-item order (item 0's particles first).  Written
- * once per particle; caller-owned, device or host memory (all arrays in the
- * same space), each of length n. */
+ * the g-th particle in work-item order (item 0's particles first).
+ * Caller-owned, device or host memory (all arrays in the same space), each of
+ * length n.  While the launch runs, an entry may hold the state of a path on
+ * its way from one kernel to the next; arrays that share memory (one array
+ * given for several fields that are not wanted) rule that out, and the launch
+ * is then a single kernel. */
 typedef struct {
     double *r, *th, *ph, *lnP, *s;   /* post-step state at exit [AU, rad, rad, ln GV, day] */
     uint32_t *steps;                 /* Euler-Maruyama steps taken               */

@@ -596,7 +596,7 @@ static cosmica_status propagate_items(cosmica_model *m, const cosmica_species *s
        "cudaMemsetAsync(counters)");
     LaunchArgs a{m->d_prm, d_sp, m->tab.items, m->tab.prefix, m->tab.n_items, total, ex,
                  m->tab.counters + 1, m->tab.counters, m->tab.qitem, m->tab.qprefix, m->d_f32,
-                 m->tab.list, m->tab.list_cap, m->tab.counters + 2};
+                 m->tab.list, exit_arrays_overlap(ex, total) ? 0u : m->tab.list_cap, m->tab.counters + 2};
     cudaError_t e;
     if (m->p.precision == COSMICA_PREC_FP64) {
         e = launch_propagate_fp64(a, fp64_variant(&m->p, 1, species, 1), num_sms(), s);
@@ -1009,7 +1009,7 @@ static cosmica_status batch_launch(cosmica_batch *b, uint64_t total, const ExitP
 {
     LaunchArgs a{b->d_prm, b->d_spc, b->tab.items, b->tab.prefix, b->tab.n_items, total, ex,
                  b->tab.counters + 1, b->tab.counters, b->tab.qitem, b->tab.qprefix, b->d_f32,
-                 b->tab.list, b->tab.list_cap, b->tab.counters + 2};
+                 b->tab.list, exit_arrays_overlap(ex, total) ? 0u : b->tab.list_cap, b->tab.counters + 2};
     auto direct = [&]() -> cosmica_status {
         CK(cudaMemsetAsync(b->tab.counters, 0, kLaunchCounters * sizeof(unsigned long long), s),
        "cudaMemsetAsync(counters)");

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 
 #include "common.cuh"
 #include "cosmica.h"
@@ -145,6 +146,19 @@ inline DevItem make_item(double T, uint64_t first_pid, uint64_t seed, uint32_t p
     it.out_item = out_item;
     it.pad = 0;
     return it;
+}
+// Whether two arrays of an exit record share memory.  A caller may give one array several times for fields it
+// does not want; such a record cannot hold a path's state between two kernels of a launch.
+inline bool exit_arrays_overlap(const ExitPtrs &e, uint64_t n)
+{
+    const std::pair<const void *, uint64_t> in[] = {{e.r, 8 * n}, {e.th, 8 * n}, {e.ph, 8 * n}, {e.lnP, 8 * n}, {e.s, 8 * n},
+                                                    {e.lw, e.lw ? 8 * n : 0}, {e.steps, 4 * n}, {e.item, 4 * n}, {e.status, n}};
+    for (const auto &a : in)
+        for (const auto &b : in) {
+            const uintptr_t pa = (uintptr_t)a.first, pb = (uintptr_t)b.first;
+            if (&a != &b && a.second && b.second && pa <= pb && pb < pa + a.second) return true;
+        }
+    return false;
 }
 int num_sms();
 int untuned_layers(uint64_t n_total, uint64_t n_long, int sms, int max_blocks);

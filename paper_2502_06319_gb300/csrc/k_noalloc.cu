@@ -228,6 +228,7 @@ extern "C" cosmica_status cosmica_propagate_noalloc(const cosmica_params *params
                  ExitPtrs{out->r, out->th, out->ph, out->lnP, out->s, out->steps, out->status, out->item, out->lw},
                  d_counters + 1, d_counters, nullptr, d_prefix, d_f32,
                  list, list_cap, d_counters + 2};
+    if (exit_arrays_overlap(a.out, total)) a.list_cap = 0;
     if (params->precision == COSMICA_PREC_FP64) {
         e = launch_propagate_fp64(a, fp64_variant(params, 1, species, 1), num_sms(), s);
     } else {
