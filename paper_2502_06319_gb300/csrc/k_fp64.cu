@@ -173,9 +173,9 @@ __global__ void __launch_bounds__(128) k_propagate_fp64(const DevParams *__restr
 // A launch that starts with so few paths starts there.  (A mixture of isotropic and other sets
 // stays with k_finish64.)
 // Measured against one thread per path with the plain step: a step of the full model 52 us, 29 in
-// k_propagate64 (a lane a path), 17.4 in k_finish64 (477 slots, the FP64 pipe 84 % busy), 10.1 in
-// k_quad64 (242 slots on its longest warp); 1e4 isotropic paths 86.8 -> 23.2 ms, 2.5e4 paths of the
-// full model 1385 -> 352 ms.  The paths are the same bits.
+// k_propagate64 (a lane a path), 17.4 in k_finish64 (477 slots, the FP64 pipe 84 % busy), 10.0 in
+// k_quad64 (242 slots on its longest warp); 1e4 isotropic paths 91.5 -> 24.0 ms, 2.5e4 paths of the
+// full model 1371 -> 318 ms.  The paths are the same bits.
 struct Path64 {
     uint64_t g, pid, seed;
     const DevParams *p;

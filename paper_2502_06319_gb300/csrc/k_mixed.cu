@@ -165,11 +165,11 @@ __device__ __forceinline__ bool settle(const LaunchArgs &a, Lane &L, Acc<ACC> &x
 // path on whatever they hold (nobody looks at the results).  What bounds it: a warp alone on its
 // scheduler is bound by its ~400 instructions a step and their dependences, four warps by the
 // issue rate.  The loop being one block, the compiler interleaves the generator with the
-// coefficients and keeps the parameter set in registers (114-123 instead of 64, so 16 warps
+// coefficients and keeps the parameter set in registers (122-160 instead of 64, so 12 or 16 warps
 // per SM instead of 32).  Measured, against a loop that tested everything every step and drew the
 // normals after the tests: a lone path's step 0.68 -> 0.30 us (375 instructions), a warp's step
-// with four warps per scheduler 1.05 -> 0.87 us, one spectrum of 6e5 paths 143 -> 93 ms, 1.8e6
-// paths of 16 heliospheres 869 -> 657 ms (8.5e10 steps/s).
+// with four warps per scheduler 1.05 -> 0.87 us, one spectrum of 6e5 paths 144 -> 93 ms, 1.8e6
+// paths of 16 heliospheres 893 -> 669 ms.
 template <int ACC, bool EN, int EXT, bool FULL>
 __global__ void __launch_bounds__(256, 1) k_propagate_mixed(LaunchArgs a, MixedStage st)
 {

@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(128, 1) k_serve(ServeArgs a)
 
         // steps until some lane has a boundary or an end to see to, or the budget ends (it ends for
         // all lanes of a warp at once: they have stepped together since the launch began); one
-        // block, as in the batched kernel.  Four requests of some 5e4 paths: 357 -> 146 ms
+        // block, as in the batched kernel.  Four requests of some 5e4 paths: 348 -> 140 ms
         const P32<1> q{S.L.q};
         bool see;
         while (true) {

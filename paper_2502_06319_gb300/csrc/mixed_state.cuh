@@ -140,9 +140,9 @@ struct Acc<COSMICA_PREC_MIXED> {
 // FP64 accumulation of FP32 increments.
 // The FP64 pipe takes 64 clocks per warp instruction and scheduler, so only the sums stay on it;
 // conversions, comparisons and the finiteness test run on the bits (f64bits.h).  The results
-// are the same bits.  Measured: 1.4e5 paths of 4 heliospheres 738 -> 328 ms by the integer
-// forms, 781 -> 181 ms with the step as one block whose vote does not wait for the sums (a lone
-// path's step 2.16 -> 0.53 us).
+// are the same bits.  Measured, conversion instructions and a step in branches against these and a
+// step in one block whose vote does not wait for the sums: a lone path's step 2.16 -> 0.51 us, 1.2e5
+// paths of 4 heliospheres 854 -> 160 ms.
 template <>
 struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     double r, th, ph, lnP, s, Rout, r_in;
