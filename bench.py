@@ -71,8 +71,8 @@ SM_LANES_PER_CLK = 128      # 4 SMSPs x 32 lanes: one warp instruction per SMSP 
 # reduced count; the bytes are the work-item reads and exit-record writes, so they scale
 # with the particles of a launch (commands in profiles/).  They describe the kernel built
 # from the sources whose SHA-256 is recorded; any other build reports traffic null.
-TRAFFIC = {"c3": {"bytes_per_particle": 178110208 / 3715361,   # 24 089 344 read + 154 020 864 written, 5 % scale
-                  "sources_sha256": "e2bf3ff9649f05d674daea831e310330d1fdbbc3c495dd45c6fd482e68a969d0"}}
+TRAFFIC = {"c3": {"bytes_per_particle": 177309696 / 3715361,   # 23 920 640 read + 153 389 056 written, 5 % scale
+                  "sources_sha256": "28f25c646a8351d08f706e071367ec979ebb581edd51aa1b93b06d2f7186c9b9"}}
 KERNEL_SOURCES = ("common.cuh", "philox.cuh", "f64bits.h", "model32.cuh", "mixed_state.cuh", "k_mixed.cu")
 
 

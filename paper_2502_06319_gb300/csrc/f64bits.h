@@ -97,7 +97,7 @@ COSMICA_HD uint64_t from_u32(uint32_t n)
 // first counts where a step from far out ends beside r_in, hence the share of reach.
 COSMICA_HD float vote_floor(float r_in, float reach) { return r_in * 1.000001f + reach * 2.4e-7f; }
 COSMICA_HD float vote_ceiling(float R) { return R * 0.999999f; }
-constexpr float kNoCeiling = 1e30f;      // where another test bounds r: keeps an infinity out
+constexpr float kMostRise = 1e30f;       // of r in a step where another test bounds r: keeps an infinity out
 
 // FP64 comparisons on the bits, with b > 0 finite: right for every a but NaN.
 COSMICA_HD bool less(uint64_t a, uint64_t b) { return (int64_t)a < (int64_t)b; }

@@ -177,8 +177,8 @@ struct Acc<COSMICA_PREC_MIXED_F64ACC> {
     __device__ bool add(float fr, float fth, float fph, float dr, float dth, float dph, float dlnP, float dt, float, bool sphere)
     {
         const float nr = fr + dr, nth = fth + dth, nph = fph + dph;
-        const bool still = (nr > r_lo) & (nr < (sphere ? r_hi : f64bits::kNoCeiling)) & (nth > 1e-5f) & (nth < 3.14158f) & (nph > 1e-5f) &
-                           (nph < 6.28317f) & isfinite(dlnP + dt);
+        const bool still = (sphere | (dr < f64bits::kMostRise)) & (nr > r_lo) & (!sphere | (nr < r_hi)) & (nth > 1e-5f) &
+                           (nth < 3.14158f) & (nph > 1e-5f) & (nph < 6.28317f) & isfinite(dlnP + dt);
         th += widen64(dth); r += widen64(dr);
         if (P) lnP += widen64(dlnP);
         ph += widen64(dph); s += widen64(dt);

@@ -13,8 +13,11 @@ SRC = r"""
 using namespace cosmica::f64bits;
 extern "C" void vote(const float *fr, const float *dr, float r_in, float R, int sphere, uint8_t *o, int n)
 {
-    const float lo = vote_floor(r_in, R), hi = sphere ? vote_ceiling(R) : kNoCeiling;
-    for (int i = 0; i < n; ++i) { const float nr = fr[i] + dr[i]; o[i] = (nr > lo) & (nr < hi); }
+    const float lo = vote_floor(r_in, R), hi = vote_ceiling(R);
+    for (int i = 0; i < n; ++i) {
+        const float nr = fr[i] + dr[i];
+        o[i] = (nr > lo) & (sphere ? nr < hi : dr[i] < kMostRise);
+    }
 }
 """
 
